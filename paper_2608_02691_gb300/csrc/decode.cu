@@ -15,6 +15,7 @@
 // softmax weights are exp2(l - m) (Sec. 3 Eq. 1 with the 1/sqrt(d) scale).
 #include "decode_common.cuh"
 #include "append_small.cuh"
+#include "qrot.cuh"
 #include "window.cuh"
 
 namespace optr {
@@ -23,20 +24,6 @@ namespace {
 constexpr float kLog2e = 1.4426950408889634f;
 
 // ---------------------------------------------------------------- qrot
-
-// One CTA per (sequence, KV head), 512 threads = 4 slices x 128 channels:
-// slice s sums q[i] R[i][j] over i in [32s, 32s+32) for the 4 query heads of
-// the group, the slices are added in shared memory.
-constexpr int kQrotThreads = 512;
-
-struct QrotSmem {
-  float qsm[4][kD];
-  float part[4][4][kD];  // [slice][head][channel]
-  float qrs[4][kD];
-  float hmax[4][4];
-  int warp_tot[2][kQrotThreads / 32];
-  long long koff_part[kQrotThreads / 32][kGroups];
-};
 
 // CTA (b, h) of the query rotation; 512 threads.
 __device__ __forceinline__ void qrot_body(
@@ -47,119 +34,17 @@ __device__ __forceinline__ void qrot_body(
     float* __restrict__ koff, float* __restrict__ invs, int* __restrict__ pref,
     int* __restrict__ nzpref, int* __restrict__ cnt_ws, unsigned* err,
     int sink, int recent) {
-  float (&qsm)[4][kD] = sm.qsm;
-  float (&part)[4][4][kD] = sm.part;
-  float (&qrs)[4][kD] = sm.qrs;
-  float (&hmax)[4][4] = sm.hmax;
   int (&warp_tot)[2][kQrotThreads / 32] = sm.warp_tot;
-  long long (&koff_part)[kQrotThreads / 32][kGroups] = sm.koff_part;
   const int tid = threadIdx.x;
-  const int sl = tid >> 7, j = tid & 127;
   const int warp = tid >> 5, lane = tid & 31;
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  const float* R = R_k + (size_t)h * kD * kD + (size_t)(32 * sl) * kD + j;
   float rv[32];
-#pragma unroll
-  for (int i = 0; i < 32; ++i) rv[i] = __ldg(R + i * kD);  // all in flight
+  load_rotation_slice(R_k, h, rv);
   pdl_wait();  // the query, lengths and workspace may belong to earlier kernels
   pdl_trigger();
-  // Global stores wait until the end: a __syncthreads() after a store waits
-  // for it to complete, which made each phase an L2 round trip.
-  {
-    const int r = tid >> 7;  // 512 threads load the 4 x 128 query values
-    qsm[r][j] = __bfloat162float(q[((size_t)b * h_q + 4 * h + r) * kD + j]);
-  }
-  __syncthreads();
-#pragma unroll
-  for (int i4 = 0; i4 < 8; ++i4)
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const float4 qv = *reinterpret_cast<const float4*>(&qsm[r][32 * sl + 4 * i4]);
-      acc[r] = fmaf(qv.x, rv[4 * i4 + 0], acc[r]);
-      acc[r] = fmaf(qv.y, rv[4 * i4 + 1], acc[r]);
-      acc[r] = fmaf(qv.z, rv[4 * i4 + 2], acc[r]);
-      acc[r] = fmaf(qv.w, rv[4 * i4 + 3], acc[r]);
-    }
-#pragma unroll
-  for (int r = 0; r < 4; ++r) part[sl][r][j] = acc[r];
-  __syncthreads();
-  // thread (r, j): the 4 slices of head r, channel j (512 threads)
-  const int qr = tid >> 7;
-  const size_t qrow = (size_t)b * h_q + 4 * h + qr;
-  const float qx = (part[0][qr][j] + part[1][qr][j] + part[2][qr][j] + part[3][qr][j]) * qscale;
-  float qsum = qx;
-  {
-    const int r = qr;
-    const float x = qx;
-    qrs[r][j] = x;
-    float s = x, a = fabsf(x);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      s += __shfl_xor_sync(0xffffffffu, s, o);
-      a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, o));
-    }
-    qsum = s;
-    if (lane == 0) hmax[r][j >> 5] = a;
-  }
-  __syncthreads();
-  // Tensor-core B fragments (see decode_tc.cu): per head a power-of-two
-  // prescale 2^e brings max |q'| * 2^e into [2^13, 2^14), so that the fp16
-  // hi/lo split stays in the normal range for all but tiny elements.  The
-  // key codes enter the MMA as 1024 + code * 2^pos (pos = kCodePos[G&1][r]),
-  // so the fragment of channel 32G + 4w + r also carries 2^-pos, and koff
-  // holds the offset sum 1024 * sum over the group of the fragment values,
-  // per (query head, group, hi/lo column), which the MMA starts from
-  // (negated) so that the accumulator sums code * q' exactly as before.
-  {
-    const int ridx = tid;  // 512 fragment registers, one per thread
-    const int L = ridx >> 4, reg = ridx & 15;
-    const int G = reg >> 2, kk = (reg >> 1) & 1, which = reg & 1;
-    const int g = L >> 2, c = L & 3;
-    const int head = g >> 1, part_hl = g & 1;
-    const float mx = fmaxf(fmaxf(hmax[head][0], hmax[head][1]),
-                           fmaxf(hmax[head][2], hmax[head][3]));
-    const int e = max(-100, min(100, mx > 0.f ? 13 - ilogbf(mx) : 0));
-    const int r = 2 * kk + which;
-    const int ch = 32 * G + 8 * c + r;   // low half; +4 high
-    const float sc = ldexpf(1.f, e - code_pos(G, r));
-    const float x0 = qrs[head][ch] * sc, x1 = qrs[head][ch + 4] * sc;
-    const __half h0 = __float2half_rn(x0), h1 = __float2half_rn(x1);
-    __half v0 = h0, v1 = h1;
-    if (part_hl) {
-      v0 = __float2half_rn(x0 - __half2float(h0));
-      v1 = __float2half_rn(x1 - __half2float(h1));
-    }
-    const uint32_t fragv =
-        (uint32_t)__half_as_ushort(v0) | ((uint32_t)__half_as_ushort(v1) << 16);
-    // offset sum over the 32 channels of group G for column g: reduce over
-    // (kk, which) = lane bits 0-1, c bit 0 = lane bit 4, c bit 1 = warp bit 0.
-    // Exact, in fixed point: an fp16 value times 2^24 is an integer below
-    // 2^40, so 64 of them sum exactly in int64; one rounding to float, then
-    // 1024 * 2^-24 = 2^-14 (exact) gives the correctly rounded koff.
-    long long t = __float2ll_rn(__half2float(v0) * 16777216.0f) +
-                  __float2ll_rn(__half2float(v1) * 16777216.0f);
-    t += __shfl_xor_sync(0xffffffffu, t, 1);
-    t += __shfl_xor_sync(0xffffffffu, t, 2);
-    t += __shfl_xor_sync(0xffffffffu, t, 16);
-    if ((lane & 15) % 4 == 0) koff_part[warp][G] = t;
-    __syncthreads();
-    if (tid < 32) {  // tid = (g, G): koff[head][G][hl] for column g
-      const int gg = tid >> 2, GG = tid & 3;
-      const long long tot = koff_part[2 * gg][GG] + koff_part[2 * gg + 1][GG];
-      koff[((size_t)b * h_kv + h) * 32 + (gg >> 1) * 8 + GG * 2 + (gg & 1)] =
-          __ll2float_rn(tot) * 0x1p-14f;
-    }
-    if (ridx < 4) {
-      const float m2 = fmaxf(fmaxf(hmax[ridx][0], hmax[ridx][1]),
-                             fmaxf(hmax[ridx][2], hmax[ridx][3]));
-      const int e2 = max(-100, min(100, m2 > 0.f ? 13 - ilogbf(m2) : 0));
-      invs[(size_t)b * h_q + 4 * h + ridx] = ldexpf(1.f, -e2);
-    }
-    frag[((size_t)b * h_kv + h) * 512 + ridx] = fragv;
-  }
-  qf[qrow * kD + j] = qx;
-  if (lane == 0) qs[qrow * kGroups + (j >> 5)] = qsum;
-  if (tid == 0) cnt_ws[(size_t)b * h_kv + h] = 0;  // combine arrivals
+  const size_t row = (size_t)b * h_q + 4 * h, seg = (size_t)b * h_kv + h;
+  rotate_query(sm, q + row * kD, rv, qscale, qf + row * kD, qs + row * kGroups,
+               frag + seg * 512, koff + seg * 32, invs + row);
+  if (tid == 0) cnt_ws[seg] = 0;  // combine arrivals
 
   if (b != 0 || h != 0) return;
   // Split-K plan: pref[b] = INT2 pages of sequences < b, nzpref[b] =
@@ -317,7 +202,7 @@ partial_cuda_core_kernel(const uint8_t* __restrict__ pool,
   // reads only inputs and library-owned state); stage and p are free until
   // the first segment
   if constexpr (WIN) {
-    if (w < wp.Ww) window_phase(w, wp, S.wst, reinterpret_cast<uint8_t*>(&S.p[0][0]));
+    if (w < wp.Ww) window_warp(w, wp, S.wst, reinterpret_cast<uint8_t*>(&S.p[0][0]));
   }
   pdl_wait();
   pdl_trigger();
@@ -872,6 +757,13 @@ cudaError_t launch_partial_tensor(const optr_params* p, const uint8_t* pool,
                                   const int32_t* step_cu, const int32_t* step_pos0,
                                   const WinPhase& wp, cudaStream_t s);
 
+int decode_one_cluster(const optr_params* p, int B, int max_pages);
+cudaError_t launch_decode_one(const optr_params* p, int cs, const __nv_bfloat16* q,
+                              const uint8_t* pool, const int32_t* bt, const int32_t* seq_lens,
+                              int B, int max_pages, int num_pages, float qscale, float* out,
+                              const int32_t* step_cu, const int32_t* step_pos0,
+                              const WinPhase& wp, cudaStream_t s);
+
 cudaError_t launch_window_copy(const optr_params* p, const __nv_bfloat16* k,
                                const __nv_bfloat16* v, int n_tok,
                                const int32_t* cu_new, const int32_t* pos0,
@@ -932,9 +824,11 @@ cudaError_t launch_decode(const optr_params* p, int variant,
 
   int* cnt_ws = reinterpret_cast<int*>(w + plan.off_cnt);
   cudaError_t e;
+  // CTAs per segment of the one-launch decode (0: split-K)
+  const int cs = variant != OPTR_VARIANT_CUDA_CORE ? decode_one_cluster(p, B, max_pages) : 0;
   if (app) {
     // the cache write of the step (INT2 records and window copies) and the
-    // query rotation in one launch
+    // query rotation in one launch (the one-launch decode rotates its own)
     prof_mark(p, 0, s);
     const int T = small_tile(app->n_tok);
     const int tiles = (app->n_tok + T - 1) / T;
@@ -948,7 +842,8 @@ cudaError_t launch_decode(const optr_params* p, int variant,
                                 : step_prologue_kernel<kSmallTok>;
     e = ensure_dynamic_smem(reinterpret_cast<const void*>(fn), sm_bytes);
     if (e != cudaSuccess) return e;
-    e = launch_pdl(fn, dim3(n_app + n_wcp + B * h_kv), dim3(512),
+    const int n_rot = cs ? 0 : B * h_kv;
+    e = launch_pdl(fn, dim3(n_app + n_wcp + n_rot), dim3(512),
                    sm_bytes, s, n_app, tiles, app->k, app->v, app->n_tok,
                    app->cu_new, app->pos0, bt, app->pool, num_pages,
                    (const float*)p->R_v, (const float*)p->muR, p->cfg.clip_k,
@@ -959,10 +854,12 @@ cudaError_t launch_decode(const optr_params* p, int variant,
                    windows ? win->slot : (const int32_t*)nullptr,
                    windows ? win->n_slots : 0, sink, recent,
                    p->cfg.group == 128 ? 1 : 0,
-                   std::max(0, std::min(B * h_kv, p->num_sms - n_app - n_wcp)));
+                   std::max(0, std::min(n_rot, p->num_sms - n_app - n_wcp)));
     if (e != cudaSuccess) return e;
     prof_mark(p, 1, s);  // the append stage covers the fused launch,
     prof_mark(p, 2, s);  // the query-rotation stage is empty
+  } else if (cs) {
+    prof_mark(p, 2, s);
   } else {
     prof_mark(p, 2, s);
     e = launch_pdl(qrot_kernel, dim3(B, h_kv), dim3(kQrotThreads), 0, s, q,
@@ -972,6 +869,13 @@ cudaError_t launch_decode(const optr_params* p, int variant,
     if (e != cudaSuccess) return e;
   }
   prof_mark(p, 3, s);
+  if (cs) {
+    e = launch_decode_one(p, cs, q, pool, bt, seq_lens, B, max_pages, num_pages, qscale, out,
+                          app ? app->cu_new : nullptr, app ? app->pos0 : nullptr, wp, s);
+    prof_mark(p, 4, s);  // the partial stage covers the launch
+    prof_mark(p, 5, s);
+    return e;
+  }
   if (variant != OPTR_VARIANT_CUDA_CORE) {
     // after a separate append the pool is complete before qrot starts, so
     // the partial kernel may fetch pages before waiting for qrot; after the

@@ -36,6 +36,7 @@
 #include <type_traits>
 
 #include "decode_common.cuh"
+#include "qrot.cuh"
 #include "window.cuh"
 
 namespace optr {
@@ -63,6 +64,8 @@ static_assert(offsetof(WarpSmemTC, pt) + sizeof(WarpSmemTC::pt) -
               "window row scratch");
 static_assert(sizeof(WarpSmemTC::qfr) >= (size_t)kWinPBytes, "window P scratch");
 
+// one-launch decode: pages that take as long as a unit of 16 window tokens
+constexpr int kUnitPages = 4;
 constexpr int kPrefCache = 256;  // sequences whose page prefix sums a CTA caches
 
 __device__ __forceinline__ void mma16816(float* d, uint32_t a0, uint32_t a1,
@@ -232,14 +235,67 @@ __device__ __noinline__ void page_prefix(const int32_t* __restrict__ seq_lens,
   __syncthreads();
 }
 
+// One-launch decode of a small batch (ONE): a cluster of CTAs per (sequence,
+// KV head) rotates the query itself, goes through its pages, merges its
+// partials in (distributed) shared memory and applies R_v^T.  A split-K decode
+// of such a batch is three launches that each wait for the one before and hand
+// their results over in global memory, ~15 us for a few pages per warp.
+struct OneArgs {
+  const __nv_bfloat16* q;
+  const float* R_k;
+  const float* R_vT;
+  float* out;
+  float qscale;
+  int fold_v;
+  int step;  // the previous kernel is the step's cache write
+};
+
+struct OneSmem {
+  union {
+    QrotSmem rot;
+    struct {
+      float o[4 * kD], ow[4 * kD], M[4], L[4];  // the CTA's partial: INT2, windows
+    } part;
+  };
+  uint32_t frag[512];
+  float koff[32], invs[4], qs[4 * kGroups];
+  float orot[4][kD], ow[4][kD];  // normalised output before R_v^T, window output
+  float red[4 * kQrotThreads];   // [part of k][head][channel of the slice]
+};
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t cluster_size() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;"
+               ::: "memory");
+}
+// x of the same shared variable in CTA `rank` of the cluster
+__device__ __forceinline__ float cluster_load(const float* x, uint32_t rank) {
+  const uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(x));
+  float v;
+  asm volatile(
+      "{\n .reg .u32 r;\n mapa.shared::cluster.u32 r, %1, %2;\n"
+      " ld.shared::cluster.f32 %0, [r];\n}\n"
+      : "=f"(v) : "r"(a), "r"(rank) : "memory");
+  return v;
+}
+
 // WIN: the BF16-window phase is compiled in (a separate instance, so that
 // the INT2-only kernel keeps its own register allocation).  CMP: the compact
 // G = 128 record (1152 bytes per page and KV head, one (scale, min) pair per
 // slot at 4-byte stride), read as the G = 32 record's four entries with the
 // pair repeated, so the page arithmetic is the same.
-template <bool WIN, bool CMP>
-__global__ void __launch_bounds__(kWarps * 32, 1)
-partial_tensor_kernel(const uint8_t* __restrict__ pool,
+template <bool WIN, bool CMP, bool ONE>
+__device__ __forceinline__ void
+partial_body(const uint8_t* __restrict__ pool,
                       const int32_t* __restrict__ bt,
                       const int32_t* __restrict__ seq_lens, int B,
                       int max_pages, int num_pages, int h_q, int h_kv,
@@ -252,7 +308,8 @@ partial_tensor_kernel(const uint8_t* __restrict__ pool,
                       float* __restrict__ part, int W, int early_pages,
                       const int32_t* __restrict__ step_cu,
                       const int32_t* __restrict__ step_pos0,
-                      unsigned* err, int sink, int recent, WinPhase wp) {
+                      unsigned* err, int sink, int recent, const WinPhase& wp,
+                      const OneArgs& one) {
   // One 16-warp CTA per SM: the warp schedulers favour the CTAs that
   // arrived first on an SM, and with four 4-warp CTAs per SM the last CTA
   // finished ~20% after the first; within one CTA the warps keep pace.
@@ -269,7 +326,8 @@ partial_tensor_kernel(const uint8_t* __restrict__ pool,
   // With BF16 windows, warps kWinIntWarps.. of every CTA are window warps
   // (their loads overlap the INT2 pages of the others); the INT2 work is
   // split over the first kWinIntWarps warps of each CTA.
-  constexpr int kInt = WIN ? kWinIntWarps : kWarps;
+  // ONE: as many as the segment's pages and window units ask for.
+  int kInt = WIN ? kWinIntWarps : kWarps;
   const int w = blockIdx.x * kInt + warp;  // INT2 warp index (warp < kInt)
 
   // Page prefix sums.  For up to kPrefCache sequences the CTA scans the
@@ -282,10 +340,37 @@ partial_tensor_kernel(const uint8_t* __restrict__ pool,
   // pool was complete before the previous kernel began (early_pages: a
   // separate append); after the fused step prologue, which writes the pool,
   // they follow the wait.
-  const bool cached = B <= kPrefCache;
+  const bool cached = !ONE && B <= kPrefCache;
   static_assert(kPrefCache < kWarps * 32, "one thread per sequence");
   int F;
-  if (cached) {
+  // ONE: this CTA's (sequence, KV head), its rank among the cluster's CTAs
+  OneSmem& O = *reinterpret_cast<OneSmem*>(smem + kWarps);
+  const int cs = ONE ? (int)cluster_size() : 1, rank = ONE ? (int)cluster_rank() : 0;
+  const int oseg = ONE ? (int)blockIdx.x / cs : 0, ob = oseg / h_kv, oh = oseg - ob * h_kv;
+  float rv[ONE ? 32 : 1];
+  if constexpr (ONE) {
+    load_rotation_slice(one.R_k, oh, rv);
+    // In a step every input was complete before the cache write began; alone,
+    // inputs may come from the previous kernel.
+    if (!one.step) {
+      pdl_wait();
+      pdl_trigger();
+    }
+    const int len = __ldcg(seq_lens + ob);
+    const bool bad = len < 0 || (long long)len > (long long)max_pages * kPage;
+    if (bad && threadIdx.x == 0 && rank == 0 && oh == 0) atomicOr(err, OPTR_DEVERR_SEQ_LEN);
+    F = bad ? 0 : int2_pages(len, sink, recent);
+    if constexpr (WIN) {
+      // lane i: how long a CTA with i window warps takes; the fewest pages
+      const int units = ((bad ? 0 : win_count(len, sink, recent)) + kWinUnit - 1) / kWinUnit;
+      const int np = (F + cs - 1) / cs, nu = (units + cs - 1) / cs;
+      int cost = 1 << 24;
+      if (lane <= kWarps && (nu == 0 || lane > 0) && (np == 0 || lane < kWarps))
+        cost = max(nu ? (units + cs * lane - 1) / (cs * lane) * kUnitPages : 0,
+                   np ? (F + cs * (kWarps - lane) - 1) / (cs * (kWarps - lane)) : 0);
+      kInt = kWarps - (int)(__reduce_min_sync(0xffffffffu, (unsigned)(cost << 5 | lane)) & 31u);
+    }
+  } else if (cached) {
     page_prefix(seq_lens, B, max_pages, spref, wsum, sink, recent, step_cu, step_pos0,
                 sstep);
     F = spref[B] * h_kv;
@@ -293,7 +378,7 @@ partial_tensor_kernel(const uint8_t* __restrict__ pool,
     pdl_wait();
     F = __ldcg(pref + B) * h_kv;
   }
-  if constexpr (WIN) {
+  if constexpr (WIN && !ONE) {
     if (warp >= kInt) {
       // window warp ww, numbered across the CTAs first so that a partial set
       // is spread over the SMs.  The phase reads only inputs and
@@ -301,31 +386,55 @@ partial_tensor_kernel(const uint8_t* __restrict__ pool,
       // previous kernel, in the warp's own page stages.
       const int ww = (warp - kInt) * gridDim.x + blockIdx.x;
       if (ww < wp.Ww)
-        window_phase(ww, wp, &S.stage[0][0], reinterpret_cast<uint8_t*>(&S.qfr[0][0]));
+        window_warp(ww, wp, &S.stage[0][0], reinterpret_cast<uint8_t*>(&S.qfr[0][0]));
       pdl_wait();
       pdl_trigger();
       return;
     }
   }
-  const int f0 = (int)((long long)w * F / W), f1 = (int)((long long)(w + 1) * F / W);
-  if (f0 >= f1) {
-    pdl_wait();
-    pdl_trigger();
-    return;
+  const bool int_warp = warp < kInt;
+  // ONE: the segment's pages over the cluster's INT2 warps
+  const int wi = ONE ? rank * kInt + warp : w, wn = ONE ? cs * kInt : W;
+  const int f0 = int_warp ? (int)((long long)wi * F / wn) : 0,
+            f1 = int_warp ? (int)((long long)(wi + 1) * F / wn) : 0;
+  if constexpr (!ONE) {
+    if (f0 >= f1) {
+      pdl_wait();
+      pdl_trigger();
+      return;
+    }
   }
   PageChunk chk;
   int f_issue = f0;
   int lpage;
-  load_chunk(chk, f0, f1, pref, spref, cached, seq_lens, bt, B, h_kv,
-             max_pages, num_pages, err, lane, sink, recent, lpage);
+  auto next_chunk = [&](int base) {
+    if constexpr (ONE) {  // load_chunk() of one segment
+      chk.base = base;
+      chk.unit = -1;
+      chk.key = oseg;
+      chk.nvalid = 0;
+      lpage = sink / kPage + base + lane;
+      if (base + lane < f1) {
+        const int phys = __ldcg(bt + (size_t)ob * max_pages + lpage);
+        if (phys >= 0 && phys < num_pages) {
+          chk.unit = phys * h_kv + oh;
+          chk.nvalid = min(kPage, int2_end(__ldcg(seq_lens + ob), sink, recent) - lpage * kPage);
+        } else {
+          atomicOr(err, OPTR_DEVERR_PAGE_ID);
+        }
+      }
+    } else {
+      load_chunk(chk, base, f1, pref, spref, cached, seq_lens, bt, B, h_kv,
+                 max_pages, num_pages, err, lane, sink, recent, lpage);
+    }
+  };
+  next_chunk(f0);
 
   // issue one page into stage s (no commit); every lane records what the
   // stage holds
   auto issue = [&](int s) {
     if (f_issue < f1) {
-      if (f_issue - chk.base == 32)
-        load_chunk(chk, f_issue, f1, pref, spref, cached, seq_lens, bt, B, h_kv,
-                   max_pages, num_pages, err, lane, sink, recent, lpage);
+      if (f_issue - chk.base == 32) next_chunk(f_issue);
       const int j = f_issue - chk.base;
       const int unit = __shfl_sync(0xffffffffu, chk.unit, j);
       const int key = __shfl_sync(0xffffffffu, chk.key, j);
@@ -354,7 +463,7 @@ partial_tensor_kernel(const uint8_t* __restrict__ pool,
   // none of whose 16 positions is among them holds only records written
   // before the step, so the pair is fetched before the wait when both pages
   // are such (a step's written pages are not read by another sequence).
-  bool pre = early_pages != 0;
+  bool pre = ONE ? !one.step : early_pages != 0;  // (ONE alone: past the wait)
   if (!pre && step_cu != nullptr) {
     bool safe = true;
     if (lane < 2 && f0 + lane < f1 && chk.key >= 0) {
@@ -368,9 +477,26 @@ partial_tensor_kernel(const uint8_t* __restrict__ pool,
     pre = __all_sync(0xffffffffu, safe);
   }
   if (pre) issue_pair(0);
+  if constexpr (ONE)
+  {
+    rotate_query(O.rot, one.q + ((size_t)ob * h_q + 4 * oh) * kD, rv, one.qscale, nullptr, O.qs,
+                 O.frag, O.koff, O.invs);
+    if constexpr (WIN) {
+      if (!int_warp) {  // reads inputs only: ahead of the wait in a step
+        float* mine = reinterpret_cast<float*>(&S.stage[0][0]);
+        if (lane < 8) mine[kPartM + lane] = lane < 4 ? -INFINITY : 0.f;
+        __syncwarp();
+        const int ww = rank * (kWarps - kInt) + warp - kInt, n = cs * (kWarps - kInt);
+        window_phase((long long)oseg * wp.Uw + (long long)ww * wp.Uw / n,
+                     (long long)oseg * wp.Uw + (long long)(ww + 1) * wp.Uw / n, wp, mine, -oseg,
+                     &S.stage[0][0], reinterpret_cast<uint8_t*>(&S.qfr[0][0]));
+      }
+    }
+  }
   pdl_wait();  // (returns at once when already passed above)
   pdl_trigger();
   if (!pre) issue_pair(0);
+  if constexpr (ONE) __syncthreads();  // the rotated query
 
   // per-segment state
   uint32_t bmin = 0;           // key min-term B fragment (sum q' per group)
@@ -394,7 +520,8 @@ partial_tensor_kernel(const uint8_t* __restrict__ pool,
       for (int o = 4; o < 32; o <<= 1)
         mv[G] += __shfl_xor_sync(0xffffffffu, mv[G], o);
     const int cb = cur_key / h_kv, ch = cur_key - cb * h_kv;
-    float* slot = part + (size_t)(w + __ldcg(nzpref + cb) * h_kv + ch) * kPartFloats;
+    float* slot = ONE ? reinterpret_cast<float*>(&S.stage[0][0])
+                      : part + (size_t)(w + __ldcg(nzpref + cb) * h_kv + ch) * kPartFloats;
     float* dst = slot + c * kD;
 #pragma unroll
     for (int G = 0; G < kGroups; ++G) {
@@ -417,17 +544,20 @@ partial_tensor_kernel(const uint8_t* __restrict__ pool,
   auto begin_segment = [&](int key) {
     cur_key = key;
     const int cb = key / h_kv, ch = key - cb * h_kv;
+    // ONE: from shared memory
+    auto load4 = [](const float4* p) { return ONE ? *p : __ldcg(p); };
+    auto load1 = [](const float* p) { return ONE ? *p : __ldcg(p); };
     const uint4* fq = reinterpret_cast<const uint4*>(
-        frag + (((size_t)cb * h_kv + ch) * 32 + lane) * 16);
+        (ONE ? O.frag : frag + ((size_t)cb * h_kv + ch) * 512) + lane * 16);
 #pragma unroll
     for (int G = 0; G < kGroups; ++G) {
-      const uint4 v = __ldcg(fq + G);
+      const uint4 v = ONE ? fq[G] : __ldcg(fq + G);
       S.qfr[G][lane] = v;
     }
     {
       const float4* ko = reinterpret_cast<const float4*>(
-          koff + ((size_t)cb * h_kv + ch) * 32 + c * 8);
-      const float4 k01 = __ldcg(ko), k23 = __ldcg(ko + 1);
+          (ONE ? O.koff : koff + ((size_t)cb * h_kv + ch) * 32) + c * 8);
+      const float4 k01 = load4(ko), k23 = load4(ko + 1);
       if constexpr (CMP) {
         // one scale per token: the four groups share one accumulator,
         // started from the sum of their offsets
@@ -441,15 +571,15 @@ partial_tensor_kernel(const uint8_t* __restrict__ pool,
         S.kq[3][lane] = make_float4(-k23.z, -k23.w, -k23.z, -k23.w);
       }
     }
-    const size_t row = (size_t)cb * h_q + 4 * ch + c;
+    const size_t row0 = (size_t)cb * h_q + 4 * ch;
     {
       // column g of the min-term MMA: head g/2, fp16 limb g%2 of the
       // group-c sum of q'; rows k = 2c (scale entries) are 0
-      const float qg = __ldcg(qs + ((size_t)cb * h_q + 4 * ch + (g >> 1)) * kGroups + c);
+      const float qg = load1((ONE ? O.qs : qs + row0 * kGroups) + (g >> 1) * kGroups + c);
       const uint32_t hl = split_hilo(qg);
       bmin = (g & 1) ? (hl & 0xffff0000u) : (hl << 16);
     }
-    inv_s = __ldcg(invs + row);
+    inv_s = load1((ONE ? O.invs : invs + row0) + c);
 #pragma unroll
     for (int G = 0; G < kGroups; ++G) {
       mv[G] = 0.f;
@@ -736,7 +866,7 @@ partial_tensor_kernel(const uint8_t* __restrict__ pool,
   // Pages go through the stages in pairs: pair q (stages 2q, 2q+1) is
   // processed while the other pair is in flight.
   // the first segment's query data, loaded while the first pages land
-  begin_segment(__shfl_sync(0xffffffffu, chk.key, 0));
+  if (!ONE || f0 < f1) begin_segment(__shfl_sync(0xffffffffu, chk.key, 0));
   static_assert(kStages == 4, "two pairs of stages");
   const int total = f1 - f0;
 #pragma unroll 1
@@ -755,7 +885,131 @@ partial_tensor_kernel(const uint8_t* __restrict__ pool,
       if (done + 1 < total) single(2 * q + 1);
     }
   }
-  flush();
+  if constexpr (!ONE) {
+    flush();
+  } else {
+    float* mine = reinterpret_cast<float*>(&S.stage[0][0]);  // partial of this warp
+    if (f0 < f1) {
+      flush();
+    } else if (int_warp && lane < 8) {
+      mine[kPartM + lane] = lane < 4 ? -INFINITY : 0.f;  // (nothing: m, l)
+    }
+    // R_v^T columns [rank sw, (rank + 1) sw), eight rows per warp, into the
+    // warp's query fragments (free now)
+    const int sw = kD / cs;
+    float* rows = reinterpret_cast<float*>(&S.qfr[0][0]);
+    __syncwarp();
+    if (!one.fold_v) {
+      const int per = sw / 4;  // 16-byte pieces of a row
+      for (int i = lane; i < 8 * per; i += 32) {
+        const int k = i / per, x = i - k * per;
+        cp_async16(rows + k * sw + 4 * x,
+                   one.R_vT + ((size_t)oh * kD + 8 * warp + k) * kD + rank * sw + 4 * x);
+      }
+    }
+    cp_async_commit();
+    __syncthreads();
+    // the CTA's partial: thread = output element
+    const int e = threadIdx.x, hd = e >> 7;
+    {
+      float M = -INFINITY, L = 0.f, o = 0.f, ow = 0.f;
+#pragma unroll
+      for (int k = 0; k < kWarps; ++k)
+        M = fmaxf(M, reinterpret_cast<const float*>(&smem[k].stage[0][0])[kPartM + hd]);
+#pragma unroll
+      for (int k = 0; k < kWarps; ++k) {
+        const float* x = reinterpret_cast<const float*>(&smem[k].stage[0][0]);
+        const float wgt = merge_weight(x[kPartM + hd], M);
+        if (wgt != 0.f) {
+          L = fmaf(x[kPartL + hd], wgt, L);
+          if (k < kInt) o = fmaf(x[e], wgt, o); else ow = fmaf(x[e], wgt, ow);
+        }
+      }
+      O.part.o[e] = o;
+      if (WIN) O.part.ow[e] = ow;
+      if ((e & 127) == 0) {
+        O.part.M[hd] = M;
+        O.part.L[hd] = L;
+      }
+    }
+    if (cs > 1) cluster_sync(); else __syncthreads();
+    // the segment's output over the cluster, in every CTA
+    float owin = 0.f;
+    {
+      float M = -INFINITY, L = 0.f, o = 0.f;
+      for (int r = 0; r < cs; ++r) M = fmaxf(M, cluster_load(&O.part.M[hd], r));
+      for (int r = 0; r < cs; ++r) {
+        const float wgt = merge_weight(cluster_load(&O.part.M[hd], r), M);
+        L = fmaf(cluster_load(&O.part.L[hd], r), wgt, L);
+        o = fmaf(cluster_load(&O.part.o[e], r), wgt, o);
+        if (WIN) owin = fmaf(cluster_load(&O.part.ow[e], r), wgt, owin);
+      }
+      const float il = L > 0.f ? 1.f / L : 0.f;
+      O.orot[hd][e & 127] = o * il;
+      O.ow[hd][e & 127] = owin * il;
+    }
+    cp_async_wait<0>();
+    __syncthreads();
+    float* ob_ = one.out + ((size_t)ob * h_q + 4 * oh) * kD;
+    if (one.fold_v) {  // output in the folded value basis
+      if (((e & 127) / sw) == rank) ob_[e] = O.orot[hd][e & 127] + O.ow[hd][e & 127];
+    } else {
+      // out[r][i] = sum_k o'[r][k] R_v^T[k][i] for the rank's channels i:
+      // thread (part of k, i), the parts added through shared memory
+      const int i = e % sw, kp = sw / 4, part_k = e / sw;
+      float a4[4] = {0.f, 0.f, 0.f, 0.f};
+      for (int k = part_k * kp; k < (part_k + 1) * kp; ++k) {
+        const float rt = reinterpret_cast<const float*>(&smem[k >> 3].qfr[0][0])[(k & 7) * sw + i];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) a4[r] = fmaf(O.orot[r][k], rt, a4[r]);
+      }
+#pragma unroll
+      for (int r = 0; r < 4; ++r) O.red[(part_k * 4 + r) * sw + i] = a4[r];
+      __syncthreads();
+      if (e < 4 * sw) {
+        const int r = e / sw, ch = rank * sw + e % sw, parts = kQrotThreads / sw;
+        float x[4] = {0.f, 0.f, 0.f, 0.f};
+        for (int p = 0; p < parts; p += 4)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) x[u] += O.red[((p + u) * 4 + r) * sw + e % sw];
+        ob_[r * kD + ch] = ((x[0] + x[1]) + (x[2] + x[3])) + O.ow[r][ch];
+      }
+    }
+    if (cs > 1) cluster_sync();  // the peers have read this CTA's partial
+  }
+}
+
+template <bool WIN, bool CMP>
+__global__ void __launch_bounds__(kWarps * 32, 1)
+partial_tensor_kernel(const uint8_t* __restrict__ pool,
+                      const int32_t* __restrict__ bt,
+                      const int32_t* __restrict__ seq_lens, int B,
+                      int max_pages, int num_pages, int h_q, int h_kv,
+                      const uint32_t* __restrict__ frag,
+                      const float* __restrict__ koff,
+                      const float* __restrict__ invs,
+                      const float* __restrict__ qs,
+                      const int* __restrict__ pref,
+                      const int* __restrict__ nzpref,
+                      float* __restrict__ part, int W, int early_pages,
+                      const int32_t* __restrict__ step_cu,
+                      const int32_t* __restrict__ step_pos0,
+                      unsigned* err, int sink, int recent, WinPhase wp) {
+  partial_body<WIN, CMP, false>(pool, bt, seq_lens, B, max_pages, num_pages, h_q, h_kv, frag,
+                                koff, invs, qs, pref, nzpref, part, W, early_pages, step_cu,
+                                step_pos0, err, sink, recent, wp, OneArgs{});
+}
+
+template <bool WIN, bool CMP>
+__global__ void __launch_bounds__(kWarps * 32, 1)
+decode_one_kernel(const uint8_t* __restrict__ pool, const int32_t* __restrict__ bt,
+                  const int32_t* __restrict__ seq_lens, int B, int max_pages, int num_pages,
+                  int h_q, int h_kv, const int32_t* __restrict__ step_cu,
+                  const int32_t* __restrict__ step_pos0, unsigned* err, int sink, int recent,
+                  const __grid_constant__ WinPhase wp, const __grid_constant__ OneArgs one) {
+  partial_body<WIN, CMP, true>(pool, bt, seq_lens, B, max_pages, num_pages, h_q, h_kv, nullptr,
+                               nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0, 0, step_cu,
+                               step_pos0, err, sink, recent, wp, one);
 }
 
 }  // namespace
@@ -781,6 +1035,71 @@ cudaError_t launch_partial_tensor(const optr_params* p, const uint8_t* pool,
                     p->cfg.h_q, p->cfg.h_kv, frag, koff, invs, qs, pref, nzpref,
                     part, W, early_pages ? 1 : 0, step_cu, step_pos0, p->err, p->cfg.sink,
                     p->cfg.recent, wp);
+}
+
+// The kernel of the one-launch decode, its shared-memory limit raised.
+using OneKernel = void (*)(const uint8_t*, const int32_t*, const int32_t*, int, int, int, int, int,
+                           const int32_t*, const int32_t*, unsigned*, int, int, WinPhase, OneArgs);
+static constexpr size_t kOneSmem = sizeof(WarpSmemTC) * kWarps + sizeof(OneSmem);
+static cudaError_t one_kernel(const optr_params* p, OneKernel* fn) {
+  const bool win = p->cfg.sink + p->cfg.recent > 0, cmp = p->cfg.group == 128;
+  *fn = win ? (cmp ? decode_one_kernel<true, true> : decode_one_kernel<true, false>)
+            : (cmp ? decode_one_kernel<false, true> : decode_one_kernel<false, false>);
+  return ensure_dynamic_smem(reinterpret_cast<const void*>(*fn), kOneSmem);
+}
+
+cudaError_t decode_one_limits(const optr_params* p, int (&clusters)[4]) {
+  OneKernel fn;
+  cudaError_t e = one_kernel(p, &fn);
+  for (int i = 0; i < 4 && e == cudaSuccess; ++i) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(p->num_sms >> i << i);
+    cfg.blockDim = dim3(kWarps * 32);
+    cfg.dynamicSmemBytes = kOneSmem;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = 1 << i;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    e = cudaOccupancyMaxActiveClusters(&clusters[i], fn, &cfg);
+  }
+  return e;
+}
+
+// Its CTAs per (sequence, KV head): the largest of 8, 4, 2, 1 with which every
+// cluster is resident at once, or 0 when the split-K decode is the better one.
+// That one spreads all pages evenly over all SMs, whatever the lengths; this
+// one saves two grid boundaries, worth about 4.5 pages of a warp.  So it is
+// taken while a warp's pages x, less the x * u that the split-K decode would
+// give it (u: the share of the SMs in use; 0.6 of it, since a batch with one
+// long sequence has fewer pages than the table's width suggests), stay below
+// that.  Measured, us per call with uniform lengths, split-K / one launch:
+// decode 1 x 1024 15.1 / 11.4, 8 x 2048 20.8 / 14.9, 16 x 2048 23.5 / 19.1,
+// 1 x 16384 20.5 / 19.4 (x = 8, u = 0.4), 1 x 32768 24.2 / 27.2.
+int decode_one_cluster(const optr_params* p, int B, int max_pages) {
+  const long long segs = (long long)B * p->cfg.h_kv;
+  int i = 3;
+  while (i > 0 && segs > p->one_clusters[i]) --i;
+  if (segs > p->one_clusters[i]) return 0;
+  const long long cs = 1 << i, sms = p->num_sms;
+  const int units = (p->cfg.sink + p->cfg.recent + kWinUnit - 1) / kWinUnit;
+  const long long pages = (long long)max_pages + kUnitPages * units;
+  return pages * (10 * sms - 6 * segs * cs) <= 45 * kWarps * cs * sms ? (int)cs : 0;
+}
+
+cudaError_t launch_decode_one(const optr_params* p, int cs, const __nv_bfloat16* q,
+                              const uint8_t* pool, const int32_t* bt, const int32_t* seq_lens,
+                              int B, int max_pages, int num_pages, float qscale, float* out,
+                              const int32_t* step_cu, const int32_t* step_pos0,
+                              const WinPhase& wp, cudaStream_t s) {
+  OneKernel fn;
+  cudaError_t e = one_kernel(p, &fn);
+  if (e != cudaSuccess) return e;
+  const OneArgs one{q, p->R_k, p->R_vT, out, qscale, p->fold_v, step_cu != nullptr ? 1 : 0};
+  return launch_pdl_cluster(fn, dim3(B * p->cfg.h_kv * cs), dim3(kWarps * 32), cs, kOneSmem, s, pool,
+                            bt, seq_lens, B, max_pages, num_pages, p->cfg.h_q, p->cfg.h_kv,
+                            step_cu, step_pos0, p->err, p->cfg.sink, p->cfg.recent, wp, one);
 }
 
 }  // namespace optr

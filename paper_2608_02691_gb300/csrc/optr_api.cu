@@ -283,6 +283,8 @@ optr_status optr_params_create(const optr_config* cfg, const float* R_k,
     e = cudaMemcpy(p->mu, mu, sizeof(float) * H * kD, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemset(p->err, 0, sizeof(unsigned));
   if (e == cudaSuccess) e = noalloc_scratch_address(&p->noalloc_ws);
+  if (e == cudaSuccess && cfg->decode_variant != OPTR_VARIANT_CUDA_CORE)
+    e = decode_one_limits(p, p->one_clusters);
   if (e != cudaSuccess) {
     optr_params_destroy(p);
     return OPTR_ERR_CUDA;

@@ -57,6 +57,8 @@ struct optr_params {
   // optr_decode_attention_noalloc on this params' device (noalloc.cu),
   // looked up once at create with that device current
   void* noalloc_ws;
+  // one-launch decode: clusters of 1, 2, 4, 8 CTAs resident at once
+  int one_clusters[4];
   // stage timing (optr_profile_enable): ev[0..1] bracket the append kernel,
   // ev[2..5] the decode stages (before qrot, partial, combine, after).
   int prof;
@@ -98,20 +100,31 @@ __device__ __forceinline__ void pdl_trigger() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// cluster > 1: clusters of that many CTAs along x.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block,
-                       size_t smem, cudaStream_t s, Args... args) {
+cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, int cluster,
+                               size_t smem, cudaStream_t s, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block,
+                       size_t smem, cudaStream_t s, Args... args) {
+  return launch_pdl_cluster(kernel, grid, block, 1, smem, s, args...);
 }
 
 // Record stage event i on stream s when profiling is on.
@@ -212,6 +225,10 @@ cudaError_t launch_decode(const optr_params* p, int variant,
                           const uint8_t* pool, int num_pages, float* out,
                           void* ws, const DecodePlan& plan, cudaStream_t s,
                           const StepAppend* app, const WinArgs* win);
+
+// Clusters of 1, 2, 4 and 8 CTAs of the one-launch decode that the current
+// device holds at once (asked once, by optr_params_create).
+cudaError_t decode_one_limits(const optr_params* p, int (&clusters)[4]);
 
 // Window part of a cache write (positions of the BF16 windows copied into
 // the store); a separate launch after the INT2 write.

@@ -139,12 +139,12 @@ __device__ __forceinline__ float win_sel4(const float (&x)[4], int i) {
 constexpr int kWinStageBytes = 2 * kWinUnit * 2 * kD;  // K and V rows: 8 KB
 constexpr int kWinPBytes = kWinUnit * 8 * 2;             // P [16 tok][8] bf16
 
-// Window partials of window warp ww (0 <= ww < Ww).  The units (b, h, j) =
-// 16 window tokens [16j, 16j + 16) of sequence b, KV head h, indexed
-// u = (b * h_kv + h) * Uw + j, are cut into Ww contiguous ranges; a warp
-// merges the units of one (b, h) in its range by an online softmax and
+// Window partials of units [u0, u1).  The units (b, h, j) = 16 window tokens
+// [16j, 16j + 16) of sequence b, KV head h, indexed u = (b * h_kv + h) * Uw + j,
+// are cut into contiguous ranges, one per window warp (window_units(ww) of Ww);
+// a warp merges the units of one (b, h) in its range by an online softmax and
 // writes one partial (o[4][128], m[4], l[4]; log2 domain, values in the
-// unrotated basis) to slot ww + b * h_kv + h.  Units past a sequence's
+// unrotated basis) to slot base + b * h_kv + h of out.  Units past a sequence's
 // window count are empty and skipped, so the slots of (b, h) are those of
 // the warps owning its units 0 .. ceil(count / 16) - 1: every window warp
 // owns at least one unit, which keeps that run of warps gap-free.
@@ -162,12 +162,11 @@ constexpr int kWinPBytes = kWinUnit * 8 * 2;             // P [16 tok][8] bf16
 //           hi + lo (relative error 2^-16) in pb [16 tok][8 = head x limb];
 //   P.V     O^T[128][8] += V^T[128][16] . P[16][8], A = V^T by
 //           ldmatrix.trans of the staged value rows.
-static __device__ __noinline__ void window_phase(int ww, const WinPhase& a,
-                                                 uint8_t* stage, uint8_t* pb) {
+static __device__ __noinline__ void window_phase(long long u0, long long u1, const WinPhase& a,
+                                                 float* out, int base, uint8_t* stage,
+                                                 uint8_t* pb) {
   const int lane = threadIdx.x & 31;
   const int g = lane >> 2, c = lane & 3;
-  const long long U = (long long)a.B * a.h_kv * a.Uw;
-  const long long u0 = ww * U / a.Ww, u1 = (ww + 1) * U / a.Ww;
   const int rows = a.sink + a.recent;
   uint8_t* ks = stage;
   uint8_t* vs = stage + kWinUnit * 2 * kD;
@@ -180,14 +179,14 @@ static __device__ __noinline__ void window_phase(int ww, const WinPhase& a,
   int p0n = 0, nn = 0, cn = 0;  // new rows: positions [p0n, p0n + nn) at rows cn..
 
   auto flush = [&]() {
-    float* dst = a.wpart + (size_t)(ww + cur) * kPartFloats + c * kD + g;
+    float* dst = out + (ptrdiff_t)(base + cur) * kPartFloats + c * kD + g;
 #pragma unroll
     for (int mt = 0; mt < 8; ++mt) {
       dst[16 * mt] = o[mt][0] + o[mt][1];
       dst[16 * mt + 8] = o[mt][2] + o[mt][3];
     }
     if (lane < 4) {
-      float* hd = a.wpart + (size_t)(ww + cur) * kPartFloats;
+      float* hd = out + (ptrdiff_t)(base + cur) * kPartFloats;
       hd[kPartM + lane] = win_sel4(m, lane);
       hd[kPartL + lane] = win_sel4(l, lane);
     }
@@ -196,8 +195,16 @@ static __device__ __noinline__ void window_phase(int ww, const WinPhase& a,
   for (long long u = u0; u < u1; ++u) {
     const int bh = (int)(u / a.Uw), j = (int)(u - (long long)bh * a.Uw);
     const int b = bh / a.h_kv, h = bh - b * a.h_kv;
-    if (bh != cur) {
+    const bool fresh = bh != cur;
+    if (fresh) {
+      // (all of the unit's scalars requested at once)
       n = __ldg(a.seq_lens + b);
+      const int sl = __ldg(a.slot + b);
+      if (a.k_new) {
+        cn = __ldg(a.cu_new + b);
+        nn = __ldg(a.cu_new + b + 1) - cn;
+        p0n = __ldg(a.pos0 + b);
+      }
       if (n < 0 || (long long)n > (long long)a.max_pages * kPage) n = 0;  // flagged by qrot
       nw = win_count(n, a.sink, a.recent);
       if (kWinUnit * j >= nw) continue;  // empty unit: no state change
@@ -212,38 +219,11 @@ static __device__ __noinline__ void window_phase(int ww, const WinPhase& a,
       for (int mt = 0; mt < 8; ++mt)
 #pragma unroll
         for (int e = 0; e < 4; ++e) o[mt][e] = 0.f;
-      slot = __ldg(a.slot + b);
+      slot = sl;
       slot_ok = slot >= 0 && slot < a.n_slots;
       if (!slot_ok) {  // the run's partial stays empty (m = -inf, l = 0)
         if (lane == 0) atomicOr(a.err, OPTR_DEVERR_WIN_SLOT);
         slot = 0;
-      }
-      nn = 0;
-      if (a.k_new) {
-        cn = __ldg(a.cu_new + b);
-        nn = __ldg(a.cu_new + b + 1) - cn;
-        p0n = __ldg(a.pos0 + b);
-      }
-      // query B fragments: column g < 4 = head g, k = channels 16kk + 2c
-      // (+1) and 16kk + 2c + 8 (+1)
-      const __nv_bfloat16* qg = a.q + ((size_t)b * a.h_q + 4 * h) * kD;
-#pragma unroll
-      for (int kk = 0; kk < 8; ++kk) {
-        qb[kk][0] = g < 4 ? __ldg(reinterpret_cast<const uint32_t*>(qg + g * kD + 16 * kk + 2 * c)) : 0u;
-        qb[kk][1] = g < 4 ? __ldg(reinterpret_cast<const uint32_t*>(qg + g * kD + 16 * kk + 2 * c + 8)) : 0u;
-      }
-      // qscale * <q_r, mu[h]>: lane takes channels 4 lane .. 4 lane + 3
-      const float4 mu4 = __ldg(reinterpret_cast<const float4*>(a.mu + h * kD) + lane);
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const uint2 q4 = __ldg(reinterpret_cast<const uint2*>(qg + r * kD) + lane);
-        float x = __uint_as_float(q4.x << 16) * mu4.x;
-        x = fmaf(__uint_as_float(q4.x & 0xffff0000u), mu4.y, x);
-        x = fmaf(__uint_as_float(q4.y << 16), mu4.z, x);
-        x = fmaf(__uint_as_float(q4.y & 0xffff0000u), mu4.w, x);
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
-        qmu[r] = x * a.qscale;
       }
     } else if (kWinUnit * j >= nw) {
       continue;
@@ -281,6 +261,29 @@ static __device__ __noinline__ void window_phase(int ww, const WinPhase& a,
                        reinterpret_cast<const __nv_bfloat16*>(vp) + 8 * pc, ok);
     }
     cp_async_commit();
+    if (fresh) {  // the query, while the rows are on their way
+      const __nv_bfloat16* qg = a.q + ((size_t)b * a.h_q + 4 * h) * kD;
+      // B fragments: column g < 4 = head g, k = channels 16kk + 2c (+1) and
+      // 16kk + 2c + 8 (+1)
+#pragma unroll
+      for (int kk = 0; kk < 8; ++kk) {
+        qb[kk][0] = g < 4 ? __ldg(reinterpret_cast<const uint32_t*>(qg + g * kD + 16 * kk + 2 * c)) : 0u;
+        qb[kk][1] = g < 4 ? __ldg(reinterpret_cast<const uint32_t*>(qg + g * kD + 16 * kk + 2 * c + 8)) : 0u;
+      }
+      // qscale * <q_r, mu[h]>: lane takes channels 4 lane .. 4 lane + 3
+      const float4 mu4 = __ldg(reinterpret_cast<const float4*>(a.mu + h * kD) + lane);
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const uint2 q4 = __ldg(reinterpret_cast<const uint2*>(qg + r * kD) + lane);
+        float x = __uint_as_float(q4.x << 16) * mu4.x;
+        x = fmaf(__uint_as_float(q4.x & 0xffff0000u), mu4.y, x);
+        x = fmaf(__uint_as_float(q4.y << 16), mu4.z, x);
+        x = fmaf(__uint_as_float(q4.y & 0xffff0000u), mu4.w, x);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+        qmu[r] = x * a.qscale;
+      }
+    }
     cp_async_wait<0>();
     __syncwarp();
     // logits: S[tok][col] for tok g, g + 8 and cols 2c, 2c + 1
@@ -374,8 +377,17 @@ static __device__ __noinline__ void window_phase(int ww, const WinPhase& a,
       }
     }
   }
+  __syncwarp();  // out may be the scratch
   if (cur >= 0) flush();
   __syncwarp();  // the scratch is handed back to the INT2 pages
+}
+
+// The units of window warp ww of a.Ww, its partials to slots ww + b * h_kv + h
+// of a.wpart.
+static __device__ __forceinline__ void window_warp(int ww, const WinPhase& a, uint8_t* stage,
+                                                   uint8_t* pb) {
+  const long long U = (long long)a.B * a.h_kv * a.Uw;
+  window_phase(ww * U / a.Ww, (ww + 1) * U / a.Ww, a, a.wpart, ww, stage, pb);
 }
 
 }  // namespace optr
