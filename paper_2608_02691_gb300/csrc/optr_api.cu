@@ -10,6 +10,8 @@
 #include <mutex>
 #include <vector>
 
+#include <cudaTypedefs.h>
+
 #include "optr_internal.cuh"
 
 using namespace optr;
@@ -31,7 +33,33 @@ size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // mapping (*host set), which the kernels then read or write in place over
 // the host link.  Pageable host memory, or a pointer the runtime does not
 // know, is refused (false), so no kernel ever dereferences it.
+//
+// Device memory is the common answer and the driver gives it alone faster
+// than cudaPointerGetAttributes gives every attribute.
+PFN_cuPointerGetAttribute_v4000 pointer_attribute_fn() {
+  static PFN_cuPointerGetAttribute_v4000 fn = nullptr;
+  static std::once_flag once;
+  std::call_once(once, [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &f, 4000, cudaEnableDefault,
+                                         &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      fn = reinterpret_cast<PFN_cuPointerGetAttribute_v4000>(f);
+  });
+  return fn;
+}
+
 bool io_pointer(const void* ptr, const void** dev, bool* host) {
+  unsigned type = 0;
+  if (auto fn = pointer_attribute_fn())
+    if (fn(&type, CU_POINTER_ATTRIBUTE_MEMORY_TYPE, reinterpret_cast<CUdeviceptr>(ptr)) ==
+            CUDA_SUCCESS &&
+        type == CU_MEMORYTYPE_DEVICE) {
+      *dev = ptr;
+      if (host) *host = false;
+      return true;
+    }
   cudaPointerAttributes a;
   if (cudaPointerGetAttributes(&a, ptr) != cudaSuccess) {
     (void)cudaGetLastError();  // the failed query leaves no error behind

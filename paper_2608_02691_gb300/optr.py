@@ -105,6 +105,8 @@ def library_path() -> str:
 def lib():
     """The loaded ``liboptr.so``; raises if it has not been built."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             path = _build.LIB
@@ -113,6 +115,7 @@ def lib():
                     f"{path} is missing: build the CUDA library first "
                     "(python -c 'import __graft_entry__ as g; g.build()')")
             L = ctypes.CDLL(path)
+            L.raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
             for name, (res, args) in _SIG.items():
                 fn = getattr(L, name)
                 fn.restype = res
@@ -135,10 +138,19 @@ def _ptr(t):
 
 
 def _stream(stream):
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    raw = lib().raw_stream  # the handle without a Stream object around it
+    if raw is not None:
+        return raw(torch.cuda.current_device())
+    return torch.cuda.current_stream().cuda_stream
 
+
+# The binding is on the path of every token, and for a small batch a call's
+# time is mostly its host time: pointers go to ctypes as plain integers, the
+# checks are three attribute reads per tensor, and whether a host tensor is
+# pinned is left to the library (which refuses any other host memory before
+# any launch) and asked here only to word the error.
 
 # per-step activations: CUDA tensors or pinned host tensors, which the
 # kernels read or write in place
@@ -146,11 +158,30 @@ _IO = ("q", "k", "v", "out")
 
 
 def _dev(t, dtype, name):
-    where = t.is_cuda or (name in _IO and t.is_pinned())
-    if not (where and t.dtype == dtype and t.is_contiguous()):
-        kind = "CUDA or pinned host" if name in _IO else "CUDA"
-        raise ValueError(f"{name} must be a contiguous {kind} {dtype} tensor")
-    return t
+    """The data pointer of t, a contiguous CUDA tensor of the dtype."""
+    if t.dtype is dtype and t.is_cuda and t.is_contiguous():
+        return t.data_ptr()
+    kind = "CUDA or pinned host" if name in _IO else "CUDA"
+    raise ValueError(f"{name} must be a contiguous {kind} {dtype} tensor")
+
+
+def _act(t, dtype, name):
+    """_dev for an activation, which may also be pinned host memory; an empty
+    host tensor is looked at here, since the library may not."""
+    if t.dtype is dtype and t.is_contiguous() and (
+            t.is_cuda or (t.device.type == "cpu" and (t.numel() > 0 or t.is_pinned()))):
+        return t.data_ptr()
+    return _dev(t, dtype, name)
+
+
+def _done(status: int, what: str, *acts):
+    """Raises for a status other than 0: a pageable activation among the
+    named ones first."""
+    if status != 0:
+        for t, name in acts:
+            if not t.is_cuda and not t.is_pinned():
+                _dev(t, t.dtype, name)
+        raise OptrError(status, what)
 
 
 class Params:
@@ -211,18 +242,15 @@ def optr_kv_append(p: Params, k, v, cu_new, pos0, block_table, pool,
                    stream=None) -> None:
     """k, v bf16 [n_tok][h_kv][128]; cu_new int32 [B+1]; pos0 int32 [B];
     block_table int32 [B][max_pages]; pool uint8 [num_pages][h_kv][1536]."""
-    _dev(k, torch.bfloat16, "k")
-    _dev(v, torch.bfloat16, "v")
-    _dev(cu_new, torch.int32, "cu_new")
-    _dev(pos0, torch.int32, "pos0")
-    _dev(block_table, torch.int32, "block_table")
-    _dev(pool, torch.uint8, "pool")
+    bf16, i32 = torch.bfloat16, torch.int32
+    kp, vp = _act(k, bf16, "k"), _act(v, bf16, "v")
     B, max_pages = block_table.shape
-    _check(lib().optr_kv_append(p.handle, _ptr(k), _ptr(v), k.shape[0],
-                                _ptr(cu_new), _ptr(pos0), _ptr(block_table),
-                                B, max_pages, _ptr(pool), pool.shape[0],
-                                _stream(stream)),
-           "optr_kv_append")
+    st = lib().optr_kv_append(
+        p.handle, kp, vp, k.shape[0], _dev(cu_new, i32, "cu_new"), _dev(pos0, i32, "pos0"),
+        _dev(block_table, i32, "block_table"), B, max_pages, _dev(pool, torch.uint8, "pool"),
+        pool.shape[0], _stream(stream))
+    if st:
+        _done(st, "optr_kv_append", (k, "k"), (v, "v"))
 
 
 def optr_decode_workspace_size(p: Params, B: int, max_pages: int) -> int:
@@ -233,17 +261,15 @@ def optr_decode_attention(p: Params, q, block_table, seq_lens, pool, out,
                           workspace, stream=None) -> None:
     """q bf16 [B][h_q][128]; out float32 [B][h_q][128]; workspace uint8 of
     at least optr_decode_workspace_size bytes (256-byte aligned)."""
-    _dev(q, torch.bfloat16, "q")
-    _dev(block_table, torch.int32, "block_table")
-    _dev(seq_lens, torch.int32, "seq_lens")
-    _dev(pool, torch.uint8, "pool")
-    _dev(out, torch.float32, "out")
-    _dev(workspace, torch.uint8, "workspace")
+    i32, u8 = torch.int32, torch.uint8
     B, max_pages = block_table.shape
-    _check(lib().optr_decode_attention(
-        p.handle, _ptr(q), _ptr(block_table), _ptr(seq_lens), B, max_pages,
-        _ptr(pool), pool.shape[0], _ptr(out), _ptr(workspace),
-        workspace.numel(), _stream(stream)), "optr_decode_attention")
+    st = lib().optr_decode_attention(
+        p.handle, _act(q, torch.bfloat16, "q"), _dev(block_table, i32, "block_table"),
+        _dev(seq_lens, i32, "seq_lens"), B, max_pages, _dev(pool, u8, "pool"), pool.shape[0],
+        _act(out, torch.float32, "out"), _dev(workspace, u8, "workspace"), workspace.numel(),
+        _stream(stream))
+    if st:
+        _done(st, "optr_decode_attention", (q, "q"), (out, "out"))
 
 
 def optr_decode_step(p: Params, q, k, v, cu_new, pos0, block_table, seq_lens,
@@ -251,20 +277,16 @@ def optr_decode_step(p: Params, q, k, v, cu_new, pos0, block_table, seq_lens,
     """optr_kv_append of the step's new tokens (k, v, cu_new, pos0) followed
     by optr_decode_attention over the updated cache; seq_lens counts the new
     tokens."""
-    for t, dt, nm in ((q, torch.bfloat16, "q"), (k, torch.bfloat16, "k"),
-                      (v, torch.bfloat16, "v"), (cu_new, torch.int32, "cu_new"),
-                      (pos0, torch.int32, "pos0"),
-                      (block_table, torch.int32, "block_table"),
-                      (seq_lens, torch.int32, "seq_lens"),
-                      (pool, torch.uint8, "pool"), (out, torch.float32, "out"),
-                      (workspace, torch.uint8, "workspace")):
-        _dev(t, dt, nm)
+    bf16, i32, u8 = torch.bfloat16, torch.int32, torch.uint8
     B, max_pages = block_table.shape
-    _check(lib().optr_decode_step(
-        p.handle, _ptr(q), _ptr(k), _ptr(v), k.shape[0], _ptr(cu_new),
-        _ptr(pos0), _ptr(block_table), _ptr(seq_lens), B, max_pages,
-        _ptr(pool), pool.shape[0], _ptr(out), _ptr(workspace),
-        workspace.numel(), _stream(stream)), "optr_decode_step")
+    st = lib().optr_decode_step(
+        p.handle, _act(q, bf16, "q"), _act(k, bf16, "k"), _act(v, bf16, "v"), k.shape[0],
+        _dev(cu_new, i32, "cu_new"), _dev(pos0, i32, "pos0"),
+        _dev(block_table, i32, "block_table"), _dev(seq_lens, i32, "seq_lens"), B, max_pages,
+        _dev(pool, u8, "pool"), pool.shape[0], _act(out, torch.float32, "out"),
+        _dev(workspace, u8, "workspace"), workspace.numel(), _stream(stream))
+    if st:
+        _done(st, "optr_decode_step", (q, "q"), (k, "k"), (v, "v"), (out, "out"))
 
 
 def optr_window_bytes(p: Params, n_slots: int) -> int:
@@ -274,46 +296,43 @@ def optr_window_bytes(p: Params, n_slots: int) -> int:
 def _win_args(p, win, win_slot):
     if win is None:
         return None, None, 0
-    _dev(win, torch.bfloat16, "win")
-    _dev(win_slot, torch.int32, "win_slot")
-    rows = p.cfg.sink + p.cfg.recent
-    if tuple(win.shape[1:]) != (p.h_kv, 2, rows, 128):
+    ptr, slots = _dev(win, torch.bfloat16, "win"), _dev(win_slot, torch.int32, "win_slot")
+    n, h, two, rows, d = win.shape if win.dim() == 5 else (0,) * 5
+    if h != p.cfg.h_kv or two != 2 or rows != p.cfg.sink + p.cfg.recent or d != 128:
         raise ValueError("win must be [n_slots][h_kv][2][sink + recent][128]")
-    return _ptr(win), _ptr(win_slot), win.shape[0]
+    return ptr, slots, n
 
 
 def optr_kv_append_win(p: Params, k, v, cu_new, pos0, block_table, pool, win,
                        win_slot, stream=None) -> None:
     """optr_kv_append plus the BF16-window copy: win bf16
     [n_slots][h_kv][2][sink + recent][128], win_slot int32 [B]."""
-    for t, dt, nm in ((k, torch.bfloat16, "k"), (v, torch.bfloat16, "v"),
-                      (cu_new, torch.int32, "cu_new"), (pos0, torch.int32, "pos0"),
-                      (block_table, torch.int32, "block_table"),
-                      (pool, torch.uint8, "pool")):
-        _dev(t, dt, nm)
+    bf16, i32 = torch.bfloat16, torch.int32
+    kp, vp = _act(k, bf16, "k"), _act(v, bf16, "v")
+    cu, p0, bt = _dev(cu_new, i32, "cu_new"), _dev(pos0, i32, "pos0"), _dev(block_table, i32, "block_table")
+    pl = _dev(pool, torch.uint8, "pool")
     w, ws_, n_slots = _win_args(p, win, win_slot)
     B, max_pages = block_table.shape
-    _check(lib().optr_kv_append_win(
-        p.handle, _ptr(k), _ptr(v), k.shape[0], _ptr(cu_new), _ptr(pos0),
-        _ptr(block_table), B, max_pages, _ptr(pool), pool.shape[0], w, ws_,
-        n_slots, _stream(stream)), "optr_kv_append_win")
+    st = lib().optr_kv_append_win(p.handle, kp, vp, k.shape[0], cu, p0, bt, B, max_pages, pl,
+                                  pool.shape[0], w, ws_, n_slots, _stream(stream))
+    if st:
+        _done(st, "optr_kv_append_win", (k, "k"), (v, "v"))
 
 
 def optr_decode_attention_win(p: Params, q, block_table, seq_lens, pool, win,
                               win_slot, out, workspace, stream=None) -> None:
     """optr_decode_attention with the BF16 windows read from win."""
-    for t, dt, nm in ((q, torch.bfloat16, "q"),
-                      (block_table, torch.int32, "block_table"),
-                      (seq_lens, torch.int32, "seq_lens"),
-                      (pool, torch.uint8, "pool"), (out, torch.float32, "out"),
-                      (workspace, torch.uint8, "workspace")):
-        _dev(t, dt, nm)
+    i32, u8 = torch.int32, torch.uint8
+    qp, bt = _act(q, torch.bfloat16, "q"), _dev(block_table, i32, "block_table")
+    lens, pl = _dev(seq_lens, i32, "seq_lens"), _dev(pool, u8, "pool")
+    op, wsp = _act(out, torch.float32, "out"), _dev(workspace, u8, "workspace")
     w, ws_, n_slots = _win_args(p, win, win_slot)
     B, max_pages = block_table.shape
-    _check(lib().optr_decode_attention_win(
-        p.handle, _ptr(q), _ptr(block_table), _ptr(seq_lens), B, max_pages,
-        _ptr(pool), pool.shape[0], w, ws_, n_slots, _ptr(out), _ptr(workspace),
-        workspace.numel(), _stream(stream)), "optr_decode_attention_win")
+    st = lib().optr_decode_attention_win(p.handle, qp, bt, lens, B, max_pages, pl, pool.shape[0],
+                                         w, ws_, n_slots, op, wsp, workspace.numel(),
+                                         _stream(stream))
+    if st:
+        _done(st, "optr_decode_attention_win", (q, "q"), (out, "out"))
 
 
 def optr_decode_step_win(p: Params, q, k, v, cu_new, pos0, block_table,
@@ -321,21 +340,18 @@ def optr_decode_step_win(p: Params, q, k, v, cu_new, pos0, block_table,
                          stream=None) -> None:
     """optr_decode_step with BF16 windows: the step's window copies and the
     windowed decode."""
-    for t, dt, nm in ((q, torch.bfloat16, "q"), (k, torch.bfloat16, "k"),
-                      (v, torch.bfloat16, "v"), (cu_new, torch.int32, "cu_new"),
-                      (pos0, torch.int32, "pos0"),
-                      (block_table, torch.int32, "block_table"),
-                      (seq_lens, torch.int32, "seq_lens"),
-                      (pool, torch.uint8, "pool"), (out, torch.float32, "out"),
-                      (workspace, torch.uint8, "workspace")):
-        _dev(t, dt, nm)
+    bf16, i32, u8 = torch.bfloat16, torch.int32, torch.uint8
+    qp, kp, vp = _act(q, bf16, "q"), _act(k, bf16, "k"), _act(v, bf16, "v")
+    cu, p0, bt = _dev(cu_new, i32, "cu_new"), _dev(pos0, i32, "pos0"), _dev(block_table, i32, "block_table")
+    lens, pl = _dev(seq_lens, i32, "seq_lens"), _dev(pool, u8, "pool")
+    op, wsp = _act(out, torch.float32, "out"), _dev(workspace, u8, "workspace")
     w, ws_, n_slots = _win_args(p, win, win_slot)
     B, max_pages = block_table.shape
-    _check(lib().optr_decode_step_win(
-        p.handle, _ptr(q), _ptr(k), _ptr(v), k.shape[0], _ptr(cu_new),
-        _ptr(pos0), _ptr(block_table), _ptr(seq_lens), B, max_pages,
-        _ptr(pool), pool.shape[0], w, ws_, n_slots, _ptr(out), _ptr(workspace),
-        workspace.numel(), _stream(stream)), "optr_decode_step_win")
+    st = lib().optr_decode_step_win(p.handle, qp, kp, vp, k.shape[0], cu, p0, bt, lens, B, max_pages,
+                                    pl, pool.shape[0], w, ws_, n_slots, op, wsp, workspace.numel(),
+                                    _stream(stream))
+    if st:
+        _done(st, "optr_decode_step_win", (q, "q"), (k, "k"), (v, "v"), (out, "out"))
 
 
 def new_windows(p: Params, n_slots: int, device="cuda") -> torch.Tensor:
@@ -353,16 +369,14 @@ def optr_decode_attention_noalloc(p: Params, q, block_table, seq_lens, pool,
     """Decode without a workspace argument: the library uses its own fixed
     16 MiB device scratch array, so this call allocates nothing.  Calls
     that overlap on the GPU share that array and must be serialised."""
-    _dev(q, torch.bfloat16, "q")
-    _dev(block_table, torch.int32, "block_table")
-    _dev(seq_lens, torch.int32, "seq_lens")
-    _dev(pool, torch.uint8, "pool")
-    _dev(out, torch.float32, "out")
+    i32 = torch.int32
     B, max_pages = block_table.shape
-    _check(lib().optr_decode_attention_noalloc(
-        p.handle, _ptr(q), _ptr(block_table), _ptr(seq_lens), B, max_pages,
-        _ptr(pool), pool.shape[0], _ptr(out), _stream(stream)),
-        "optr_decode_attention_noalloc")
+    st = lib().optr_decode_attention_noalloc(
+        p.handle, _act(q, torch.bfloat16, "q"), _dev(block_table, i32, "block_table"),
+        _dev(seq_lens, i32, "seq_lens"), B, max_pages, _dev(pool, torch.uint8, "pool"),
+        pool.shape[0], _act(out, torch.float32, "out"), _stream(stream))
+    if st:
+        _done(st, "optr_decode_attention_noalloc", (q, "q"), (out, "out"))
 
 
 def optr_device_error(p: Params) -> int:
