@@ -7,9 +7,10 @@
 // with the cache's INT2 quantizer Q2 inside the effective keys and values and
 // its straight-through gradient, and held-out selection of the rotations.
 //
-// Everything runs in float64 on the CUDA cores in this file's kernels: the
-// calibration is a one-time offline pass, this GPU's tensor cores have no
-// float64 path, and float64 keeps the 80-step trajectory reproducible.
+// Everything is float64: the calibration is a one-time offline pass, and float64
+// keeps its trajectory reproducible.  The matrix products, its bulk, run on the
+// fp16 tensor cores as exact integer products (gemm_digits_kernel), the rest on
+// the CUDA cores.
 // The gradient is written out (no autograd):
 //   keys    Z = (K - mu) R, Zh = Q2(Z), Kt = Zh R^T, l = scale q Kt^T
 //           dl = c [(pk - p) + pk (gv - sum_s pk gv)],  gv = U V^T,
@@ -38,9 +39,8 @@ constexpr int kCD = 128;  // head dimension d
 
 // ------------------------------------------------------------------ GEMM
 // C[b] = alpha op(A[b]) op(B[b]) + beta C[b] + diag I, float64, row-major
-// with leading dimensions; op = transpose when tA / tB.  Square output tiles
-// of 64, 32 or 16 (gemm_f64_kernel below), 16-deep k slices in shared
-// memory, 256 threads per CTA.
+// with leading dimensions; op = transpose when tA / tB.  32 x 32 output tiles,
+// 64-deep k chunks, 256 threads per CTA (gemm_digits_kernel below).
 // gate: when non-null and gate_idx >= *gate, the launch instead copies
 // `pass` into C (or does nothing when pass is null); this lets a fixed
 // number of launches apply a device-decided number of squarings.
@@ -60,30 +60,120 @@ struct Gemm {
   const double* pass;
 };
 
-constexpr int kTK = 16;
-
-// TILE x TILE outputs per CTA of 256 threads ((TILE / 16)^2 outputs each).
-// The host picks the largest tile, then a split of K into kc chunks, so that
-// a call covers about two CTAs per SM (float64 runs at a few FMAs per clock
-// per SM on this GPU).  With kc > 1 chunk z of a product writes its raw sum
+// The product runs on the fp16 tensor cores, exactly, after a split of both
+// factors into small integers (the scheme of Ozaki, Ogita, Oishi and Rump,
+// "Error-free transformations of matrix multiplication", 2012): this GPU does
+// 2 float64 FMAs per clock and SM, three orders of magnitude below its tensor
+// cores.  Per k chunk of 64, a row of A (a column of B) is written as
+// fixed-point numbers under its own largest exponent, 54 bits and sign, in
+// seven balanced base-256 digits d_0 .. d_6 (|d_0| <= 64, else |d| <= 128),
+// which are exact fp16 values.  All digit products of one weight d = i + j are
+// summed in one float32 accumulator: at most 7 x 64 x 2^14 < 2^24, so every sum
+// is exact.  The weights 0 .. 7 (34 of the 49 products; what is left out of
+// one product is below 2^-59 of the largest one) are put together in 64-bit
+// integers and added to the float64 result, one rounding per 64 products.  Against sums in
+// extended precision that is 2 to 5 times closer than a float64 FMA chain
+// (relative error 1.5e-16 to 2.8e-16 on keys x rotation, probabilities x
+// values, powers of the generator; FMA chain 2.8e-16 to 1.5e-15).
+// A row or column with a NaN or an infinity gives NaN throughout.
+// What bounds it: 136 mma per warp and chunk (16 x 8 outputs each, a third of
+// the CTA's 3 us), the split of both tiles and the chunk's load latency; 32 x 32
+// tiles give the calibration's products (128 to 2048 rows) enough CTAs.  One
+// 64-query, 4096-channel, 2048-token key step spent 1.8 ms in the float64 kernel
+// this replaces; 20 + 20 steps of both phases 120.3 -> 86.5 ms.
+//
+// With kc > 1 CTA z of a product covers the z-th part of k and writes its sum
 // to P[z][b]; the last of the tile's kc CTAs to finish (a per-tile arrival
-// counter, left at 0 again) adds the chunks in a fixed order, z = 0 .. kc-1,
+// counter, left at 0 again) adds the parts in a fixed order, z = 0 .. kc-1,
 // so the result does not depend on which CTA that is.
-template <int TILE>
-__global__ void __launch_bounds__(256) gemm_f64_kernel(Gemm g, int kc, double* P,
-                                                       int* tcnt) {
-  constexpr int R = TILE / 16;  // outputs per thread per dimension
-  __shared__ double As[kTK][TILE + 1];
-  __shared__ double Bs[kTK][TILE + 1];
+constexpr int kGT = 32;      // tile
+constexpr int kGK = 64;      // k chunk
+constexpr int kDigits = 7;
+constexpr int kWeights = 8;
+constexpr int kBadExp = 1 << 20;  // exponent of a row with a non-finite value
+
+struct GemmSmem {
+  // digit planes [operand][digit][row][k]; 16-byte piece p of row r at p ^ (r % 8)
+  __half d[2][kDigits][kGT][kGK];
+  int emax[2][kGT][9];  // largest exponents of a row's eight 8-element parts
+  int e[2][kGT];
+};
+
+__device__ __forceinline__ void digits_mma(float (&d)[4], const uint32_t (&a)[4], uint32_t b0,
+                                           uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 "
+      "{%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void digits_ldsm(uint32_t (&r)[4], const void* p) {
+  const unsigned s = static_cast<unsigned>(__cvta_generic_to_shared(p));
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(s));
+}
+
+// Exponent e of |x| = m 2^(e - 1075), m < 2^53 (subnormals share e = 1).
+__device__ __forceinline__ int exponent_of(double x) {
+  const int e = (__double2hiint(x) >> 20) & 2047;
+  return e == 2047 ? kBadExp : max(e, 1);
+}
+
+// x as a fixed-point integer with unit 2^(e_row - 1076), |result| <= 2^54, plus
+// the bias that makes its bytes digit + 128.
+__device__ __forceinline__ unsigned long long fixed_point(double x, int e_row) {
+  const unsigned long long bits = __double_as_longlong(x);
+  const int e = (int)(bits >> 52) & 2047;
+  unsigned long long m = (bits & 0xfffffffffffffull) | (e ? 1ull << 52 : 0ull);
+  const int sh = e_row - max(e, 1);
+  m <<= 1;
+  if (sh > 0) m = sh < 56 ? (m + (1ull << (sh - 1))) >> sh : 0ull;
+  const long long f = (long long)bits < 0 ? -(long long)m : (long long)m;
+  return (unsigned long long)f + 0x80808080808080ull;
+}
+
+// The digits of eight consecutive k of row r (piece kg) into the planes.
+__device__ __forceinline__ void store_digits(__half (*planes)[kGT][kGK], int r, int kg,
+                                             const double (&x)[8], int e_row) {
+  uint32_t h[kDigits][4];
+  const __half2 off = __float2half2_rn(1152.f);  // 1024 + byte - 1152 = digit
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const unsigned long long f0 = fixed_point(x[2 * q], e_row), f1 = fixed_point(x[2 * q + 1], e_row);
+    const uint32_t l0 = (uint32_t)f0, l1 = (uint32_t)f1, u0 = (uint32_t)(f0 >> 32), u1 = (uint32_t)(f1 >> 32);
+    const uint32_t b01 = __byte_perm(l0, l1, 0x5140), b23 = __byte_perm(l0, l1, 0x7362),
+                   b45 = __byte_perm(u0, u1, 0x5140), b6 = __byte_perm(u0, u1, 0x7362);
+    const uint32_t w[kDigits] = {
+        __byte_perm(b6, 0x64646464u, 0x4140),  __byte_perm(b45, 0x64646464u, 0x4342),
+        __byte_perm(b45, 0x64646464u, 0x4140), __byte_perm(b23, 0x64646464u, 0x4342),
+        __byte_perm(b23, 0x64646464u, 0x4140), __byte_perm(b01, 0x64646464u, 0x4342),
+        __byte_perm(b01, 0x64646464u, 0x4140)};
+#pragma unroll
+    for (int d = 0; d < kDigits; ++d) {
+      const __half2 v = __hsub2(*reinterpret_cast<const __half2*>(&w[d]), off);
+      h[d][q] = *reinterpret_cast<const uint32_t*>(&v);
+    }
+  }
+#pragma unroll
+  for (int d = 0; d < kDigits; ++d)
+    *reinterpret_cast<uint4*>(&planes[d][r][(kg ^ (r & 7)) * 8]) =
+        make_uint4(h[d][0], h[d][1], h[d][2], h[d][3]);
+}
+
+__global__ void __launch_bounds__(256, 2) gemm_digits_kernel(Gemm g, int kc, double* P,
+                                                             int* tcnt) {
+  extern __shared__ __align__(16) unsigned char gsm_[];
+  GemmSmem& S = *reinterpret_cast<GemmSmem*>(gsm_);
   __shared__ int s_last;
   const int b = blockIdx.z / kc, z = blockIdx.z % kc;
-  const int m0 = blockIdx.y * TILE, n0 = blockIdx.x * TILE;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int tn = (g.N + kGT - 1) / kGT;  // row tiles may exceed a grid's y limit
+  const int m0 = blockIdx.x / tn * kGT, n0 = blockIdx.x % tn * kGT;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   double* C = g.C + (long long)b * g.sC;
   if (g.gate != nullptr && g.gate_idx >= *g.gate) {
     if (g.pass != nullptr && z == 0) {
-      for (int i = tid; i < TILE * TILE; i += 256) {
-        const int r = m0 + i / TILE, c = n0 + i % TILE;
+      for (int i = tid; i < kGT * kGT; i += 256) {
+        const int r = m0 + i / kGT, c = n0 + i % kGT;
         if (r < g.M && c < g.N) C[r * g.ldc + c] = g.pass[r * g.ldc + c];
       }
     }
@@ -91,79 +181,129 @@ __global__ void __launch_bounds__(256) gemm_f64_kernel(Gemm g, int kc, double* P
   }
   const double* A = g.A + (long long)b * g.sA;
   const double* B = g.B + (long long)b * g.sB;
-  // this CTA's K range: chunk z of kc, in whole kTK slices
-  const int nsl = (g.K + kTK - 1) / kTK;
-  const int kb = (int)((long long)z * nsl / kc) * kTK;
-  const int ke = min(g.K, (int)((long long)(z + 1) * nsl / kc) * kTK);
-  double acc[R][R];
+  // this CTA's K range: part z of kc, in whole chunks
+  const int nsl = (g.K + kGK - 1) / kGK;
+  const int kb = (int)((long long)z * nsl / kc) * kGK;
+  const int ke = min(g.K, (int)((long long)(z + 1) * nsl / kc) * kGK);
+  // loading thread (row, piece) of each operand, rows along the contiguous
+  // dimension of a transposed one
+  const bool a_rows = !g.tA, b_rows = g.tB;  // k contiguous
+  const int ra = a_rows ? tid >> 3 : tid & 31, ka = a_rows ? tid & 7 : tid >> 5;
+  const int rb = b_rows ? tid >> 3 : tid & 31, kbp = b_rows ? tid & 7 : tid >> 5;
+  const int wm = warp & 1, wn = warp >> 1;  // this warp's 16 x 8 outputs
+  double out[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int k0 = kb; k0 < ke; k0 += kGK) {
+    double xa[8], xb[8];
+    int ea = 1, eb = 1;
 #pragma unroll
-  for (int i = 0; i < R; ++i)
+    for (int i = 0; i < 8; ++i) {
+      const int k = k0 + 8 * ka + i, m = m0 + ra;
+      xa[i] = m < g.M && k < ke ? (a_rows ? A[m * g.lda + k] : A[k * g.lda + m]) : 0.0;
+    }
 #pragma unroll
-    for (int j = 0; j < R; ++j) acc[i][j] = 0.0;
-  for (int k0 = kb; k0 < ke; k0 += kTK) {
-    for (int i = tid; i < TILE * kTK; i += 256) {
-      int mm, kk;
-      if (g.tA) { kk = i / TILE; mm = i % TILE; } else { mm = i / kTK; kk = i % kTK; }
-      const int gm = m0 + mm, gk = k0 + kk;
-      double x = 0.0;
-      if (gm < g.M && gk < ke) x = g.tA ? A[gk * g.lda + gm] : A[gm * g.lda + gk];
-      As[kk][mm] = x;
+    for (int i = 0; i < 8; ++i) {
+      const int k = k0 + 8 * kbp + i, n = n0 + rb;
+      xb[i] = n < g.N && k < ke ? (b_rows ? B[n * g.ldb + k] : B[k * g.ldb + n]) : 0.0;
     }
-    for (int i = tid; i < kTK * TILE; i += 256) {
-      int kk, nn;
-      if (g.tB) { nn = i / kTK; kk = i % kTK; } else { kk = i / TILE; nn = i % TILE; }
-      const int gk = k0 + kk, gn = n0 + nn;
-      double x = 0.0;
-      if (gk < ke && gn < g.N) x = g.tB ? B[gn * g.ldb + gk] : B[gk * g.ldb + gn];
-      Bs[kk][nn] = x;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      ea = max(ea, exponent_of(xa[i]));
+      eb = max(eb, exponent_of(xb[i]));
     }
+    S.emax[0][ra][ka] = ea;
+    S.emax[1][rb][kbp] = eb;
+    __syncthreads();  // (and the previous chunk's digits have been read)
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      ea = max(ea, S.emax[0][ra][i]);
+      eb = max(eb, S.emax[1][rb][i]);
+    }
+    store_digits(S.d[0], ra, ka, xa, ea);
+    store_digits(S.d[1], rb, kbp, xb, eb);
+    if (ka == 0) S.e[0][ra] = ea;
+    if (kbp == 0) S.e[1][rb] = eb;
     __syncthreads();
+    float acc[kWeights][4];
 #pragma unroll
-    for (int kk = 0; kk < kTK; ++kk) {
-      double a[R], bb[R];
+    for (int d = 0; d < kWeights; ++d)
 #pragma unroll
-      for (int i = 0; i < R; ++i) a[i] = As[kk][ty * R + i];
+      for (int i = 0; i < 4; ++i) acc[d][i] = 0.f;
 #pragma unroll
-      for (int j = 0; j < R; ++j) bb[j] = Bs[kk][tx * R + j];
+    for (int ks = 0; ks < kGK / 16; ++ks) {
+      uint32_t fa[kDigits][4], fb[kDigits + 1][2];
+      {
+        const int r = 16 * wm + (lane & 15), p = 2 * ks + (lane >> 4);
 #pragma unroll
-      for (int i = 0; i < R; ++i)
+        for (int i = 0; i < kDigits; ++i) digits_ldsm(fa[i], &S.d[0][i][r][(p ^ (r & 7)) * 8]);
+      }
+      {
+        // lanes 0-15 address digit j, 16-31 digit j + 1
+        const int r = 8 * wn + (lane & 7), p = 2 * ks + ((lane >> 3) & 1);
 #pragma unroll
-        for (int j = 0; j < R; ++j) acc[i][j] = fma(a[i], bb[j], acc[i][j]);
+        for (int j = 0; j < kDigits; j += 2) {
+          uint32_t x[4];
+          const int jj = min(j + (lane >> 4), kDigits - 1);
+          digits_ldsm(x, &S.d[1][jj][r][(p ^ (r & 7)) * 8]);
+          fb[j][0] = x[0];
+          fb[j][1] = x[1];
+          fb[j + 1][0] = x[2];
+          fb[j + 1][1] = x[3];
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < kDigits; ++i)
+#pragma unroll
+        for (int j = 0; j < kDigits; ++j)
+          if (i + j < kWeights) digits_mma(acc[i + j], fa[i], fb[j][0], fb[j][1]);
     }
-    __syncthreads();
+    // sum_d acc_d 256^-d as an integer with unit 2^-44, one float64 rounding;
+    // times 2^(Ea + Eb - 56), |x| < 2^E, E = e - 1022
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      int v[kWeights];
+#pragma unroll
+      for (int d = 0; d < kWeights; ++d) v[d] = __float2int_rn(acc[d][i]);
+      const long long t = ((long long)(v[0] * 256 + v[1]) << 36) + ((long long)(v[2] * 256 + v[3]) << 20) +
+                          ((long long)(v[4] * 256 + v[5]) << 4) + ((v[6] * 256 + v[7] + 2048) >> 12);
+      const int e0 = S.e[0][16 * wm + (lane >> 2) + 8 * (i >> 1)],
+                e1 = S.e[1][8 * wn + 2 * (lane & 3) + (i & 1)];
+      const int sc = e0 + e1 - 2 * 1022 - 56;
+      if (sc >= -1022 && sc <= 1023)
+        out[i] = fma((double)t, __hiloint2double((sc + 1023) << 20, 0), out[i]);
+      else if (max(e0, e1) >= kBadExp)
+        out[i] = __hiloint2double(0x7ff80000, 0);
+      else
+        out[i] += scalbn((double)t, sc);
+    }
   }
 #pragma unroll
-  for (int i = 0; i < R; ++i) {
-    const int r = m0 + ty * R + i;
-    if (r >= g.M) continue;
-#pragma unroll
-    for (int j = 0; j < R; ++j) {
-      const int c = n0 + tx * R + j;
-      if (c >= g.N) continue;
-      if (kc > 1) {
-        P[(((long long)z * gridDim.z / kc + b) * g.M + r) * g.N + c] = acc[i][j];
-        continue;
-      }
-      double x = g.alpha * acc[i][j];
-      if (g.beta != 0.0) x += g.beta * C[r * g.ldc + c];
-      if (r == c) x += g.diag;
-      C[r * g.ldc + c] = x;
+  for (int i = 0; i < 4; ++i) {
+    const int r = m0 + 16 * wm + (lane >> 2) + 8 * (i >> 1), c = n0 + 8 * wn + 2 * (lane & 3) + (i & 1);
+    if (r >= g.M || c >= g.N) continue;
+    if (kc > 1) {
+      P[(((long long)z * gridDim.z / kc + b) * g.M + r) * g.N + c] = out[i];
+      continue;
     }
+    double x = g.alpha * out[i];
+    if (g.beta != 0.0) x += g.beta * C[r * g.ldc + c];
+    if (r == c) x += g.diag;
+    C[r * g.ldc + c] = x;
   }
   if (kc == 1) return;
-  // split K: the tile's last CTA to arrive adds the kc chunk sums in order
+  // split K: the tile's last CTA to arrive adds the kc sums in order
   __threadfence();
   __syncthreads();
-  const int tile_id = (b * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+  const int tile_id = b * gridDim.x + blockIdx.x;
   if (tid == 0) s_last = atomicAdd(tcnt + tile_id, 1) == kc - 1;
   __syncthreads();
   if (!s_last) return;
   __threadfence();
   const int batch = gridDim.z / kc;
-  for (int i = tid; i < TILE * TILE; i += 256) {
-    const int r = m0 + i / TILE, c = n0 + i % TILE;
+  for (int i = tid; i < kGT * kGT; i += 256) {
+    const int r = m0 + i / kGT, c = n0 + i % kGT;
     if (r >= g.M || c >= g.N) continue;
     double sum = 0.0;
+#pragma unroll 4
     for (int zz = 0; zz < kc; ++zz)
       sum += __ldcg(P + (((long long)zz * batch + b) * g.M + r) * g.N + c);
     double x = g.alpha * sum;
@@ -526,7 +666,7 @@ inline int nblk(long long n, int t = 256) {
 }
 
 constexpr long long kGemmScratch = 1 << 21;  // split-K doubles (16 MiB)
-constexpr int kGemmTiles = 512;  // K is split only while a call has < 300 tiles
+constexpr int kGemmTiles = 512;  // K is split only while a call has fewer tiles
 
 struct GemmCall {
   cudaStream_t s;
@@ -541,19 +681,16 @@ struct GemmCall {
                   const double* pass = nullptr) const {
     Gemm g{M, N, K, A, lda, sA, tA ? 1 : 0, B, ldb, sB, tB ? 1 : 0, C, ldc, sC,
            alpha, beta, diag, gate, gate_idx, pass};
-    auto ctas = [&](int t) {
-      return (long long)((N + t - 1) / t) * ((M + t - 1) / t) * batch;
-    };
-    const int tile = ctas(64) >= 300 ? 64 : (ctas(32) >= 300 ? 32 : 16);
-    // split K when the output alone gives too few CTAs (chunks of >= 64)
+    const int tm = (M + kGT - 1) / kGT, tn = (N + kGT - 1) / kGT;
+    const long long tiles = (long long)tm * tn * batch;
+    // split K when the output alone gives too few CTAs (two per SM): a CTA
+    // takes ~3 us per chunk whatever its neighbours do
     int kc = 1;
-    while (kc < 64 && ctas(tile) * kc < 300 && K / (2 * kc) >= 64 &&
+    const int chunks = (K + kGK - 1) / kGK;
+    while (tiles <= kGemmTiles && tiles * kc < 300 && 2 * kc <= chunks &&
            (long long)(2 * kc) * batch * M * N <= scratch_len)
       kc *= 2;
-    const dim3 grid((N + tile - 1) / tile, (M + tile - 1) / tile, batch * kc);
-    if (tile == 64) gemm_f64_kernel<64><<<grid, 256, 0, s>>>(g, kc, scratch, tcnt);
-    else if (tile == 32) gemm_f64_kernel<32><<<grid, 256, 0, s>>>(g, kc, scratch, tcnt);
-    else gemm_f64_kernel<16><<<grid, 256, 0, s>>>(g, kc, scratch, tcnt);
+    gemm_digits_kernel<<<dim3(tn * tm, 1, batch * kc), 256, sizeof(GemmSmem), s>>>(g, kc, scratch, tcnt);
   }
 };
 
@@ -864,7 +1001,7 @@ namespace {
 bool calib_config_ok(const optr_calib_config* c) {
   if (!c) return false;
   const bool held = c->T_held > 0;
-  // tokens and query rows: GEMM grids stay within 65535 row tiles
+  // tokens and query rows: launch grids stay within their limits
   const double lim = 4000000.0;
   return c->g >= 1 && c->g <= 64 && c->d_model >= 1 && c->d_model <= (1 << 20) &&
          c->T >= 1 && c->T <= lim && c->nt >= 1 &&
@@ -877,15 +1014,19 @@ bool calib_config_ok(const optr_calib_config* c) {
          c->lr > 0.0 && c->lr < 1e6 && c->lam >= 0.0 && c->lam < 1e12;
 }
 
-void calib_init(Calib& C, const optr_calib_config* c, void* ws, const double* W_O,
+bool calib_init(Calib& C, const optr_calib_config* c, void* ws, const double* W_O,
                 cudaStream_t s) {
   C = Calib{};
+  if (ensure_dynamic_smem(reinterpret_cast<const void*>(&gemm_digits_kernel), sizeof(GemmSmem)) !=
+      cudaSuccess)
+    return false;
   C.c = *c;
   C.windows = c->sink > 0 || c->recent > 0;
   C.scale = 1.0 / sqrt((double)kCD);
   carve(C, static_cast<char*>(ws));
   C.W = W_O;
   C.st = s;
+  return true;
 }
 
 optr_status calib_finish(Calib& C) {
@@ -927,7 +1068,7 @@ extern "C" optr_status optr_calibrate_head(
   if (!workspace || ws_bytes < need || (reinterpret_cast<uintptr_t>(workspace) & 255))
     return OPTR_ERR_WORKSPACE;
   Calib C;
-  calib_init(C, c, workspace, W_O, stream);
+  if (!calib_init(C, c, workspace, W_O, stream)) return OPTR_ERR_CUDA;
   const int n = kCD * kCD;
   if (cudaMemsetAsync(C.err, 0, sizeof(unsigned), stream) != cudaSuccess ||
       cudaMemsetAsync(C.gcnt, 0, sizeof(int) * kGemmTiles, stream) != cudaSuccess)
@@ -971,7 +1112,7 @@ extern "C" optr_status optr_calib_loss_grad(
   if (!workspace || ws_bytes < need || (reinterpret_cast<uintptr_t>(workspace) & 255))
     return OPTR_ERR_WORKSPACE;
   Calib C;
-  calib_init(C, c, workspace, W_O, stream);
+  if (!calib_init(C, c, workspace, W_O, stream)) return OPTR_ERR_CUDA;
   const int n = kCD * kCD;
   if (cudaMemsetAsync(C.err, 0, sizeof(unsigned), stream) != cudaSuccess ||
       cudaMemsetAsync(C.gcnt, 0, sizeof(int) * kGemmTiles, stream) != cudaSuccess)
