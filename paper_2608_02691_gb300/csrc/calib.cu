@@ -21,9 +21,10 @@
 //           dR = dVt^T Zh + V^T (1{inside} (dVt R))
 //   both    dE = R0^T dR, dS = L_exp(S^T, dE), dA = dS - dS^T
 // where L_exp(X, H) is the Frechet derivative of the matrix exponential
-// (the adjoint of L_exp(S, .) is L_exp(S^T, .)).  exp and L_exp come from
-// one Taylor series of the block matrix [[X, H], [0, X]] with scaling and
-// squaring: the upper-right block of its exponential is L_exp(X, H).
+// (the adjoint of L_exp(S, .) is L_exp(S^T, .)); it is taken as
+// dS^T = L_exp(S, dR^T R0).  exp comes from a Taylor polynomial with scaling
+// and squaring, L_exp from the same chain of products differentiated
+// (mat_product_kernel, expm and generator_grad below).
 #include <math.h>
 #include <string.h>
 
@@ -38,12 +39,8 @@ namespace {
 constexpr int kCD = 128;  // head dimension d
 
 // ------------------------------------------------------------------ GEMM
-// C[b] = alpha op(A[b]) op(B[b]) + beta C[b] + diag I, float64, row-major
-// with leading dimensions; op = transpose when tA / tB.  32 x 32 output tiles,
+// C[b] = alpha op(A[b]) op(B[b]) + beta C[b], float64, row-major with leading dimensions; op = transpose when tA / tB.  32 x 32 output tiles,
 // 64-deep k chunks, 256 threads per CTA (gemm_digits_kernel below).
-// gate: when non-null and gate_idx >= *gate, the launch instead copies
-// `pass` into C (or does nothing when pass is null); this lets a fixed
-// number of launches apply a device-decided number of squarings.
 struct Gemm {
   int M, N, K;
   const double* A;
@@ -54,10 +51,7 @@ struct Gemm {
   int tB;
   double* C;
   long long ldc, sC;
-  double alpha, beta, diag;
-  const int* gate;
-  int gate_idx;
-  const double* pass;
+  double alpha, beta;
 };
 
 // The product runs on the fp16 tensor cores, exactly, after a split of both
@@ -132,8 +126,9 @@ __device__ __forceinline__ unsigned long long fixed_point(double x, int e_row) {
   return (unsigned long long)f + 0x80808080808080ull;
 }
 
-// The digits of eight consecutive k of row r (piece kg) into the planes.
-__device__ __forceinline__ void store_digits(__half (*planes)[kGT][kGK], int r, int kg,
+// The digits of eight k of row r (piece kg) into the planes.
+template <int ROWS, int KS>
+__device__ __forceinline__ void store_digits(__half (*planes)[ROWS][KS], int r, int kg,
                                              const double (&x)[8], int e_row) {
   uint32_t h[kDigits][4];
   const __half2 off = __float2half2_rn(1152.f);  // 1024 + byte - 1152 = digit
@@ -170,15 +165,6 @@ __global__ void __launch_bounds__(256, 2) gemm_digits_kernel(Gemm g, int kc, dou
   const int m0 = blockIdx.x / tn * kGT, n0 = blockIdx.x % tn * kGT;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   double* C = g.C + (long long)b * g.sC;
-  if (g.gate != nullptr && g.gate_idx >= *g.gate) {
-    if (g.pass != nullptr && z == 0) {
-      for (int i = tid; i < kGT * kGT; i += 256) {
-        const int r = m0 + i / kGT, c = n0 + i % kGT;
-        if (r < g.M && c < g.N) C[r * g.ldc + c] = g.pass[r * g.ldc + c];
-      }
-    }
-    return;
-  }
   const double* A = g.A + (long long)b * g.sA;
   const double* B = g.B + (long long)b * g.sB;
   // this CTA's K range: part z of kc, in whole chunks
@@ -186,7 +172,8 @@ __global__ void __launch_bounds__(256, 2) gemm_digits_kernel(Gemm g, int kc, dou
   const int kb = (int)((long long)z * nsl / kc) * kGK;
   const int ke = min(g.K, (int)((long long)(z + 1) * nsl / kc) * kGK);
   // loading thread (row, piece) of each operand, rows along the contiguous
-  // dimension of a transposed one
+  // dimension of a transposed one; piece p holds k = p, p + 8, .. p + 56 (both
+  // operands alike), so that a warp reads whole sectors
   const bool a_rows = !g.tA, b_rows = g.tB;  // k contiguous
   const int ra = a_rows ? tid >> 3 : tid & 31, ka = a_rows ? tid & 7 : tid >> 5;
   const int rb = b_rows ? tid >> 3 : tid & 31, kbp = b_rows ? tid & 7 : tid >> 5;
@@ -197,12 +184,12 @@ __global__ void __launch_bounds__(256, 2) gemm_digits_kernel(Gemm g, int kc, dou
     int ea = 1, eb = 1;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const int k = k0 + 8 * ka + i, m = m0 + ra;
+      const int k = k0 + ka + 8 * i, m = m0 + ra;
       xa[i] = m < g.M && k < ke ? (a_rows ? A[m * g.lda + k] : A[k * g.lda + m]) : 0.0;
     }
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const int k = k0 + 8 * kbp + i, n = n0 + rb;
+      const int k = k0 + kbp + 8 * i, n = n0 + rb;
       xb[i] = n < g.N && k < ke ? (b_rows ? B[n * g.ldb + k] : B[k * g.ldb + n]) : 0.0;
     }
 #pragma unroll
@@ -286,7 +273,6 @@ __global__ void __launch_bounds__(256, 2) gemm_digits_kernel(Gemm g, int kc, dou
     }
     double x = g.alpha * out[i];
     if (g.beta != 0.0) x += g.beta * C[r * g.ldc + c];
-    if (r == c) x += g.diag;
     C[r * g.ldc + c] = x;
   }
   if (kc == 1) return;
@@ -308,10 +294,205 @@ __global__ void __launch_bounds__(256, 2) gemm_digits_kernel(Gemm g, int kc, dou
       sum += __ldcg(P + (((long long)zz * batch + b) * g.M + r) * g.N + c);
     double x = g.alpha * sum;
     if (g.beta != 0.0) x += g.beta * C[r * g.ldc + c];
-    if (r == c) x += g.diag;
     C[r * g.ldc + c] = x;
   }
   if (tid == 0) tcnt[tile_id] = 0;
+}
+
+// ------------------------------------------------ 128 x 128 products
+// The generator's exponential and its derivative are chains of 128 x 128
+// products; each launch is one link:
+//   v_h  = f sum_{i < passes} op(A[h][i]) B[h][i],  h = 0, 1 (halves of a CTA)
+//   out0 = v_0 + v_1 + diag I + sum_{j < 4} cy[j] Y[j]            (out[1] null)
+//   out0 = v_0, out1 = v_1, P = diag I + cy[0] Y[0] + cy[1] Y[1]
+//          + cy[2] v_0 + cy[3] v_1                            (out[1] given)
+// with f = 2^-(fs *s), s the device-decided number of squarings.  In digit
+// products as above, over the whole depth of 128 under one exponent (sums below
+// 7 x 128 x 2^14 < 2^24, still exact).
+//
+// What bounds it: the chain, 26 to 32 links per Adam step, so a link's latency
+// (launch, one load, the split, 68 mma per warp, the sum over the four warps
+// that share the depth).  16 x 16 tiles on 64 CTAs of one or two halves (256
+// threads each) take 6.6 us (10 with two products) where the 32 x 32 tiles above,
+// 16 of them in two chunks, take 9.4 us a product.
+constexpr int kMT = 16;
+constexpr int kMaxSquare = 16;  // norms up to 2^15
+
+struct MatOp {
+  const double *A[2][2], *B[2][2];
+  int passes, tA;
+  double* out[2];
+  double* P;
+  const double* Y;  // four consecutive matrices
+  double cy[4], diag;
+  int* s;
+  int gate;   // >= 0: nothing is done when gate >= *s
+  int fs;     // f = 2^-(fs *s)
+  int sel_b;  // B[0][0] is the *s-th of consecutive matrices
+  // first link (A = B = S, unscaled): *s is set here, the smallest with
+  // max(norm) 2^-s <= 1/2, at most s_max, and X = 2^-s S is written
+  const double* norm;
+  int s_max;
+  double* X;
+  unsigned* err;
+};
+
+struct MatHalf {
+  __half d[2][kDigits][kMT][kCD];  // as in GemmSmem, rows of 16 pieces
+  long long part[4][kMT][kMT];     // sums of the four depth slices
+  int emax[kMT][17];
+  int e[2][kMT];
+  double v[kMT][kMT];
+};
+
+template <int H>
+__global__ void __launch_bounds__(256 * H) mat_product_kernel(MatOp o) {
+  extern __shared__ __align__(16) unsigned char gsm_[];
+  __shared__ unsigned long long s_norm[4];
+  const int half = threadIdx.x >> 8, tid = threadIdx.x & 255, warp = tid >> 5, lane = tid & 31;
+  MatHalf& S = reinterpret_cast<MatHalf*>(gsm_)[half];
+  const int m0 = (blockIdx.x >> 3) * kMT, n0 = (blockIdx.x & 7) * kMT;
+  pdl_wait();
+  pdl_trigger();
+  int s = 0;
+  if (o.norm != nullptr) {
+    // non-negative doubles compare as their bits; a NaN is the largest
+    if (threadIdx.x < kCD) {
+      unsigned long long b = __double_as_longlong(__ldcg(o.norm + threadIdx.x));
+#pragma unroll
+      for (int i = 16; i > 0; i >>= 1) {
+        const unsigned long long u = __shfl_xor_sync(0xffffffffu, b, i);
+        b = u > b ? u : b;
+      }
+      if (lane == 0) s_norm[threadIdx.x >> 5] = b;
+    }
+    __syncthreads();
+    unsigned long long b = s_norm[0];
+#pragma unroll
+    for (int i = 1; i < 4; ++i) b = s_norm[i] > b ? s_norm[i] : b;
+    double nrm = __longlong_as_double(b);
+    while (nrm > 0.5 && s < o.s_max) {
+      nrm *= 0.5;
+      ++s;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      if (!(nrm <= 0.5)) atomicOr(o.err, OPTR_DEVERR_CALIB_RANGE);
+      *o.s = s;
+    }
+  } else if (o.s != nullptr) {
+    s = __ldcg(o.s);
+  }
+  if (o.gate >= s && o.gate >= 0) return;
+  const int ra = tid >> 4, ka = tid & 15, rb = tid & 15, kb = tid >> 4;
+  const int wn = warp & 1, ws = warp >> 1;  // 16 x 8 outputs, depth slice of 32
+  const int r = tid >> 4, c = tid & 15;
+  double v = 0.0;
+  for (int ps = 0; ps < o.passes; ++ps) {
+    const double* A = o.A[half][ps];
+    const double* B = o.B[half][ps] + (o.sel_b ? s * kCD * kCD : 0);
+    double xa[8], xb[8];
+    int ea = 1, eb = 1;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int k = ka + 16 * i;  // piece p holds k = p, p + 16, ..
+      xa[i] = __ldcg(o.tA ? A + k * kCD + m0 + ra : A + (m0 + ra) * kCD + k);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) xb[i] = __ldcg(B + (kb + 16 * i) * kCD + n0 + rb);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      ea = max(ea, exponent_of(xa[i]));
+      eb = max(eb, exponent_of(xb[i]));
+    }
+#pragma unroll
+    for (int i = 8; i > 0; i >>= 1) ea = max(ea, __shfl_xor_sync(0xffffffffu, ea, i));
+    S.emax[rb][kb] = eb;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 16; ++i) eb = max(eb, S.emax[rb][i]);
+    store_digits(S.d[0], ra, ka, xa, ea);
+    store_digits(S.d[1], rb, kb, xb, eb);
+    if (ka == 0) S.e[0][ra] = ea;
+    if (kb == 0) S.e[1][rb] = eb;
+    __syncthreads();
+    float acc[kWeights][4];
+#pragma unroll
+    for (int d = 0; d < kWeights; ++d)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[d][i] = 0.f;
+#pragma unroll
+    for (int ks = 0; ks < 2; ++ks) {
+      uint32_t fa[kDigits][4], fb[kDigits + 1][2];
+      {
+        const int rr = lane & 15, p = 4 * ws + 2 * ks + (lane >> 4);
+#pragma unroll
+        for (int i = 0; i < kDigits; ++i) digits_ldsm(fa[i], &S.d[0][i][rr][(p ^ (rr & 7)) * 8]);
+      }
+      {
+        const int rr = 8 * wn + (lane & 7), p = 4 * ws + 2 * ks + ((lane >> 3) & 1);
+#pragma unroll
+        for (int j = 0; j < kDigits; j += 2) {
+          uint32_t x[4];
+          const int jj = min(j + (lane >> 4), kDigits - 1);
+          digits_ldsm(x, &S.d[1][jj][rr][(p ^ (rr & 7)) * 8]);
+          fb[j][0] = x[0];
+          fb[j][1] = x[1];
+          fb[j + 1][0] = x[2];
+          fb[j + 1][1] = x[3];
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < kDigits; ++i)
+#pragma unroll
+        for (int j = 0; j < kDigits; ++j)
+          if (i + j < kWeights) digits_mma(acc[i + j], fa[i], fb[j][0], fb[j][1]);
+    }
+    // unit 2^-43: four slices of at most 32 x 2^12 keep the sum below 2^63
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      int w[kWeights];
+#pragma unroll
+      for (int d = 0; d < kWeights; ++d) w[d] = __float2int_rn(acc[d][i]);
+      S.part[ws][(lane >> 2) + 8 * (i >> 1)][8 * wn + 2 * (lane & 3) + (i & 1)] =
+          ((long long)(w[0] * 256 + w[1]) << 35) + ((long long)(w[2] * 256 + w[3]) << 19) +
+          ((long long)(w[4] * 256 + w[5]) << 3) + ((w[6] * 256 + w[7] + 4096) >> 13);
+    }
+    __syncthreads();
+    const long long t = S.part[0][r][c] + S.part[1][r][c] + S.part[2][r][c] + S.part[3][r][c];
+    const int e0 = S.e[0][r], e1 = S.e[1][c], sc = e0 + e1 - 2 * 1022 - 55 - o.fs * s;
+    if (sc >= -1022 && sc <= 1023)
+      v = fma((double)t, __hiloint2double((sc + 1023) << 20, 0), v);
+    else if (max(e0, e1) >= kBadExp)
+      v = __hiloint2double(0x7ff80000, 0);
+    else
+      v += scalbn((double)t, sc);
+  }
+  const int idx = (m0 + r) * kCD + n0 + c;
+  const double dg = m0 + r == n0 + c ? o.diag : 0.0;
+  if (H == 2) {
+    if (half == 1) S.v[r][c] = v;
+    __syncthreads();
+    if (half == 1) return;
+    const double v1 = reinterpret_cast<MatHalf*>(gsm_)[1].v[r][c];
+    if (o.out[1] != nullptr) {
+      o.out[0][idx] = v;
+      o.out[1][idx] = v1;
+      if (o.P != nullptr)
+        o.P[idx] = dg + (o.cy[0] * __ldcg(o.Y + idx) + (o.cy[1] * __ldcg(o.Y + kCD * kCD + idx) +
+                                                        (o.cy[2] * v + o.cy[3] * v1)));
+      return;
+    }
+    v += v1;
+  }
+  if (o.Y != nullptr) {
+    double y = 0.0;
+#pragma unroll
+    for (int j = 3; j >= 0; --j)
+      if (o.cy[j] != 0.0) y += o.cy[j] * __ldcg(o.Y + j * kCD * kCD + idx);
+    v = (v + y) + dg;
+  }
+  o.out[0][idx] = v;
+  if (o.norm != nullptr) o.X[idx] = ldexp(__ldcg(o.A[0][0] + idx), -s);
 }
 
 // ------------------------------------------------------- small kernels
@@ -333,10 +514,29 @@ __global__ void center_kernel(const double* __restrict__ K,
     Kc[i] = K[i] - mu[i % kCD];
 }
 
-// S = X - X^T (d x d)
-__global__ void skew_kernel(const double* __restrict__ X, double* __restrict__ S) {
+// Sum over a block of 128 threads of v, on thread 0.
+__device__ __forceinline__ double row_sum128(double v) {
+  __shared__ double sh[4];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+  __syncthreads();
+  return (sh[0] + sh[1]) + (sh[2] + sh[3]);
+}
+
+// S = X - X^T (d x d; X the (*s & 1)-th of two when s is given) and, when
+// given, norm[i] = sum_j |S[i][j]|: the largest is both |S|_1 and |S|_inf.
+__global__ void __launch_bounds__(kCD) skew_kernel(const double* X, const int* s, double* S,
+                                                   double* norm) {
   const int i = blockIdx.x, j = threadIdx.x;
-  S[i * kCD + j] = X[i * kCD + j] - X[j * kCD + i];
+  pdl_wait();
+  pdl_trigger();
+  if (s != nullptr) X += (__ldcg(s) & 1) * kCD * kCD;
+  const double v = __ldcg(X + i * kCD + j) - __ldcg(X + j * kCD + i);
+  S[i * kCD + j] = v;
+  if (norm == nullptr) return;
+  const double n = row_sum128(fabs(v));
+  if (j == 0) norm[i] = n;
 }
 
 // normalised Sylvester-Hadamard matrix: (-1)^popcount(i & j) / sqrt(d)
@@ -356,6 +556,12 @@ __global__ void copy_kernel(const double* __restrict__ x, long long n,
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x)
     y[i] = x[i];
+}
+
+__global__ void neg_kernel(const double* __restrict__ x, long long n, double* __restrict__ y) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
+       i += (long long)gridDim.x * blockDim.x)
+    y[i] = -x[i];
 }
 
 // C = A - B
@@ -572,19 +778,32 @@ __global__ void __launch_bounds__(1024) loss_reduce_kernel(const double* __restr
 // Adam (Kingma & Ba), in the order m = b1 m + (1 - b1) g,
 // v = b2 v + ((1 - b2) g) g, x -= (lr mh) / (sqrt(vh) + eps), mh = m / bc1,
 // vh = v / bc2; separate roundings (no contraction).
-__global__ void adam_kernel(double* __restrict__ x, const double* __restrict__ g,
-                            double* __restrict__ m, double* __restrict__ v,
-                            int n, double lr, double b1, double omb1, double b2,
-                            double omb2, double bc1, double bc2, double eps) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const double gi = g[i];
-  const double mi = __dadd_rn(__dmul_rn(b1, m[i]), __dmul_rn(omb1, gi));
-  const double vi = __dadd_rn(__dmul_rn(b2, v[i]), __dmul_rn(__dmul_rn(omb2, gi), gi));
+// The gradient g = dA = L^T - L comes from the derivative buffers L (the
+// (*s & 1)-th of two).  It is skew to the last bit, and so is x when it starts
+// from 0: S = x - x^T = 2 x, written with its row norms for the next rotation.
+// One block per row: at 2 float64 FMAs per clock and SM one SM alone would take
+// 50 us for the norms.
+__global__ void __launch_bounds__(kCD) adam_kernel(double* x, const double* L, const int* s,
+                                                   double* m, double* v, double* S,
+                                                   double* norm, double lr, double b1,
+                                                   double omb1, double b2, double omb2,
+                                                   double bc1, double bc2, double eps) {
+  pdl_wait();
+  pdl_trigger();
+  const int i = blockIdx.x * kCD + threadIdx.x;
+  L += (__ldcg(s) & 1) * kCD * kCD;
+  const double gi = __ldcg(L + threadIdx.x * kCD + blockIdx.x) - __ldcg(L + i);
+  const double mi = __dadd_rn(__dmul_rn(b1, __ldcg(m + i)), __dmul_rn(omb1, gi));
+  const double vi = __dadd_rn(__dmul_rn(b2, __ldcg(v + i)), __dmul_rn(__dmul_rn(omb2, gi), gi));
   m[i] = mi;
   v[i] = vi;
   const double mh = __ddiv_rn(mi, bc1), vh = __ddiv_rn(vi, bc2);
-  x[i] = __dsub_rn(x[i], __ddiv_rn(__dmul_rn(lr, mh), __dadd_rn(__dsqrt_rn(vh), eps)));
+  const double xi = __dsub_rn(
+      __ldcg(x + i), __ddiv_rn(__dmul_rn(lr, mh), __dadd_rn(__dsqrt_rn(vh), eps)));
+  x[i] = xi;
+  S[i] = 2.0 * xi;
+  const double n = row_sum128(fabs(2.0 * xi));
+  if (threadIdx.x == 0) norm[blockIdx.x] = n;
 }
 
 // Held-out selection: keep R when its score is the first or a lower one.
@@ -602,60 +821,11 @@ __global__ void select_kernel(const double* __restrict__ score,
     for (int i = threadIdx.x; i < kCD * kCD; i += blockDim.x) bestR[i] = R[i];
 }
 
-// Scaling for exp: s = smallest integer with max(|S|_1, |S|_inf) 2^-s <= 1/2
-// (at most kMaxSquare), X = sign * S * 2^-s and, when H is given,
-// Hs = H * 2^-s (the block matrix [[X, H], [0, X]] is scaled as a whole).
-constexpr int kMaxSquare = 16;  // norms up to 2^15
-__global__ void expm_prep_kernel(const double* __restrict__ S, double sign,
-                                 const double* __restrict__ H,
-                                 double* __restrict__ Xs, double* __restrict__ Hs,
-                                 int* __restrict__ s_out, unsigned* err) {
-  __shared__ double red[kCD];
-  __shared__ int s_sh;
-  const int i = threadIdx.x;  // 128 threads
-  double rs = 0.0, cs = 0.0;
-  for (int j = 0; j < kCD; ++j) {
-    rs += fabs(S[i * kCD + j]);
-    cs += fabs(S[j * kCD + i]);
-  }
-  red[i] = fmax(rs, cs);
-  __syncthreads();
-  for (int w = kCD / 2; w > 0; w >>= 1) {
-    if (i < w) red[i] = fmax(red[i], red[i + w]);
-    __syncthreads();
-  }
-  if (i == 0) {
-    int s = 0;
-    double nrm = red[0];
-    while (nrm > 0.5 && s < kMaxSquare) {
-      nrm *= 0.5;
-      ++s;
-    }
-    if (nrm > 0.5 || !(red[0] == red[0])) atomicOr(err, OPTR_DEVERR_CALIB_RANGE);
-    s_sh = s;
-    *s_out = s;
-  }
-  __syncthreads();
-  const double f = sign * ldexp(1.0, -s_sh);
-  for (int j = 0; j < kCD; ++j) {
-    Xs[i * kCD + j] = f * S[i * kCD + j];
-    if (H != nullptr) Hs[i * kCD + j] = ldexp(H[i * kCD + j], -s_sh);
-  }
-}
-
 }  // namespace
 
 // ------------------------------------------------------------ host side
 
 namespace {
-
-constexpr int kTaylor = 18;        // Taylor degree of exp on ||X|| <= 1/2
-constexpr int kSquareLaunches = kMaxSquare;  // one gated launch per possible squaring
-
-__global__ void eye_kernel(double* __restrict__ X) {
-  const int i = blockIdx.x, j = threadIdx.x;
-  X[i * kCD + j] = i == j ? 1.0 : 0.0;
-}
 
 // blocks of 256 threads for one warp per row (no grid-stride loop)
 inline int nwarp_blocks(long long rows) { return (int)((rows * 32 + 255) / 256); }
@@ -676,11 +846,9 @@ struct GemmCall {
   void operator()(int M, int N, int K, const double* A, long long lda, bool tA,
                   const double* B, long long ldb, bool tB, double* C, long long ldc,
                   double alpha = 1.0, double beta = 0.0, int batch = 1,
-                  long long sA = 0, long long sB = 0, long long sC = 0,
-                  double diag = 0.0, const int* gate = nullptr, int gate_idx = 0,
-                  const double* pass = nullptr) const {
+                  long long sA = 0, long long sB = 0, long long sC = 0) const {
     Gemm g{M, N, K, A, lda, sA, tA ? 1 : 0, B, ldb, sB, tB ? 1 : 0, C, ldc, sC,
-           alpha, beta, diag, gate, gate_idx, pass};
+           alpha, beta};
     const int tm = (M + kGT - 1) / kGT, tn = (N + kGT - 1) / kGT;
     const long long tiles = (long long)tm * tn * batch;
     // split K when the output alone gives too few CTAs (two per SM): a CTA
@@ -713,12 +881,18 @@ struct Calib {
   Trace tr[2];   // calibration, held-out
   // working buffers (sized for the larger trace)
   double *Z, *Zh, *inside, *Kt, *dKt, *dZh;  // [T][d]
-  double *L, *PK, *GV;                       // [g][nt][T]
+  double *X, *PK, *GV;                       // [g][nt][T]
   double *rowv;                              // [g][nt]
   double *DV, *U;                            // [g][nt][d]
-  double *E;                                 // [g][nt][d_model]
+  double *Eo;                                // [g][nt][d_model]
   // d x d
-  double *R0[2], *A, *m, *v, *dA, *S, *Xs, *Hs, *T1[2], *T2[2], *R, *dR, *dE, *best;
+  double *R0[2], *A, *m, *v, *dA, *S, *R, *dR, *best;
+  double *Y, *dY;        // powers X .. X^4 of the scaled generator, and derivatives
+  double *P, *dP[2];     // P3, P2, P1 of the polynomial; derivatives
+  double *F;             // exp(X)^(2^i) - I, i = 0 .. kMaxSquare
+  double *L;             // derivative of F[i], two buffers, i & 1
+  double *norm;          // row norms of S
+  int squares;           // squarings launched: a bound on *s_dev
   double* scal;  // [0] training loss scratch, [1] score, [2] best score
   int* s_dev;
   unsigned* err;
@@ -766,72 +940,171 @@ size_t carve(Calib& C, char* base) {
   C.Kt = L.take<double>(Tm * D);
   C.dKt = L.take<double>(Tm * D);
   C.dZh = L.take<double>(Tm * D);
-  C.L = L.take<double>(g * nm * Tm);
+  C.X = L.take<double>(g * nm * Tm);
   C.PK = L.take<double>(g * nm * Tm);
   C.GV = L.take<double>(g * nm * Tm);
   C.rowv = L.take<double>(g * nm);
   C.DV = L.take<double>(g * nm * D);
   C.U = L.take<double>(g * nm * D);
-  C.E = L.take<double>(g * nm * c.d_model);
+  C.Eo = L.take<double>(g * nm * c.d_model);
   C.gsc = L.take<double>(kGemmScratch);
   C.gcnt = L.take<int>(kGemmTiles);
-  double** dd[] = {&C.R0[0], &C.R0[1], &C.A, &C.m, &C.v, &C.dA, &C.S, &C.Xs,
-                   &C.Hs, &C.T1[0], &C.T1[1], &C.T2[0], &C.T2[1], &C.R, &C.dR,
-                   &C.dE, &C.best};
+  double** dd[] = {&C.R0[0], &C.R0[1], &C.A, &C.m, &C.v, &C.dA, &C.S, &C.R, &C.dR, &C.best,
+                   &C.dP[0], &C.dP[1]};
   for (double** p : dd) *p = L.take<double>(D2);
+  C.Y = L.take<double>(4 * D2);
+  C.dY = L.take<double>(4 * D2);
+  C.P = L.take<double>(3 * D2);
+  C.F = L.take<double>((kMaxSquare + 1) * D2);
+  C.L = L.take<double>(2 * D2);
+  C.norm = L.take<double>(kCD);
   return L.off;
 }
 
-// E = exp(sign * S) into T1[*], and with H, L = L_exp(sign * S, H) into
-// T2[*]; returns the buffer index holding the results.  Taylor series of
-// the block matrix [[X, H], [0, X]] in Horner form (T1 <- I + X T1 / k,
-// T2 <- (X T2 + H T1) / k), X = sign S 2^-s, H scaled alike, then s
-// squarings ([[E, L], [0, E]]^2 = [[E E, E L + L E], [0, E E]]), s decided
-// on the device.
-int expm(Calib& C, const double* S, double sign, const double* H) {
-  GemmCall gm = C.gemm();
-  expm_prep_kernel<<<1, kCD, 0, C.st>>>(S, sign, H, C.Xs, C.Hs, C.s_dev, C.err);
-  int cur = 0;
-  eye_kernel<<<kCD, kCD, 0, C.st>>>(C.T1[0]);
-  if (H) fill_kernel<<<nblk(kCD * kCD), 256, 0, C.st>>>(C.T2[0], kCD * kCD, 0.0);
-  for (int k = kTaylor; k >= 1; --k) {
-    const int nx = cur ^ 1;
-    const double a = 1.0 / (double)k;
-    gm(kCD, kCD, kCD, C.Xs, kCD, false, C.T1[cur], kCD, false, C.T1[nx], kCD, a, 0.0,
-       1, 0, 0, 0, 1.0);
-    if (H) {
-      gm(kCD, kCD, kCD, C.Xs, kCD, false, C.T2[cur], kCD, false, C.T2[nx], kCD, a, 0.0);
-      gm(kCD, kCD, kCD, C.Hs, kCD, false, C.T1[cur], kCD, false, C.T2[nx], kCD, a, 1.0);
-    }
-    cur = nx;
-  }
-  for (int i = 0; i < kSquareLaunches; ++i) {
-    const int nx = cur ^ 1;
-    gm(kCD, kCD, kCD, C.T1[cur], kCD, false, C.T1[cur], kCD, false, C.T1[nx], kCD,
-       1.0, 0.0, 1, 0, 0, 0, 0.0, C.s_dev, i, C.T1[cur]);
-    if (H) {
-      gm(kCD, kCD, kCD, C.T1[cur], kCD, false, C.T2[cur], kCD, false, C.T2[nx], kCD,
-         1.0, 0.0, 1, 0, 0, 0, 0.0, C.s_dev, i, C.T2[cur]);
-      gm(kCD, kCD, kCD, C.T2[cur], kCD, false, C.T1[cur], kCD, false, C.T2[nx], kCD,
-         1.0, 1.0, 1, 0, 0, 0, 0.0, C.s_dev, i, nullptr);
-    }
-    cur = nx;
-  }
-  return cur;
+// One link of the 128 x 128 chain on C.st.
+void link(Calib& C, int halves, const MatOp& o) {
+  auto k = halves == 2 ? &mat_product_kernel<2> : &mat_product_kernel<1>;
+  launch_pdl(k, dim3(64), dim3(256 * halves), halves * sizeof(MatHalf), C.st, o);
+}
+MatOp product(const double* A, const double* B, double* out) {
+  MatOp o{};
+  o.A[0][0] = A;
+  o.B[0][0] = B;
+  o.passes = 1;
+  o.out[0] = out;
+  o.gate = -1;
+  return o;
+}
+MatOp& plus(MatOp& o, const double* A, const double* B) {
+  o.A[1][0] = A;
+  o.B[1][0] = B;
+  return o;
 }
 
-// R = R0 exp(A - A^T) into C.R (S = A - A^T kept in C.S)
+constexpr int kD2 = kCD * kCD;
+
+// 1 / k!
+double inv_fact(int k) {
+  double f = 1.0;
+  for (int i = 2; i <= k; ++i) f *= i;
+  return 1.0 / f;
+}
+void taylor(MatOp& o, const double* Y, int k0, int n, bool constant) {
+  o.Y = Y;
+  o.diag = constant ? inv_fact(k0) : 0.0;
+  for (int j = 0; j < 4; ++j) o.cy[j] = j < n ? inv_fact(k0 + 1 + j) : 0.0;
+}
+
+// I + F[s] = exp(S) with X = S 2^-s, |X| <= 1/2: the Taylor polynomial of degree
+// 16 (remainder 2e-20) in Paterson and Stockmeyer's form ("On the number of
+// nonscalar multiplications necessary to evaluate polynomials", 1973),
+//   P3 = sum_{j <= 4} X^j / (12 + j)!,  P_i = X^4 P_{i+1} + sum_{j < 4} X^j / (4 i + j)!,
+// F[0] = P0 - I, then s squarings (I + F)^2 = I + (2 F + F^2); 5 dependent links
+// and the squarings, where Horner's rule has 18.  F rather than I + F is kept
+// because each squaring doubles the relative error, and entries of F round at
+// their own size, not at 1: the gradient's relative error against quad precision
+// is 1e-15 to 6e-15 for entries of A of 0.005 to 0.4 (FMA chain, Horner:
+// 3e-15 to 9e-14; this chain with I + F: 2e-15 to 2e-13).
+// 20 + 20 Adam steps 86.5 -> 27.5 ms (Horner and one launch per product before).
+// C.squares squarings are launched, those past s do nothing.  The powers, P_i
+// and F[i] stay for generator_grad.
+void expm(Calib& C) {
+  MatOp o = product(C.S, C.S, C.Y + kD2);
+  o.s = C.s_dev;
+  o.fs = 2;
+  o.norm = C.norm;
+  o.s_max = C.squares;
+  o.X = C.Y;
+  o.err = C.err;
+  link(C, 1, o);
+  o = product(C.Y, C.Y + kD2, C.Y + 2 * kD2);
+  plus(o, C.Y + kD2, C.Y + kD2);
+  o.out[1] = C.Y + 3 * kD2;
+  o.P = C.P;
+  taylor(o, C.Y, 12, 4, true);
+  link(C, 2, o);
+  for (int i = 2; i >= 0; --i) {
+    o = product(C.Y + 3 * kD2, C.P + (2 - i) * kD2, i ? C.P + (3 - i) * kD2 : C.F);
+    taylor(o, C.Y, 4 * i, 3, i > 0);
+    link(C, 1, o);
+  }
+  for (int i = 0; i < C.squares; ++i) {
+    o = product(C.F + i * kD2, C.F + i * kD2, C.F + (i + 1) * kD2);
+    o.Y = C.F + i * kD2;
+    o.cy[0] = 2.0;
+    o.s = C.s_dev;
+    o.gate = i;
+    link(C, 1, o);
+  }
+}
+
+// R = R0 exp(S) into C.R, S = A - A^T and its row norms given
 void rotation(Calib& C, const double* R0) {
-  skew_kernel<<<kCD, kCD, 0, C.st>>>(C.A, C.S);
-  const int e = expm(C, C.S, 1.0, nullptr);
-  C.gemm()(kCD, kCD, kCD, R0, kCD, false, C.T1[e], kCD, false, C.R, kCD);
+  expm(C);
+  MatOp o = product(R0, C.F, C.R);  // R0 + R0 F
+  o.Y = R0;
+  o.cy[0] = 1.0;
+  o.s = C.s_dev;
+  o.sel_b = 1;
+  link(C, 1, o);
 }
 
-// dA = dS - dS^T with dS = L_exp(S^T, R0^T dR) (S^T = -S)
+// dS^T = L_exp(S, dR^T R0) into C.L[*s & 1] (dA = dS - dS^T): the chain of
+// expm() differentiated, two products per link.
 void generator_grad(Calib& C, const double* R0) {
-  C.gemm()(kCD, kCD, kCD, R0, kCD, true, C.dR, kCD, false, C.dE, kCD);
-  const int e = expm(C, C.S, -1.0, C.dE);
-  skew_kernel<<<kCD, kCD, 0, C.st>>>(C.T2[e], C.dA);
+  MatOp o = product(C.dR, R0, C.dY);  // H = 2^-s dR^T R0
+  o.tA = 1;
+  o.s = C.s_dev;
+  o.fs = 1;
+  link(C, 1, o);
+  o = product(C.dY, C.Y, C.dY + kD2);  // d(X^2) = H X + X H
+  link(C, 2, plus(o, C.Y, C.dY));
+  o = product(C.dY, C.Y + kD2, C.dY + 2 * kD2);  // d(X^3) = H X^2 + X d(X^2)
+  plus(o, C.dY + kD2, C.Y + kD2);                // d(X^4) = d(X^2) X^2 + X^2 d(X^2)
+  o.passes = 2;
+  o.A[0][1] = C.Y;
+  o.B[0][1] = C.dY + kD2;
+  o.A[1][1] = C.Y + kD2;
+  o.B[1][1] = C.dY + kD2;
+  o.out[1] = C.dY + 3 * kD2;
+  o.P = C.dP[0];
+  taylor(o, C.dY, 12, 4, false);
+  link(C, 2, o);
+  for (int i = 2; i >= 0; --i) {  // dP_i = d(X^4) P_{i+1} + X^4 dP_{i+1} + ..
+    o = product(C.dY + 3 * kD2, C.P + (2 - i) * kD2, i ? C.dP[(i + 1) & 1] : C.L);
+    plus(o, C.Y + 3 * kD2, C.dP[i & 1]);
+    taylor(o, C.dY, 4 * i, 3, false);
+    link(C, 2, o);
+  }
+  for (int i = 0; i < C.squares; ++i) {
+    double *L0 = C.L + (i & 1) * kD2, *L1 = C.L + ((i + 1) & 1) * kD2;
+    o = product(C.F + i * kD2, L0, L1);  // 2 L + F L + L F
+    plus(o, L0, C.F + i * kD2);
+    o.Y = L0;
+    o.cy[0] = 2.0;
+    o.s = C.s_dev;
+    o.gate = i;
+    link(C, 2, o);
+  }
+}
+
+// Squarings that t Adam steps from A = 0 can need.  A step moves an entry by
+// at most lr |mh| / sqrt(vh), and by Cauchy and Schwarz
+//   mh^2 <= vh (1-b1)^2 / (1-b2) (bc2 / bc1^2) sum_{j < t} (b1^2 / b2)^j;
+// a row of S = 2 A has 127 entries.
+int adam_squares(double reach) {
+  double n = 2.0 * (kCD - 1) * reach * (1.0 + 1e-6);
+  int s = 0;
+  while (n > 0.5 && s < kMaxSquare) {
+    n *= 0.5;
+    ++s;
+  }
+  return s;
+}
+double adam_reach(double lr, double b1, double b2, int t) {
+  const double q = b1 * b1 / b2;
+  const double bc1 = 1.0 - pow(b1, (double)t), bc2 = 1.0 - pow(b2, (double)t);
+  return lr * (1.0 - b1) / bc1 * sqrt(bc2 / (1.0 - b2) * (1.0 - pow(q, (double)t)) / (1.0 - q));
 }
 
 }  // namespace
@@ -845,11 +1118,11 @@ void trace_setup(Calib& C, Trace& t, const double* mu) {
   const int g = C.c.g, D = kCD;
   const long long nT = (long long)t.T * D, r = (long long)g * t.nt;
   center_kernel<<<nblk(nT), 256, 0, C.st>>>(t.K, mu, nT, t.Kc);
-  // raw BF16 logits q_j K^T into L, softmax into Pref
-  gm(t.nt, t.T, D, t.q, (long long)g * D, false, t.K, D, true, C.L, t.T, 1.0, 0.0,
+  // raw BF16 logits q_j K^T into X, softmax into Pref
+  gm(t.nt, t.T, D, t.q, (long long)g * D, false, t.K, D, true, C.X, t.T, 1.0, 0.0,
      g, D, 0, (long long)t.nt * t.T);
   softmax_rows_kernel<<<(unsigned)r, 256, 0, C.st>>>(
-      C.L, nullptr, (int)r, t.nt, t.T, t.tpos, C.scale, 0, 0, t.Pref, nullptr,
+      C.X, nullptr, (int)r, t.nt, t.T, t.tpos, C.scale, 0, 0, t.Pref, nullptr,
       nullptr, nullptr);
   logclamp_kernel<<<nblk(r * t.T), 256, 0, C.st>>>(t.Pref, r * t.T, t.logPref);
   if (C.windows)
@@ -866,24 +1139,24 @@ void q2_roundtrip(Calib& C, const double* X, int T, double clip) {
   gm(T, kCD, kCD, C.Zh, kCD, false, C.R, kCD, true, C.Kt, kCD);
 }
 
-// L_K of trace t under C.R into *out; leaves PK, E for the backward.
+// L_K of trace t under C.R into *out; leaves PK, Eo for the backward.
 void key_forward(Calib& C, Trace& t, double* out) {
   GemmCall gm = C.gemm();
   const int g = C.c.g, D = kCD, dm = C.c.d_model;
   const long long r = (long long)g * t.nt, nTT = (long long)t.nt * t.T;
   q2_roundtrip(C, t.Kc, t.T, C.c.clip_k);
-  gm(t.nt, t.T, D, t.q, (long long)g * D, false, C.Kt, D, true, C.L, t.T, 1.0, 0.0,
+  gm(t.nt, t.T, D, t.q, (long long)g * D, false, C.Kt, D, true, C.X, t.T, 1.0, 0.0,
      g, D, 0, nTT);
   softmax_rows_kernel<<<(unsigned)r, 256, 0, C.st>>>(
-      C.L, C.windows ? t.Lc : nullptr, (int)r, t.nt, t.T, t.tpos, C.scale,
+      C.X, C.windows ? t.Lc : nullptr, (int)r, t.nt, t.T, t.tpos, C.scale,
       C.c.sink, C.c.recent, C.PK, t.Pref, t.logPref, C.rowv);
   // e_j = ((pk - p) V) W_j^T
   sub_kernel<<<nblk(r * t.T), 256, 0, C.st>>>(C.PK, t.Pref, r * t.T, C.GV);
   gm(t.nt, D, t.T, C.GV, t.T, false, t.V, D, false, C.DV, D, 1.0, 0.0, g, nTT, 0,
      (long long)t.nt * D);
-  gm(t.nt, dm, D, C.DV, D, false, C.W, D, true, C.E, dm, 1.0, 0.0, g,
+  gm(t.nt, dm, D, C.DV, D, false, C.W, D, true, C.Eo, dm, 1.0, 0.0, g,
      (long long)t.nt * D, (long long)dm * D, (long long)t.nt * dm);
-  row_sqsum_kernel<<<nwarp_blocks(r), 256, 0, C.st>>>(C.E, (int)r, dm, C.c.lam, 1, C.rowv);
+  row_sqsum_kernel<<<nwarp_blocks(r), 256, 0, C.st>>>(C.Eo, (int)r, dm, C.c.lam, 1, C.rowv);
   loss_reduce_kernel<<<1, 1024, 0, C.st>>>(C.rowv, (int)r, (double)r, out);
 }
 
@@ -897,7 +1170,7 @@ void key_backward(Calib& C, Trace& t) {
   const int g = C.c.g, D = kCD, dm = C.c.d_model;
   const long long r = (long long)g * t.nt, nTT = (long long)t.nt * t.T;
   // U_j = (2 lambda / d_model) e_j W_j;  GV_j = U_j V^T
-  gm(t.nt, D, dm, C.E, dm, false, C.W, D, false, C.U, D, 2.0 * C.c.lam / dm, 0.0, g,
+  gm(t.nt, D, dm, C.Eo, dm, false, C.W, D, false, C.U, D, 2.0 * C.c.lam / dm, 0.0, g,
      (long long)t.nt * dm, (long long)dm * D, (long long)t.nt * D);
   gm(t.nt, t.T, D, C.U, D, false, t.V, D, true, C.GV, t.T, 1.0, 0.0, g,
      (long long)t.nt * D, 0, nTT);
@@ -937,9 +1210,9 @@ void value_forward(Calib& C, Trace& t, double* out) {
                                                         C.Kt);
   gm(t.nt, D, t.T, t.Phat, t.T, false, C.Kt, D, false, C.DV, D, 1.0, 0.0, g, nTT, 0,
      (long long)t.nt * D);
-  gm(t.nt, dm, D, C.DV, D, false, C.W, D, true, C.E, dm, 1.0, 0.0, g,
+  gm(t.nt, dm, D, C.DV, D, false, C.W, D, true, C.Eo, dm, 1.0, 0.0, g,
      (long long)t.nt * D, (long long)dm * D, (long long)t.nt * dm);
-  row_sqsum_kernel<<<nwarp_blocks(r), 256, 0, C.st>>>(C.E, (int)r, dm, 1.0, 0, C.rowv);
+  row_sqsum_kernel<<<nwarp_blocks(r), 256, 0, C.st>>>(C.Eo, (int)r, dm, 1.0, 0, C.rowv);
   loss_reduce_kernel<<<1, 1024, 0, C.st>>>(C.rowv, (int)r, (double)r, out);
 }
 
@@ -948,7 +1221,7 @@ void value_backward(Calib& C, Trace& t) {
   GemmCall gm = C.gemm();
   const int g = C.c.g, D = kCD, dm = C.c.d_model;
   const long long r = (long long)g * t.nt, nTT = (long long)t.nt * t.T;
-  gm(t.nt, D, dm, C.E, dm, false, C.W, D, false, C.U, D, 2.0 / ((double)dm * r), 0.0,
+  gm(t.nt, D, dm, C.Eo, dm, false, C.W, D, false, C.U, D, 2.0 / ((double)dm * r), 0.0,
      g, (long long)t.nt * dm, (long long)dm * D, (long long)t.nt * D);
   for (int j = 0; j < g; ++j)
     gm(t.T, D, t.nt, t.Phat + j * nTT, t.T, true, C.U + (long long)j * t.nt * D, D,
@@ -970,8 +1243,11 @@ void adam_run(Calib& C, int kind, const double* R0, double* hist) {
   fill_kernel<<<nblk(n), 256, 0, C.st>>>(C.A, n, 0.0);
   fill_kernel<<<nblk(n), 256, 0, C.st>>>(C.m, n, 0.0);
   fill_kernel<<<nblk(n), 256, 0, C.st>>>(C.v, n, 0.0);
+  skew_kernel<<<kCD, kCD, 0, C.st>>>(C.A, nullptr, C.S, C.norm);
   const double b1 = 0.9, b2 = 0.999, eps = 1e-8;
+  double reach = 0.0;  // bound on |A| after i steps
   for (int i = 0; i <= c.steps; ++i) {
+    C.squares = adam_squares(reach);
     rotation(C, R0);
     if (i % c.select_every == 0 || i == c.steps) {
       if (kind == 0) key_forward(C, C.tr[1], C.scal + 1);
@@ -988,9 +1264,10 @@ void adam_run(Calib& C, int kind, const double* R0, double* hist) {
     }
     generator_grad(C, R0);
     const int t = i + 1;
-    adam_kernel<<<nblk(n), 256, 0, C.st>>>(C.A, C.dA, C.m, C.v, n, c.lr, b1, 1.0 - b1,
-                                           b2, 1.0 - b2, 1.0 - pow(b1, (double)t),
-                                           1.0 - pow(b2, (double)t), eps);
+    launch_pdl(&adam_kernel, dim3(kCD), dim3(kCD), 0, C.st, C.A, C.L, C.s_dev, C.m, C.v, C.S,
+               C.norm, c.lr, b1, 1.0 - b1, b2, 1.0 - b2, 1.0 - pow(b1, (double)t),
+               1.0 - pow(b2, (double)t), eps);
+    reach += adam_reach(c.lr, b1, b2, t);
   }
 }
 
@@ -1017,9 +1294,14 @@ bool calib_config_ok(const optr_calib_config* c) {
 bool calib_init(Calib& C, const optr_calib_config* c, void* ws, const double* W_O,
                 cudaStream_t s) {
   C = Calib{};
-  if (ensure_dynamic_smem(reinterpret_cast<const void*>(&gemm_digits_kernel), sizeof(GemmSmem)) !=
-      cudaSuccess)
-    return false;
+  const struct {
+    const void* kernel;
+    size_t bytes;
+  } need[] = {{reinterpret_cast<const void*>(&gemm_digits_kernel), sizeof(GemmSmem)},
+              {reinterpret_cast<const void*>(&mat_product_kernel<1>), sizeof(MatHalf)},
+              {reinterpret_cast<const void*>(&mat_product_kernel<2>), 2 * sizeof(MatHalf)}};
+  for (const auto& k : need)
+    if (ensure_dynamic_smem(k.kernel, k.bytes) != cudaSuccess) return false;
   C.c = *c;
   C.windows = c->sink > 0 || c->recent > 0;
   C.scale = 1.0 / sqrt((double)kCD);
@@ -1125,6 +1407,8 @@ extern "C" optr_status optr_calib_loss_grad(
     value_setup(C, C.tr[0]);
   }
   copy_kernel<<<nblk(n), 256, 0, stream>>>(A, n, C.A);
+  skew_kernel<<<kCD, kCD, 0, stream>>>(C.A, nullptr, C.S, C.norm);
+  C.squares = kMaxSquare;
   rotation(C, R0);
   if (which == 0) key_forward(C, C.tr[0], loss);
   else value_forward(C, C.tr[0], loss);
@@ -1132,7 +1416,9 @@ extern "C" optr_status optr_calib_loss_grad(
     if (which == 0) key_backward(C, C.tr[0]);
     else value_backward(C, C.tr[0]);
     generator_grad(C, R0);
-    copy_kernel<<<nblk(n), 256, 0, stream>>>(C.dA, n, dA);
+    // dA = L^T - L
+    skew_kernel<<<kCD, kCD, 0, stream>>>(C.L, C.s_dev, C.dA, nullptr);
+    neg_kernel<<<nblk(n), 256, 0, stream>>>(C.dA, n, dA);
   }
   return calib_finish(C);
 }
