@@ -39,8 +39,8 @@ namespace {
 constexpr int kCD = 128;  // head dimension d
 
 // ------------------------------------------------------------------ GEMM
-// C[b] = alpha op(A[b]) op(B[b]) + beta C[b], float64, row-major with leading dimensions; op = transpose when tA / tB.  32 x 32 output tiles,
-// 64-deep k chunks, 256 threads per CTA (gemm_digits_kernel below).
+// C[b] = alpha op(A[b]) op(B[b]), float64, row-major with leading dimensions;
+// op = transpose when tA / tB (gemm_digits_kernel below).
 struct Gemm {
   int M, N, K;
   const double* A;
@@ -51,46 +51,57 @@ struct Gemm {
   int tB;
   double* C;
   long long ldc, sC;
-  double alpha, beta;
+  double alpha;
+  // depth continued with a second pair of the same shape and layout (null: no)
+  const double *A2, *B2;
+  const double* mul;  // C = mul .* (..) when given, row-major with ldc
+  const double* sub;  // C = .. - sub when given, likewise
 };
 
 // The product runs on the fp16 tensor cores, exactly, after a split of both
 // factors into small integers (the scheme of Ozaki, Ogita, Oishi and Rump,
 // "Error-free transformations of matrix multiplication", 2012): this GPU does
 // 2 float64 FMAs per clock and SM, three orders of magnitude below its tensor
-// cores.  Per k chunk of 64, a row of A (a column of B) is written as
+// cores.  Per k chunk of 128, a row of A (a column of B) is written as
 // fixed-point numbers under its own largest exponent, 54 bits and sign, in
 // seven balanced base-256 digits d_0 .. d_6 (|d_0| <= 64, else |d| <= 128),
 // which are exact fp16 values.  All digit products of one weight d = i + j are
-// summed in one float32 accumulator: at most 7 x 64 x 2^14 < 2^24, so every sum
-// is exact.  The weights 0 .. 7 (34 of the 49 products; what is left out of
+// summed in one float32 accumulator: at most 7 x 128 x 2^14 < 2^24, so every
+// sum is exact.  The weights 0 .. 7 (34 of the 49 products; what is left out of
 // one product is below 2^-59 of the largest one) are put together in 64-bit
-// integers and added to the float64 result, one rounding per 64 products.  Against sums in
+// integers and added to the float64 result, one rounding per 128 products.  Against sums in
 // extended precision that is 2 to 5 times closer than a float64 FMA chain
 // (relative error 1.5e-16 to 2.8e-16 on keys x rotation, probabilities x
 // values, powers of the generator; FMA chain 2.8e-16 to 1.5e-15).
 // A row or column with a NaN or an infinity gives NaN throughout.
-// What bounds it: 136 mma per warp and chunk (16 x 8 outputs each, a third of
-// the CTA's 3 us), the split of both tiles and the chunk's load latency; 32 x 32
-// tiles give the calibration's products (128 to 2048 rows) enough CTAs.  One
-// 64-query, 4096-channel, 2048-token key step spent 1.8 ms in the float64 kernel
-// this replaces; 20 + 20 steps of both phases 120.3 -> 86.5 ms.
+// What bounds it: per CTA and chunk 272 mma a warp (4.4 us at one m16n8k16 per 8
+// cycles and SM quarter), the split of both tiles (24 values a thread, ~45
+// integer instructions each, 2.5 us) and the load's latency, one after the
+// other, as 172 KB of digits leave room for one CTA per SM.  64 x 32 tiles make
+// the calibration's products (2048 or 4 x 64 rows, 128 columns or the reverse)
+// one wave of 128 CTAs: 2048 x 128 x 128 takes 19 us from cold caches, 25 with
+// 32 x 32 tiles in two waves, 21 with 64-deep chunks and two CTAs per SM.
+// Products with fewer than half as many tiles and chunks as SMs take 32 x 16
+// tiles (8 steps on 256 tokens: 4.4 ms, 5.0 with 64 x 32 throughout).
 //
 // With kc > 1 CTA z of a product covers the z-th part of k and writes its sum
 // to P[z][b]; the last of the tile's kc CTAs to finish (a per-tile arrival
 // counter, left at 0 again) adds the parts in a fixed order, z = 0 .. kc-1,
 // so the result does not depend on which CTA that is.
-constexpr int kGT = 32;      // tile
-constexpr int kGK = 64;      // k chunk
+constexpr int kGK = 128;     // k chunk
 constexpr int kDigits = 7;
 constexpr int kWeights = 8;
 constexpr int kBadExp = 1 << 20;  // exponent of a row with a non-finite value
 
-struct GemmSmem {
-  // digit planes [operand][digit][row][k]; 16-byte piece p of row r at p ^ (r % 8)
-  __half d[2][kDigits][kGT][kGK];
-  int emax[2][kGT][9];  // largest exponents of a row's eight 8-element parts
-  int e[2][kGT];
+// MT x NT outputs, one warp per 16 x 8 of them
+template <int MT, int NT>
+struct GemmTile {
+  static constexpr int kThreads = MT / 16 * (NT / 8) * 32;
+  // digit planes [digit][row][k]; 16-byte piece p of row r at p ^ (r % 8)
+  __half a[kDigits][MT][kGK];
+  __half b[kDigits][NT][kGK];
+  int emax[MT + NT][17];  // largest exponents of a row's sixteen 8-element pieces
+  int e[MT + NT];
 };
 
 __device__ __forceinline__ void digits_mma(float (&d)[4], const uint32_t (&a)[4], uint32_t b0,
@@ -107,16 +118,18 @@ __device__ __forceinline__ void digits_ldsm(uint32_t (&r)[4], const void* p) {
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(s));
 }
 
-// Exponent e of |x| = m 2^(e - 1075), m < 2^53 (subnormals share e = 1).
-__device__ __forceinline__ int exponent_of(double x) {
-  const int e = (__double2hiint(x) >> 20) & 2047;
-  return e == 2047 ? kBadExp : max(e, 1);
+// |x| = m 2^(e - 1075), m < 2^53, e = max(biased exponent, 1).  The largest
+// exponent of a row: the maximum over its values of field(x), then row_exponent.
+__device__ __forceinline__ int field(double x) { return __double2hiint(x) & 0x7ff00000; }
+__device__ __forceinline__ int row_exponent(int f) {
+  return f == 0x7ff00000 ? kBadExp : max(f >> 20, 1);
 }
 
-// x as a fixed-point integer with unit 2^(e_row - 1076), |result| <= 2^54, plus
-// the bias that makes its bytes digit + 128.
-__device__ __forceinline__ unsigned long long fixed_point(double x, int e_row) {
+// x as a fixed-point integer with unit 2^(e_row - 1076), rounded, |result| <=
+// 2^54, plus the bias that makes its bytes digit + 128.
+__device__ __noinline__ unsigned long long fixed_point_small(double x, int e_row) {
   const unsigned long long bits = __double_as_longlong(x);
+  if (bits << 1 == 0) return 0x80808080808080ull;
   const int e = (int)(bits >> 52) & 2047;
   unsigned long long m = (bits & 0xfffffffffffffull) | (e ? 1ull << 52 : 0ull);
   const int sh = e_row - max(e, 1);
@@ -124,6 +137,21 @@ __device__ __forceinline__ unsigned long long fixed_point(double x, int e_row) {
   if (sh > 0) m = sh < 56 ? (m + (1ull << (sh - 1))) >> sh : 0ull;
   const long long f = (long long)bits < 0 ? -(long long)m : (long long)m;
   return (unsigned long long)f + 0x80808080808080ull;
+}
+// The same for e_row >= kFastExp, in 15 integer instructions: zeros and
+// subnormals (no implicit bit) are shifted out with the rest of what is below
+// the unit.
+constexpr int kFastExp = 66;
+__device__ __forceinline__ unsigned long long fixed_point(double x, int e_row) {
+  const int hi = __double2hiint(x);
+  const unsigned lo = (unsigned)__double2loint(x);
+  const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
+  // two fractional bits, then one addition rounds (half away from zero)
+  const unsigned long long m = ((unsigned long long)__funnelshift_l(lo, mh, 2) << 32) | (lo << 2);
+  const int sh = min(e_row - ((hi >> 20) & 2047), 63);
+  const unsigned long long t = ((m >> sh) + 1) >> 1;
+  const unsigned long long sg = (long long)(hi >> 31);
+  return (t ^ sg) - sg + 0x80808080808080ull;
 }
 
 // The digits of eight k of row r (piece kg) into the planes.
@@ -134,7 +162,14 @@ __device__ __forceinline__ void store_digits(__half (*planes)[ROWS][KS], int r, 
   const __half2 off = __float2half2_rn(1152.f);  // 1024 + byte - 1152 = digit
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    const unsigned long long f0 = fixed_point(x[2 * q], e_row), f1 = fixed_point(x[2 * q + 1], e_row);
+    unsigned long long f0, f1;
+    if (e_row >= kFastExp) {
+      f0 = fixed_point(x[2 * q], e_row);
+      f1 = fixed_point(x[2 * q + 1], e_row);
+    } else {
+      f0 = fixed_point_small(x[2 * q], e_row);
+      f1 = fixed_point_small(x[2 * q + 1], e_row);
+    }
     const uint32_t l0 = (uint32_t)f0, l1 = (uint32_t)f1, u0 = (uint32_t)(f0 >> 32), u1 = (uint32_t)(f1 >> 32);
     const uint32_t b01 = __byte_perm(l0, l1, 0x5140), b23 = __byte_perm(l0, l1, 0x7362),
                    b45 = __byte_perm(u0, u1, 0x5140), b6 = __byte_perm(u0, u1, 0x7362);
@@ -155,125 +190,179 @@ __device__ __forceinline__ void store_digits(__half (*planes)[ROWS][KS], int r, 
         make_uint4(h[d][0], h[d][1], h[d][2], h[d][3]);
 }
 
-__global__ void __launch_bounds__(256, 2) gemm_digits_kernel(Gemm g, int kc, double* P,
-                                                             int* tcnt) {
+// One 16-deep step of the 34 digit products on the 16 x 8 outputs at (r0, c0);
+// p0: first of the step's two 16-byte pieces.
+template <int MT, int NT, int KS>
+__device__ __forceinline__ void digits_step(float (&acc)[kWeights][4], const __half (*a)[MT][KS],
+                                            const __half (*b)[NT][KS], int r0, int c0, int p0,
+                                            int lane) {
+  uint32_t fb[kDigits + 1][2];
+  {
+    // lanes 0-15 address digit j, 16-31 digit j + 1
+    const int r = c0 + (lane & 7), p = p0 + ((lane >> 3) & 1);
+#pragma unroll
+    for (int j = 0; j < kDigits; j += 2) {
+      uint32_t x[4];
+      const int jj = min(j + (lane >> 4), kDigits - 1);
+      digits_ldsm(x, &b[jj][r][(p ^ (r & 7)) * 8]);
+      fb[j][0] = x[0];
+      fb[j][1] = x[1];
+      fb[j + 1][0] = x[2];
+      fb[j + 1][1] = x[3];
+    }
+  }
+  const int r = r0 + (lane & 15), p = p0 + (lane >> 4);
+#pragma unroll
+  for (int i = 0; i < kDigits; ++i) {
+    uint32_t fa[4];
+    digits_ldsm(fa, &a[i][r][(p ^ (r & 7)) * 8]);
+#pragma unroll
+    for (int j = 0; j < kDigits; ++j)
+      if (i + j < kWeights) digits_mma(acc[i + j], fa, fb[j][0], fb[j][1]);
+  }
+}
+
+// sum_d acc_d 256^-d of output i as an integer with unit 2^-43 (|sum| < 2^62
+// over a depth of 128)
+__device__ __forceinline__ long long digits_sum(const float (&acc)[kWeights][4], int i) {
+  int w[kWeights];
+#pragma unroll
+  for (int d = 0; d < kWeights; ++d) w[d] = __float2int_rn(acc[d][i]);
+  return ((long long)(w[0] * 256 + w[1]) << 35) + ((long long)(w[2] * 256 + w[3]) << 19) +
+         ((long long)(w[4] * 256 + w[5]) << 3) + ((w[6] * 256 + w[7] + 4096) >> 13);
+}
+
+// v + t 2^(E0 + E1 - 55 - f), |x| < 2^E in a row, E = e - 1022
+__device__ __forceinline__ double digits_add(double v, long long t, int e0, int e1, int f) {
+  const int sc = e0 + e1 - 2 * 1022 - 55 - f;
+  if (sc >= -1022 && sc <= 1023)
+    return fma((double)t, __hiloint2double((sc + 1023) << 20, 0), v);
+  if (max(e0, e1) >= kBadExp) return __hiloint2double(0x7ff80000, 0);
+  return v + scalbn((double)t, sc);
+}
+
+// The pieces of a tile of R rows that a thread loads and splits: piece p of a
+// row holds k = p, p + 16, .. p + 112 (both operands alike); lanes run along the
+// contiguous dimension (`rows`: k), so that a warp reads whole sectors.
+template <int R, int THR>
+struct Pieces {
+  static constexpr int kN = R * 16 / THR;
+  double x[kN][8];
+  __device__ __forceinline__ static int row(bool rows, int u) {
+    const int t = threadIdx.x + u * THR;
+    return rows ? t >> 4 : t % R;
+  }
+  __device__ __forceinline__ static int piece(bool rows, int u) {
+    const int t = threadIdx.x + u * THR;
+    return rows ? t & 15 : t / R;
+  }
+  // rows r0 .. of nr, depth k0 .. ke; zeros outside
+  __device__ __forceinline__ void load(const double* A, long long ld, bool rows, int r0, int nr,
+                                       int k0, int ke) {
+#pragma unroll
+    for (int u = 0; u < kN; ++u) {
+      const int r = r0 + row(rows, u), k = k0 + piece(rows, u);
+      const double* a = rows ? A + r * ld + k : A + k * ld + r;
+      const long long step = rows ? 16 : 16 * ld;
+      if (r < nr && k + 112 < ke) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[u][i] = __ldcg(a + i * step);
+      } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[u][i] = r < nr && k + 16 * i < ke ? __ldcg(a + i * step) : 0.0;
+      }
+    }
+  }
+  __device__ __forceinline__ void exponents(int (*emax)[17], bool rows) const {
+#pragma unroll
+    for (int u = 0; u < kN; ++u) {
+      int e = 0;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) e = max(e, field(x[u][i]));
+      emax[row(rows, u)][piece(rows, u)] = e;
+    }
+  }
+  __device__ __forceinline__ void split(__half (*planes)[R][kGK], const int (*emax)[17], int* er,
+                                        bool rows) const {
+#pragma unroll
+    for (int u = 0; u < kN; ++u) {
+      const int r = row(rows, u), p = piece(rows, u);
+      int e = emax[r][0];
+#pragma unroll
+      for (int i = 1; i < 16; ++i) e = max(e, emax[r][i]);
+      e = row_exponent(e);
+      store_digits(planes, r, p, x[u], e);
+      if (p == 0) er[r] = e;
+    }
+  }
+};
+
+template <int MT, int NT>
+__global__ void __launch_bounds__(GemmTile<MT, NT>::kThreads)
+    gemm_digits_kernel(Gemm g, int kc, double* P, int* tcnt) {
+  using Tile = GemmTile<MT, NT>;
+  constexpr int THR = Tile::kThreads;
   extern __shared__ __align__(16) unsigned char gsm_[];
-  GemmSmem& S = *reinterpret_cast<GemmSmem*>(gsm_);
+  Tile& S = *reinterpret_cast<Tile*>(gsm_);
   __shared__ int s_last;
   const int b = blockIdx.z / kc, z = blockIdx.z % kc;
-  const int tn = (g.N + kGT - 1) / kGT;  // row tiles may exceed a grid's y limit
-  const int m0 = blockIdx.x / tn * kGT, n0 = blockIdx.x % tn * kGT;
+  const int tn = (g.N + NT - 1) / NT;  // row tiles may exceed a grid's y limit
+  const int m0 = blockIdx.x / tn * MT, n0 = blockIdx.x % tn * NT;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   double* C = g.C + (long long)b * g.sC;
-  const double* A = g.A + (long long)b * g.sA;
-  const double* B = g.B + (long long)b * g.sB;
-  // this CTA's K range: part z of kc, in whole chunks
-  const int nsl = (g.K + kGK - 1) / kGK;
-  const int kb = (int)((long long)z * nsl / kc) * kGK;
-  const int ke = min(g.K, (int)((long long)(z + 1) * nsl / kc) * kGK);
-  // loading thread (row, piece) of each operand, rows along the contiguous
-  // dimension of a transposed one; piece p holds k = p, p + 8, .. p + 56 (both
-  // operands alike), so that a warp reads whole sectors
+  pdl_wait();
+  pdl_trigger();
+  // this CTA's chunks: part z of kc
+  const int n1 = (g.K + kGK - 1) / kGK, nsl = g.A2 != nullptr ? 2 * n1 : n1;
+  const int cb = (int)((long long)z * nsl / kc), ce = (int)((long long)(z + 1) * nsl / kc);
   const bool a_rows = !g.tA, b_rows = g.tB;  // k contiguous
-  const int ra = a_rows ? tid >> 3 : tid & 31, ka = a_rows ? tid & 7 : tid >> 5;
-  const int rb = b_rows ? tid >> 3 : tid & 31, kbp = b_rows ? tid & 7 : tid >> 5;
-  const int wm = warp & 1, wn = warp >> 1;  // this warp's 16 x 8 outputs
+  const int wm = 16 * (warp % (MT / 16)), wn = 8 * (warp / (MT / 16));
   double out[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int k0 = kb; k0 < ke; k0 += kGK) {
-    double xa[8], xb[8];
-    int ea = 1, eb = 1;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int k = k0 + ka + 8 * i, m = m0 + ra;
-      xa[i] = m < g.M && k < ke ? (a_rows ? A[m * g.lda + k] : A[k * g.lda + m]) : 0.0;
+  for (int ch = cb; ch < ce; ++ch) {
+    const bool second = ch >= n1;
+    const double* A = (second ? g.A2 : g.A) + (long long)b * g.sA;
+    const double* B = (second ? g.B2 : g.B) + (long long)b * g.sB;
+    const int k0 = (second ? ch - n1 : ch) * kGK;
+    {
+      Pieces<MT, THR> pa;
+      Pieces<NT, THR> pb;
+      pa.load(A, g.lda, a_rows, m0, g.M, k0, g.K);
+      pb.load(B, g.ldb, b_rows, n0, g.N, k0, g.K);
+      pa.exponents(S.emax, a_rows);
+      pb.exponents(S.emax + MT, b_rows);
+      __syncthreads();  // (and the previous chunk's digits and exponents have been read)
+      pa.split(S.a, S.emax, S.e, a_rows);
+      pb.split(S.b, S.emax + MT, S.e + MT, b_rows);
+      __syncthreads();
     }
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int k = k0 + kbp + 8 * i, n = n0 + rb;
-      xb[i] = n < g.N && k < ke ? (b_rows ? B[n * g.ldb + k] : B[k * g.ldb + n]) : 0.0;
-    }
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      ea = max(ea, exponent_of(xa[i]));
-      eb = max(eb, exponent_of(xb[i]));
-    }
-    S.emax[0][ra][ka] = ea;
-    S.emax[1][rb][kbp] = eb;
-    __syncthreads();  // (and the previous chunk's digits have been read)
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      ea = max(ea, S.emax[0][ra][i]);
-      eb = max(eb, S.emax[1][rb][i]);
-    }
-    store_digits(S.d[0], ra, ka, xa, ea);
-    store_digits(S.d[1], rb, kbp, xb, eb);
-    if (ka == 0) S.e[0][ra] = ea;
-    if (kbp == 0) S.e[1][rb] = eb;
-    __syncthreads();
     float acc[kWeights][4];
 #pragma unroll
     for (int d = 0; d < kWeights; ++d)
 #pragma unroll
       for (int i = 0; i < 4; ++i) acc[d][i] = 0.f;
+#pragma unroll 1
+    for (int ks = 0; ks < kGK / 16; ++ks) digits_step(acc, S.a, S.b, wm, wn, 2 * ks, lane);
 #pragma unroll
-    for (int ks = 0; ks < kGK / 16; ++ks) {
-      uint32_t fa[kDigits][4], fb[kDigits + 1][2];
-      {
-        const int r = 16 * wm + (lane & 15), p = 2 * ks + (lane >> 4);
-#pragma unroll
-        for (int i = 0; i < kDigits; ++i) digits_ldsm(fa[i], &S.d[0][i][r][(p ^ (r & 7)) * 8]);
-      }
-      {
-        // lanes 0-15 address digit j, 16-31 digit j + 1
-        const int r = 8 * wn + (lane & 7), p = 2 * ks + ((lane >> 3) & 1);
-#pragma unroll
-        for (int j = 0; j < kDigits; j += 2) {
-          uint32_t x[4];
-          const int jj = min(j + (lane >> 4), kDigits - 1);
-          digits_ldsm(x, &S.d[1][jj][r][(p ^ (r & 7)) * 8]);
-          fb[j][0] = x[0];
-          fb[j][1] = x[1];
-          fb[j + 1][0] = x[2];
-          fb[j + 1][1] = x[3];
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < kDigits; ++i)
-#pragma unroll
-        for (int j = 0; j < kDigits; ++j)
-          if (i + j < kWeights) digits_mma(acc[i + j], fa[i], fb[j][0], fb[j][1]);
-    }
-    // sum_d acc_d 256^-d as an integer with unit 2^-44, one float64 rounding;
-    // times 2^(Ea + Eb - 56), |x| < 2^E, E = e - 1022
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      int v[kWeights];
-#pragma unroll
-      for (int d = 0; d < kWeights; ++d) v[d] = __float2int_rn(acc[d][i]);
-      const long long t = ((long long)(v[0] * 256 + v[1]) << 36) + ((long long)(v[2] * 256 + v[3]) << 20) +
-                          ((long long)(v[4] * 256 + v[5]) << 4) + ((v[6] * 256 + v[7] + 2048) >> 12);
-      const int e0 = S.e[0][16 * wm + (lane >> 2) + 8 * (i >> 1)],
-                e1 = S.e[1][8 * wn + 2 * (lane & 3) + (i & 1)];
-      const int sc = e0 + e1 - 2 * 1022 - 56;
-      if (sc >= -1022 && sc <= 1023)
-        out[i] = fma((double)t, __hiloint2double((sc + 1023) << 20, 0), out[i]);
-      else if (max(e0, e1) >= kBadExp)
-        out[i] = __hiloint2double(0x7ff80000, 0);
-      else
-        out[i] += scalbn((double)t, sc);
-    }
+    for (int i = 0; i < 4; ++i)
+      out[i] = digits_add(out[i], digits_sum(acc, i), S.e[wm + (lane >> 2) + 8 * (i >> 1)],
+                          S.e[MT + wn + 2 * (lane & 3) + (i & 1)], 0);
+    if (ch + 1 < ce) __syncthreads();
   }
+  auto store = [&](int r, int c, double x) {
+    const long long i = r * g.ldc + c;
+    if (g.alpha != 1.0) x *= g.alpha;
+    if (g.sub != nullptr) x -= __ldcg(g.sub + i);
+    if (g.mul != nullptr) x *= __ldcg(g.mul + i);
+    C[i] = x;
+  };
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const int r = m0 + 16 * wm + (lane >> 2) + 8 * (i >> 1), c = n0 + 8 * wn + 2 * (lane & 3) + (i & 1);
+    const int r = m0 + wm + (lane >> 2) + 8 * (i >> 1), c = n0 + wn + 2 * (lane & 3) + (i & 1);
     if (r >= g.M || c >= g.N) continue;
-    if (kc > 1) {
+    if (kc > 1)
       P[(((long long)z * gridDim.z / kc + b) * g.M + r) * g.N + c] = out[i];
-      continue;
-    }
-    double x = g.alpha * out[i];
-    if (g.beta != 0.0) x += g.beta * C[r * g.ldc + c];
-    C[r * g.ldc + c] = x;
+    else
+      store(r, c, out[i]);
   }
   if (kc == 1) return;
   // split K: the tile's last CTA to arrive adds the kc sums in order
@@ -285,16 +374,15 @@ __global__ void __launch_bounds__(256, 2) gemm_digits_kernel(Gemm g, int kc, dou
   if (!s_last) return;
   __threadfence();
   const int batch = gridDim.z / kc;
-  for (int i = tid; i < kGT * kGT; i += 256) {
-    const int r = m0 + i / kGT, c = n0 + i % kGT;
+#pragma unroll
+  for (int i = 0; i < MT * NT / THR; ++i) {
+    const int r = m0 + (tid + i * THR) / NT, c = n0 + (tid + i * THR) % NT;
     if (r >= g.M || c >= g.N) continue;
     double sum = 0.0;
-#pragma unroll 4
+#pragma unroll 8
     for (int zz = 0; zz < kc; ++zz)
       sum += __ldcg(P + (((long long)zz * batch + b) * g.M + r) * g.N + c);
-    double x = g.alpha * sum;
-    if (g.beta != 0.0) x += g.beta * C[r * g.ldc + c];
-    C[r * g.ldc + c] = x;
+    store(r, c, sum);
   }
   if (tid == 0) tcnt[tile_id] = 0;
 }
@@ -338,7 +426,7 @@ struct MatOp {
 };
 
 struct MatHalf {
-  __half d[2][kDigits][kMT][kCD];  // as in GemmSmem, rows of 16 pieces
+  __half d[2][kDigits][kMT][kCD];  // as in GemmTile
   long long part[4][kMT][kMT];     // sums of the four depth slices
   int emax[kMT][17];
   int e[2][kMT];
@@ -391,7 +479,7 @@ __global__ void __launch_bounds__(256 * H) mat_product_kernel(MatOp o) {
     const double* A = o.A[half][ps];
     const double* B = o.B[half][ps] + (o.sel_b ? s * kCD * kCD : 0);
     double xa[8], xb[8];
-    int ea = 1, eb = 1;
+    int ea = 0, eb = 0;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const int k = ka + 16 * i;  // piece p holds k = p, p + 16, ..
@@ -401,8 +489,8 @@ __global__ void __launch_bounds__(256 * H) mat_product_kernel(MatOp o) {
     for (int i = 0; i < 8; ++i) xb[i] = __ldcg(B + (kb + 16 * i) * kCD + n0 + rb);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      ea = max(ea, exponent_of(xa[i]));
-      eb = max(eb, exponent_of(xb[i]));
+      ea = max(ea, field(xa[i]));
+      eb = max(eb, field(xb[i]));
     }
 #pragma unroll
     for (int i = 8; i > 0; i >>= 1) ea = max(ea, __shfl_xor_sync(0xffffffffu, ea, i));
@@ -410,6 +498,8 @@ __global__ void __launch_bounds__(256 * H) mat_product_kernel(MatOp o) {
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < 16; ++i) eb = max(eb, S.emax[rb][i]);
+    ea = row_exponent(ea);
+    eb = row_exponent(eb);
     store_digits(S.d[0], ra, ka, xa, ea);
     store_digits(S.d[1], rb, kb, xb, eb);
     if (ka == 0) S.e[0][ra] = ea;
@@ -421,51 +511,15 @@ __global__ void __launch_bounds__(256 * H) mat_product_kernel(MatOp o) {
 #pragma unroll
       for (int i = 0; i < 4; ++i) acc[d][i] = 0.f;
 #pragma unroll
-    for (int ks = 0; ks < 2; ++ks) {
-      uint32_t fa[kDigits][4], fb[kDigits + 1][2];
-      {
-        const int rr = lane & 15, p = 4 * ws + 2 * ks + (lane >> 4);
+    for (int ks = 0; ks < 2; ++ks)
+      digits_step(acc, S.d[0], S.d[1], 0, 8 * wn, 4 * ws + 2 * ks, lane);
 #pragma unroll
-        for (int i = 0; i < kDigits; ++i) digits_ldsm(fa[i], &S.d[0][i][rr][(p ^ (rr & 7)) * 8]);
-      }
-      {
-        const int rr = 8 * wn + (lane & 7), p = 4 * ws + 2 * ks + ((lane >> 3) & 1);
-#pragma unroll
-        for (int j = 0; j < kDigits; j += 2) {
-          uint32_t x[4];
-          const int jj = min(j + (lane >> 4), kDigits - 1);
-          digits_ldsm(x, &S.d[1][jj][rr][(p ^ (rr & 7)) * 8]);
-          fb[j][0] = x[0];
-          fb[j][1] = x[1];
-          fb[j + 1][0] = x[2];
-          fb[j + 1][1] = x[3];
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < kDigits; ++i)
-#pragma unroll
-        for (int j = 0; j < kDigits; ++j)
-          if (i + j < kWeights) digits_mma(acc[i + j], fa[i], fb[j][0], fb[j][1]);
-    }
-    // unit 2^-43: four slices of at most 32 x 2^12 keep the sum below 2^63
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      int w[kWeights];
-#pragma unroll
-      for (int d = 0; d < kWeights; ++d) w[d] = __float2int_rn(acc[d][i]);
+    for (int i = 0; i < 4; ++i)
       S.part[ws][(lane >> 2) + 8 * (i >> 1)][8 * wn + 2 * (lane & 3) + (i & 1)] =
-          ((long long)(w[0] * 256 + w[1]) << 35) + ((long long)(w[2] * 256 + w[3]) << 19) +
-          ((long long)(w[4] * 256 + w[5]) << 3) + ((w[6] * 256 + w[7] + 4096) >> 13);
-    }
+          digits_sum(acc, i);
     __syncthreads();
     const long long t = S.part[0][r][c] + S.part[1][r][c] + S.part[2][r][c] + S.part[3][r][c];
-    const int e0 = S.e[0][r], e1 = S.e[1][c], sc = e0 + e1 - 2 * 1022 - 55 - o.fs * s;
-    if (sc >= -1022 && sc <= 1023)
-      v = fma((double)t, __hiloint2double((sc + 1023) << 20, 0), v);
-    else if (max(e0, e1) >= kBadExp)
-      v = __hiloint2double(0x7ff80000, 0);
-    else
-      v += scalbn((double)t, sc);
+    v = digits_add(v, t, S.e[0][r], S.e[1][c], o.fs * s);
   }
   const int idx = (m0 + r) * kCD + n0 + c;
   const double dg = m0 + r == n0 + c ? o.diag : 0.0;
@@ -497,12 +551,28 @@ __global__ void __launch_bounds__(256 * H) mat_product_kernel(MatOp o) {
 
 // ------------------------------------------------------- small kernels
 
-__global__ void col_mean_kernel(const double* __restrict__ K, int T,
-                                double* __restrict__ mu) {
-  const int c = threadIdx.x;  // 128 threads
+// mu[c] = mean over T of K[t][c]; blocks of 256 threads, four channels (a
+// sector) each, 64 rows at a time
+__global__ void __launch_bounds__(256) col_mean_kernel(const double* __restrict__ K, int T,
+                                                       double* __restrict__ mu) {
+  __shared__ double sh[64][4];
+  const int c = threadIdx.x & 3, r = threadIdx.x >> 2;
   double s = 0.0;
-  for (int t = 0; t < T; ++t) s += K[(long long)t * kCD + c];
-  mu[c] = s / (double)T;
+  for (int t = r; t < T; t += 64) s += K[(long long)t * kCD + 4 * blockIdx.x + c];
+  sh[r][c] = s;
+  for (int w = 32; w > 0; w >>= 1) {
+    __syncthreads();
+    if (r < w) sh[r][c] += sh[r + w][c];
+  }
+  if (r == 0) mu[4 * blockIdx.x + c] = sh[0][c] / (double)T;
+}
+
+// qp[j][t] = q[t][j] (rows of d): the query rows in the order of the logits
+__global__ void permute_kernel(const double* __restrict__ q, int nt, int g,
+                               double* __restrict__ qp) {
+  const long long row = blockIdx.x;  // j nt + t
+  const long long j = row / nt, t = row % nt;
+  qp[row * kCD + threadIdx.x] = q[(t * g + j) * kCD + threadIdx.x];
 }
 
 // Kc = K - mu (rows of d)
@@ -564,30 +634,6 @@ __global__ void neg_kernel(const double* __restrict__ x, long long n, double* __
     y[i] = -x[i];
 }
 
-// C = A - B
-__global__ void sub_kernel(const double* __restrict__ A, const double* __restrict__ B,
-                           long long n, double* __restrict__ C) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x)
-    C[i] = A[i] - B[i];
-}
-
-// X *= M elementwise (M is 0 or 1)
-__global__ void mask_mul_kernel(double* __restrict__ X, const double* __restrict__ M,
-                                long long n) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x)
-    X[i] = X[i] * M[i];
-}
-
-// log(max(p, 1e-300))
-__global__ void logclamp_kernel(const double* __restrict__ P, long long n,
-                                double* __restrict__ L) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x)
-    L[i] = log(fmax(P[i], 1e-300));
-}
-
 __device__ __forceinline__ bool is_window(int s, int t, int sink, int recent) {
   return s < sink || s > t - recent;
 }
@@ -598,85 +644,153 @@ __device__ __forceinline__ bool is_window(int s, int t, int sink, int recent) {
 // r = mx - mn, u = (clamp(z, mn, mx) - mn) * 3 / r, code = clamp(rint(u), 0,
 // 3), zh = code * fp16(r / 3) + fp16(mn) (fp16 values of the float32
 // rounding), inside = mn <= z <= mx.  Degenerate groups (r <= 1e-30): code
-// 0, scale 0.  One warp per (row, group).
-__global__ void q2_kernel(const double* __restrict__ Z, int rows, int G,
-                          double clip, double* __restrict__ Zh,
-                          double* __restrict__ inside) {
+// 0, scale 0.  One warp per 256 consecutive channels (8 groups of 32 or 2 of
+// 128).  What bounds it: float64 operations, 2 per clock and SM.  Comparisons
+// are made on integers and a warp's groups share one evaluation of the scalars
+// (two divisions), each on its own lanes: 5 float64 operations per value; with
+// one group per warp 2048 rows took 15.8 us, now 5.9.
+__device__ __forceinline__ long long order_key(double z) {
+  long long b = __double_as_longlong(z);
+  if ((unsigned long long)b == 0x8000000000000000ull) b = 0;  // -0 = 0
+  return b < 0 ? b ^ 0x7fffffffffffffffll : b;
+}
+__device__ __forceinline__ double key_value(long long k) {
+  return __longlong_as_double(k < 0 ? k ^ 0x7fffffffffffffffll : k);
+}
+template <int NG>  // groups per warp: 8 (of 32 channels) or 2 (of 128)
+__global__ void __launch_bounds__(256) q2_kernel(const double* Z, long long n, double clip,
+                                                 double* Zh, double* inside) {
+  constexpr int PER = 8 / NG;  // channels of a group per lane
   const int lane = threadIdx.x & 31;
-  const long long wid = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
-  const int groups = kCD / G;
-  if (wid >= (long long)rows * groups) return;
-  const long long row = wid / groups;
-  const int g0 = (int)(wid % groups) * G;
-  const int per = G / 32;  // 1 or 4 channels per lane
-  double z[4];
-  double lo = INFINITY, hi = -INFINITY;
-  for (int e = 0; e < per; ++e) {
-    z[e] = Z[row * kCD + g0 + e * 32 + lane];
-    lo = fmin(lo, z[e]);
-    hi = fmax(hi, z[e]);
+  const long long wid = (blockIdx.x * 256ll + threadIdx.x) >> 5;
+  pdl_wait();
+  pdl_trigger();
+  const long long base = wid * 256 + lane;  // group i, channel e: base + (i PER + e) 32
+  if (wid * 256 >= n) return;  // n is a multiple of 128: the last warp may be half full
+  const long long kInf = 0x7ff0000000000000ll;
+  long long key[8], lo[NG], hi[NG];
+  double z[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) z[i] = base + 32 * i < n ? __ldcg(Z + base + 32 * i) : 0.0;
+#pragma unroll
+  for (int i = 0; i < NG; ++i) {
+    lo[i] = kInf;
+    hi[i] = order_key(__longlong_as_double(kInf | (long long)0x8000000000000000ull));
+#pragma unroll
+    for (int e = 0; e < PER; ++e) {
+      const long long k = key[i * PER + e] = order_key(z[i * PER + e]);
+      const bool nan = (__double_as_longlong(z[i * PER + e]) & 0x7fffffffffffffffll) > kInf;
+      lo[i] = !nan && k < lo[i] ? k : lo[i];
+      hi[i] = !nan && k > hi[i] ? k : hi[i];
+    }
+  }
+  // halving exchange: lane bits 4, 3, .. pick the group whose range it ends with
+  int o = 16;
+#pragma unroll
+  for (int n = NG; n > 1; n >>= 1, o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < n / 2; ++i) {
+      const long long l = __shfl_xor_sync(0xffffffffu, up ? lo[i] : lo[i + n / 2], o);
+      const long long h = __shfl_xor_sync(0xffffffffu, up ? hi[i] : hi[i + n / 2], o);
+      const long long l0 = up ? lo[i + n / 2] : lo[i], h0 = up ? hi[i + n / 2] : hi[i];
+      lo[i] = l < l0 ? l : l0;
+      hi[i] = h > h0 ? h : h0;
+    }
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-    hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  for (; o > 0; o >>= 1) {
+    const long long l = __shfl_xor_sync(0xffffffffu, lo[0], o);
+    const long long h = __shfl_xor_sync(0xffffffffu, hi[0], o);
+    lo[0] = l < lo[0] ? l : lo[0];
+    hi[0] = h > hi[0] ? h : hi[0];
   }
-  const double mn = clip * lo, mx = clip * hi;
+  const double mn = clip * key_value(lo[0]), mx = clip * key_value(hi[0]);
   const double r = mx - mn;
   const bool deg = !(r > 1e-30);
   const double inv = deg ? 0.0 : 3.0 / r;
   const double scale = deg ? 0.0 : (double)__half2float(__float2half_rn(__double2float_rn(r / 3.0)));
   const double mn16 = (double)__half2float(__float2half_rn(__double2float_rn(mn)));
-  for (int e = 0; e < per; ++e) {
-    const double u = (fmin(fmax(z[e], mn), mx) - mn) * inv;
-    const double code = fmin(fmax(rint(u), 0.0), 3.0);
-    const long long i = row * kCD + g0 + e * 32 + lane;
-    Zh[i] = __dadd_rn(__dmul_rn(code, scale), mn16);
-    inside[i] = (z[e] >= mn && z[e] <= mx) ? 1.0 : 0.0;
+#pragma unroll
+  for (int i = 0; i < NG; ++i) {
+    const int src = i * (32 / NG);  // first lane of group i
+    const double gmn = __shfl_sync(0xffffffffu, mn, src), gmx = __shfl_sync(0xffffffffu, mx, src);
+    const double ginv = __shfl_sync(0xffffffffu, inv, src);
+    const double gsc = __shfl_sync(0xffffffffu, scale, src);
+    const double g16 = __shfl_sync(0xffffffffu, mn16, src);
+    const long long kmn = order_key(gmn), kmx = order_key(gmx);
+#pragma unroll
+    for (int e = 0; e < PER; ++e) {
+      const long long k = key[i * PER + e];
+      const bool ge = k >= kmn, le = k <= kmx;
+      const double u = ((ge ? (le ? z[i * PER + e] : gmx) : gmn) - gmn) * ginv;
+      const int c = min(max(__double2int_rn(u), 0), 3);
+      // 0, 1, 2, 3 as float64 bits
+      const double code = __hiloint2double(c == 0 ? 0 : 0x3ff00000 + (c >> 1) * 0x100000 +
+                                                          (c == 3 ? 0x80000 : 0), 0);
+      const long long j = base + 32 * (i * PER + e);
+      if (j >= n) continue;
+      Zh[j] = __dadd_rn(__dmul_rn(code, gsc), g16);
+      inside[j] = ge && le ? 1.0 : 0.0;
+    }
   }
 }
 
-// Row (j, t) of [g][nt][T]: logits scale * x (x = the row of X, or of Xc
-// at the BF16-window pairs when windows), masked to s <= t_pos[t]; the
-// softmax goes to P.  When Pref is given, rowv[row] = KL(Pref || P) =
-// sum_s pref (logpref - log max(p, 1e-300)), with log p = l - m - log(sum)
-// (p = 0 entries: log 1e-300; below 1e-300 the clamp).  One block of 256
-// threads per row; exp(l - m) is stored in the sum pass and normalised in
-// the last.
-__device__ __forceinline__ double block_reduce(double v, bool is_max, double* sh) {
+// Row (j, t) of [g][nt][T]: logits x (the row of X, or of Xc at the BF16-window
+// pairs when windows; scaled already), masked to s <= t_pos[t]; the softmax goes
+// to P.  With Pref: D = P - Pref and rowv[row] = KL(Pref || P) =
+// sum_s pref (logpref - log max(p, 1e-300)), log p = x - m - log(sum) (below
+// 1e-300 the clamp); without: that log p goes to logP.  One block of 256
+// threads per row; exp(x - m) is stored in the sum pass and normalised in the
+// last.  What bounds it: float64 operations, about 20 of them in exp; the
+// maximum is taken on integers and the quotient by a product and one exact
+// correction (with a division per element, and D by a pass of its own, 256 rows
+// of 2048 took 54 us, now 36).
+__device__ __forceinline__ double block_reduce(double v, double* sh) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const double u = __shfl_xor_sync(0xffffffffu, v, o);
-    v = is_max ? fmax(v, u) : v + u;
-  }
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   __syncthreads();  // sh free from an earlier reduction
   if (lane == 0) sh[w] = v;
   __syncthreads();
   double r = sh[0];
-  for (int i = 1; i < 8; ++i) r = is_max ? fmax(r, sh[i]) : r + sh[i];
+  for (int i = 1; i < 8; ++i) r += sh[i];
   return r;
 }
 
 __global__ void __launch_bounds__(256) softmax_rows_kernel(
-    const double* __restrict__ X, const double* __restrict__ Xc, int rows, int nt,
-    int T, const int32_t* __restrict__ t_pos, double scale, int sink, int recent,
-    double* __restrict__ P, const double* __restrict__ Pref,
-    const double* __restrict__ logPref, double* __restrict__ rowv) {
+    const double* X, const double* Xc, int nt, int T, const int32_t* __restrict__ t_pos,
+    int sink, int recent, double* P, const double* Pref, double* logP, double* D, double* rowv) {
   __shared__ double sh[8];
+  __shared__ long long shk[8];
+  pdl_wait();
+  pdl_trigger();
   const long long row = blockIdx.x;
   const int t = t_pos[row % nt];
   const bool win = Xc != nullptr;
   const double* x = X + row * (long long)T;
   const double* xc = win ? Xc + row * (long long)T : nullptr;
   auto logit = [&](int s) {
-    const double v = (win && is_window(s, t, sink, recent)) ? xc[s] : x[s];
-    return v * scale;
+    return __ldcg((win && is_window(s, t, sink, recent)) ? xc + s : x + s);
   };
-  double m = -INFINITY;
+  // a NaN is passed over here and reaches the sum below
+  long long k = order_key(__longlong_as_double((long long)0xfff0000000000000ull));
   for (int s = threadIdx.x; s < T; s += 256)
-    if (s <= t) m = fmax(m, logit(s));
-  m = block_reduce(m, true, sh);
+    if (s <= t) {
+      const double v = logit(s);
+      const long long kv = order_key(v);
+      const bool nan = (__double_as_longlong(v) & 0x7fffffffffffffffll) > 0x7ff0000000000000ll;
+      k = !nan && kv > k ? kv : k;
+    }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const long long u = __shfl_xor_sync(0xffffffffu, k, o);
+    k = u > k ? u : k;
+  }
+  if ((threadIdx.x & 31) == 0) shk[threadIdx.x >> 5] = k;
+  __syncthreads();
+  for (int i = 0; i < 8; ++i) k = shk[i] > k ? shk[i] : k;
+  const double m = key_value(k);
   double* p = P + row * (long long)T;
   double sum = 0.0;
   for (int s = threadIdx.x; s < T; s += 256) {
@@ -684,46 +798,52 @@ __global__ void __launch_bounds__(256) softmax_rows_kernel(
     p[s] = e;
     sum += e;
   }
-  sum = block_reduce(sum, false, sh);
-  const double lsum = Pref != nullptr ? log(sum) : 0.0;
+  sum = block_reduce(sum, sh);
+  const double lsum = log(sum), inv = 1.0 / sum, lmin = log(1e-300);
   double kl = 0.0;
   for (int s = threadIdx.x; s < T; s += 256) {
-    const double v = p[s] / sum;
+    const long long i = row * (long long)T + s;
+    const double e = p[s];
+    double v = e * inv;
+    v = fma(fma(-v, sum, e), inv, v);  // e / sum
     p[s] = v;
+    const double lp = v > 1e-300 ? (logit(s) - m) - lsum : lmin;
     if (Pref != nullptr) {
-      const double lp = v > 1e-300 ? (logit(s) - m) - lsum : log(1e-300);
-      kl += Pref[row * (long long)T + s] * (logPref[row * (long long)T + s] - lp);
+      const double pr = __ldcg(Pref + i);
+      D[i] = v - pr;
+      kl += pr * (__ldcg(logP + i) - lp);
+    } else {
+      logP[i] = lp;
     }
   }
   if (Pref != nullptr) {
-    kl = block_reduce(kl, false, sh);
+    kl = block_reduce(kl, sh);
     if (threadIdx.x == 0) rowv[row] = kl;
   }
 }
 
 // Gradient of the key loss with respect to the raw logits x of row (j, t)
-// (l = scale x): G[s] = coef * ((pk - p) + pk (gv - sum_s pk gv)) at the
-// causal non-window pairs, 0 elsewhere.  In place over GV.  One warp per row.
-__global__ void key_row_grad_kernel(const double* __restrict__ PK,
-                                    const double* __restrict__ Pref,
-                                    double* __restrict__ GV, int rows, int nt,
-                                    int T, const int32_t* __restrict__ t_pos,
-                                    double coef, int sink, int recent, int win) {
-  const int lane = threadIdx.x & 31;
-  const long long row = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
-  if (row >= rows) return;
+// (l = scale x): G[s] = coef * (D + pk (gv - sum_s pk gv)), D = pk - p, at the
+// causal non-window pairs, 0 elsewhere.  In place over GV.  One block per row
+// (8 rows per block left most SMs idle: 68 us for 256 rows of 2048, now 9).
+__global__ void __launch_bounds__(256) key_row_grad_kernel(
+    const double* PK, const double* D, double* GV, int nt, int T,
+    const int32_t* __restrict__ t_pos, double coef, int sink, int recent, int win) {
+  __shared__ double sh[8];
+  pdl_wait();
+  pdl_trigger();
+  const long long row = blockIdx.x;
   const int t = t_pos[row % nt];
   const double* pk = PK + row * (long long)T;
-  const double* p = Pref + row * (long long)T;
+  const double* d = D + row * (long long)T;
   double* gv = GV + row * (long long)T;
   double gbar = 0.0;
-  for (int s = lane; s < T; s += 32) gbar += pk[s] * gv[s];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) gbar += __shfl_xor_sync(0xffffffffu, gbar, o);
-  for (int s = lane; s < T; s += 32) {
+  for (int s = threadIdx.x; s < T; s += 256) gbar += __ldcg(pk + s) * __ldcg(gv + s);
+  gbar = block_reduce(gbar, sh);
+  for (int s = threadIdx.x; s < T; s += 256) {
     double gsum = 0.0;
     if (s <= t && !(win && is_window(s, t, sink, recent)))
-      gsum = coef * ((pk[s] - p[s]) + pk[s] * (gv[s] - gbar));
+      gsum = coef * (__ldcg(d + s) + __ldcg(pk + s) * (__ldcg(gv + s) - gbar));
     gv[s] = gsum;
   }
 }
@@ -740,39 +860,36 @@ __global__ void zero_window_kernel(double* __restrict__ P, int rows, int nt, int
     if (is_window(s, t, sink, recent)) P[row * (long long)T + s] = 0.0;
 }
 
-// rowv[row] = (add ? rowv[row] : 0) + lam * (sum_c E[row][c]^2) / dm
-__global__ void row_sqsum_kernel(const double* __restrict__ E, int rows, int dm,
-                                 double lam, int add, double* __restrict__ rowv) {
+// rowv[row] = (add ? rowv[row] : 0) + lam * (sum_c A[row][c] B[row][c]) / dm,
+// rows of n
+__global__ void row_dot_kernel(const double* A, const double* B, int rows, int n, int dm,
+                               double lam, int add, double* rowv) {
   const int lane = threadIdx.x & 31;
   const long long row = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+  pdl_wait();
+  pdl_trigger();
   if (row >= rows) return;
   double s = 0.0;
-  for (int c = lane; c < dm; c += 32) {
-    const double e = E[row * (long long)dm + c];
-    s += e * e;
-  }
+  for (int c = lane; c < n; c += 32)
+    s += __ldcg(A + row * (long long)n + c) * __ldcg(B + row * (long long)n + c);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if (lane == 0) {
     const double v = lam * s / (double)dm;
-    rowv[row] = add ? rowv[row] + v : v;
+    rowv[row] = add ? __ldcg(rowv + row) + v : v;
   }
 }
 
-// out = (sum_i rowv[i]) / n, one block of 1024 threads, fixed order
-__global__ void __launch_bounds__(1024) loss_reduce_kernel(const double* __restrict__ rowv,
-                                                           int rows, double n,
-                                                           double* __restrict__ out) {
-  __shared__ double red[1024];
+// out = (sum_i rowv[i]) / n, one block of 256 threads, fixed order
+__global__ void __launch_bounds__(256) loss_reduce_kernel(const double* rowv, int rows, double n,
+                                                          double* out) {
+  __shared__ double sh[8];
+  pdl_wait();
+  pdl_trigger();
   double s = 0.0;
-  for (int i = threadIdx.x; i < rows; i += 1024) s += rowv[i];
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int w = 512; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) *out = red[0] / n;
+  for (int i = threadIdx.x; i < rows; i += 256) s += __ldcg(rowv + i);
+  s = block_reduce(s, sh);
+  if (threadIdx.x == 0) *out = s / n;
 }
 
 // Adam (Kingma & Ba), in the order m = b1 m + (1 - b1) g,
@@ -835,6 +952,8 @@ inline int nblk(long long n, int t = 256) {
   return (int)(b < 4096 ? (b > 0 ? b : 1) : 4096);
 }
 
+constexpr int kGSplit = 160;  // K is split up to this many CTAs, about one per SM
+constexpr int kGSmall = 76;   // fewer tiles x chunks of 64 x 32: 32 x 16 instead
 constexpr long long kGemmScratch = 1 << 21;  // split-K doubles (16 MiB)
 constexpr int kGemmTiles = 512;  // K is split only while a call has fewer tiles
 
@@ -843,22 +962,45 @@ struct GemmCall {
   double* scratch;        // split-K partial sums
   long long scratch_len;  // doubles
   int* tcnt;              // split-K arrival counters, one per output tile (0)
+  static Gemm args(int M, int N, int K, const double* A, long long lda, bool tA,
+                   const double* B, long long ldb, bool tB, double* C, long long ldc) {
+    Gemm g{};
+    g.M = M; g.N = N; g.K = K;
+    g.A = A; g.lda = lda; g.tA = tA;
+    g.B = B; g.ldb = ldb; g.tB = tB;
+    g.C = C; g.ldc = ldc;
+    g.alpha = 1.0;
+    return g;
+  }
   void operator()(int M, int N, int K, const double* A, long long lda, bool tA,
                   const double* B, long long ldb, bool tB, double* C, long long ldc,
-                  double alpha = 1.0, double beta = 0.0, int batch = 1,
-                  long long sA = 0, long long sB = 0, long long sC = 0) const {
-    Gemm g{M, N, K, A, lda, sA, tA ? 1 : 0, B, ldb, sB, tB ? 1 : 0, C, ldc, sC,
-           alpha, beta};
-    const int tm = (M + kGT - 1) / kGT, tn = (N + kGT - 1) / kGT;
+                  double alpha = 1.0, int batch = 1, long long sA = 0, long long sB = 0,
+                  long long sC = 0) const {
+    Gemm g = args(M, N, K, A, lda, tA, B, ldb, tB, C, ldc);
+    g.alpha = alpha;
+    g.sA = sA;
+    g.sB = sB;
+    g.sC = sC;
+    run(g, batch);
+  }
+  void run(const Gemm& g, int batch) const {
+    const long long tiles = (long long)((g.M + 63) / 64) * ((g.N + 31) / 32) * batch;
+    const int chunks = (g.K + kGK - 1) / kGK * (g.A2 != nullptr ? 2 : 1);
+    if (tiles * chunks < kGSmall) launch<32, 16>(g, batch);
+    else launch<64, 32>(g, batch);
+  }
+  template <int MT, int NT>
+  void launch(const Gemm& g, int batch) const {
+    const int tm = (g.M + MT - 1) / MT, tn = (g.N + NT - 1) / NT;
     const long long tiles = (long long)tm * tn * batch;
-    // split K when the output alone gives too few CTAs (two per SM): a CTA
-    // takes ~3 us per chunk whatever its neighbours do
+    // split K while the CTAs do not fill the SMs
     int kc = 1;
-    const int chunks = (K + kGK - 1) / kGK;
-    while (tiles <= kGemmTiles && tiles * kc < 300 && 2 * kc <= chunks &&
-           (long long)(2 * kc) * batch * M * N <= scratch_len)
+    const int chunks = (g.K + kGK - 1) / kGK * (g.A2 != nullptr ? 2 : 1);
+    while (tiles <= kGemmTiles && tiles * kc * 2 <= kGSplit && 2 * kc <= chunks &&
+           (long long)(2 * kc) * batch * g.M * g.N <= scratch_len)
       kc *= 2;
-    gemm_digits_kernel<<<dim3(tn * tm, 1, batch * kc), 256, sizeof(GemmSmem), s>>>(g, kc, scratch, tcnt);
+    launch_pdl(&gemm_digits_kernel<MT, NT>, dim3(tn * tm, 1, batch * kc),
+               dim3(GemmTile<MT, NT>::kThreads), sizeof(GemmTile<MT, NT>), s, g, kc, scratch, tcnt);
   }
 };
 
@@ -868,9 +1010,10 @@ struct Trace {
   const int32_t* tpos;
   int T, nt;
   double *Kc;       // [T][d]     K - mu
+  double *qp;       // [g][nt][d] the query rows
   double *Pref;     // [g][nt][T] softmax of the BF16 logits
   double *logPref;  // [g][nt][T] log max(Pref, 1e-300)
-  double *Lc;       // [g][nt][T] raw window logits q (K - mu)^T (windows only)
+  double *Lc;       // [g][nt][T] window logits scale q (K - mu)^T (windows only)
   double *Phat;     // [g][nt][T] key-phase attention, window pairs zeroed
 };
 
@@ -881,7 +1024,7 @@ struct Calib {
   Trace tr[2];   // calibration, held-out
   // working buffers (sized for the larger trace)
   double *Z, *Zh, *inside, *Kt, *dKt, *dZh;  // [T][d]
-  double *X, *PK, *GV;                       // [g][nt][T]
+  double *X, *PK, *GV, *DP;                  // [g][nt][T]
   double *rowv;                              // [g][nt]
   double *DV, *U;                            // [g][nt][d]
   double *Eo;                                // [g][nt][d_model]
@@ -897,6 +1040,7 @@ struct Calib {
   int* s_dev;
   unsigned* err;
   const double* W;  // [g][d_model][d]
+  double* M;        // [g][d][d] W^T W, or null
   double* gsc;      // split-K scratch of the GEMMs
   int* gcnt;        // split-K arrival counters (kGemmTiles, zero between calls)
   cudaStream_t st;
@@ -929,6 +1073,7 @@ size_t carve(Calib& C, char* base) {
     const long long T = k ? Th : c.T, nt = k ? nh : c.nt;
     Trace& t = C.tr[k];
     t.Kc = L.take<double>(T * D);
+    t.qp = L.take<double>(g * nt * D);
     t.Pref = L.take<double>(g * nt * T);
     t.logPref = L.take<double>(g * nt * T);
     t.Lc = C.windows ? L.take<double>(g * nt * T) : nullptr;
@@ -943,6 +1088,8 @@ size_t carve(Calib& C, char* base) {
   C.X = L.take<double>(g * nm * Tm);
   C.PK = L.take<double>(g * nm * Tm);
   C.GV = L.take<double>(g * nm * Tm);
+  C.DP = L.take<double>(g * nm * Tm);
+  C.M = L.take<double>(g * D2);
   C.rowv = L.take<double>(g * nm);
   C.DV = L.take<double>(g * nm * D);
   C.U = L.take<double>(g * nm * D);
@@ -1111,82 +1258,125 @@ double adam_reach(double lr, double b1, double b2, int t) {
 
 namespace {
 
-// Inputs that stay fixed over the steps: K - mu, the BF16 reference
-// attention p (and log p), the raw window logits.
+// Inputs that stay fixed over the steps: K - mu, the query rows by head, the
+// BF16 reference attention p and log p, the window logits.
 void trace_setup(Calib& C, Trace& t, const double* mu) {
   GemmCall gm = C.gemm();
   const int g = C.c.g, D = kCD;
-  const long long nT = (long long)t.T * D, r = (long long)g * t.nt;
+  const long long nT = (long long)t.T * D, r = (long long)g * t.nt, nD = (long long)t.nt * D;
   center_kernel<<<nblk(nT), 256, 0, C.st>>>(t.K, mu, nT, t.Kc);
-  // raw BF16 logits q_j K^T into X, softmax into Pref
-  gm(t.nt, t.T, D, t.q, (long long)g * D, false, t.K, D, true, C.X, t.T, 1.0, 0.0,
-     g, D, 0, (long long)t.nt * t.T);
-  softmax_rows_kernel<<<(unsigned)r, 256, 0, C.st>>>(
-      C.X, nullptr, (int)r, t.nt, t.T, t.tpos, C.scale, 0, 0, t.Pref, nullptr,
-      nullptr, nullptr);
-  logclamp_kernel<<<nblk(r * t.T), 256, 0, C.st>>>(t.Pref, r * t.T, t.logPref);
+  permute_kernel<<<(unsigned)r, kCD, 0, C.st>>>(t.q, t.nt, g, t.qp);
+  // BF16 logits scale q_j K^T into X, softmax into Pref
+  gm(t.nt, t.T, D, t.qp, D, false, t.K, D, true, C.X, t.T, C.scale, g, nD, 0,
+     (long long)t.nt * t.T);
+  launch_pdl(&softmax_rows_kernel, dim3((unsigned)r), dim3(256), 0, C.st, C.X, nullptr, t.nt, t.T,
+             t.tpos, 0, 0, t.Pref, nullptr, t.logPref, nullptr, nullptr);
   if (C.windows)
-    gm(t.nt, t.T, D, t.q, (long long)g * D, false, t.Kc, D, true, t.Lc, t.T, 1.0,
-       0.0, g, D, 0, (long long)t.nt * t.T);
+    gm(t.nt, t.T, D, t.qp, D, false, t.Kc, D, true, t.Lc, t.T, C.scale, g, nD, 0,
+       (long long)t.nt * t.T);
 }
 
-// Effective rotated-and-back rows Q2(X R) R^T into C.Kt (Zh, inside kept).
-void q2_roundtrip(Calib& C, const double* X, int T, double clip) {
+// Effective rotated-and-back rows Q2(X R) R^T, less `sub` when given, into C.Kt
+// (Zh, inside kept).
+void q2_roundtrip(Calib& C, const double* X, int T, double clip, const double* sub) {
   GemmCall gm = C.gemm();
   gm(T, kCD, kCD, X, kCD, false, C.R, kCD, false, C.Z, kCD);
-  const long long warps = (long long)T * (kCD / C.c.group);
-  q2_kernel<<<nwarp_blocks(warps), 256, 0, C.st>>>(C.Z, T, C.c.group, clip, C.Zh, C.inside);
-  gm(T, kCD, kCD, C.Zh, kCD, false, C.R, kCD, true, C.Kt, kCD);
+  const long long n = (long long)T * kCD;
+  launch_pdl(C.c.group == 32 ? &q2_kernel<8> : &q2_kernel<2>, dim3(nwarp_blocks((n + 255) / 256)),
+             dim3(256), 0, C.st, C.Z, n, clip, C.Zh, C.inside);
+  Gemm k = gm.args(T, kCD, kCD, C.Zh, kCD, false, C.R, kCD, true, C.Kt, kCD);
+  k.sub = sub;
+  gm.run(k, 1);
 }
 
-// L_K of trace t under C.R into *out; leaves PK, Eo for the backward.
+// rowv[j, t] (+)= lam ||e_j||^2 / d_model with e_j = DV_j W_j^T.  With the
+// products M_j = W_j^T W_j at hand ||e||^2 = DV (DV M)^T, and U0 = DV M, the
+// gradient e_j W_j, is done as well; else e_j goes to Eo.
+void output_error(Calib& C, Trace& t, double lam, int add) {
+  GemmCall gm = C.gemm();
+  const int g = C.c.g, D = kCD, dm = C.c.d_model, r = g * t.nt;
+  const long long nD = (long long)t.nt * D;
+  if (C.M != nullptr) {
+    gm(t.nt, D, D, C.DV, D, false, C.M, D, false, C.U, D, 1.0, g, nD, (long long)kD2, nD);
+    launch_pdl(&row_dot_kernel, dim3(nwarp_blocks(r)), dim3(256), 0, C.st, C.DV, C.U, r, D, dm, lam,
+               add, C.rowv);
+    return;
+  }
+  gm(t.nt, dm, D, C.DV, D, false, C.W, D, true, C.Eo, dm, 1.0, g, nD, (long long)dm * D,
+     (long long)t.nt * dm);
+  launch_pdl(&row_dot_kernel, dim3(nwarp_blocks(r)), dim3(256), 0, C.st, C.Eo, C.Eo, r, dm, dm, lam,
+             add, C.rowv);
+}
+
+// U0 = e_j W_j (after output_error on the same trace)
+void output_grad(Calib& C, Trace& t) {
+  const int g = C.c.g, D = kCD, dm = C.c.d_model;
+  if (C.M == nullptr)
+    C.gemm()(t.nt, D, dm, C.Eo, dm, false, C.W, D, false, C.U, D, 1.0, g,
+             (long long)t.nt * dm, (long long)dm * D, (long long)t.nt * D);
+}
+
+// The products M_j pay when they replace more than they cost: per step and
+// phase 2 nt rows through W (once for e, once for U) become nt rows through a
+// d x d matrix; M_j itself costs d rows through W.
+void output_setup(Calib& C) {
+  const optr_calib_config& c = C.c;
+  if (c.d_model < kCD || (double)c.steps * c.nt < kCD / 2) {
+    C.M = nullptr;
+    return;
+  }
+  C.gemm()(kCD, kCD, c.d_model, C.W, kCD, true, C.W, kCD, false, C.M, kCD, 1.0, c.g,
+           (long long)c.d_model * kCD, (long long)c.d_model * kCD, (long long)kD2);
+}
+
+void loss_mean(Calib& C, int rows, double* out) {
+  launch_pdl(&loss_reduce_kernel, dim3(1), dim3(256), 0, C.st, C.rowv, rows, (double)rows, out);
+}
+
+// L_K of trace t under C.R into *out; leaves PK, DP and the output error's
+// buffers for the backward.
 void key_forward(Calib& C, Trace& t, double* out) {
   GemmCall gm = C.gemm();
-  const int g = C.c.g, D = kCD, dm = C.c.d_model;
-  const long long r = (long long)g * t.nt, nTT = (long long)t.nt * t.T;
-  q2_roundtrip(C, t.Kc, t.T, C.c.clip_k);
-  gm(t.nt, t.T, D, t.q, (long long)g * D, false, C.Kt, D, true, C.X, t.T, 1.0, 0.0,
-     g, D, 0, nTT);
-  softmax_rows_kernel<<<(unsigned)r, 256, 0, C.st>>>(
-      C.X, C.windows ? t.Lc : nullptr, (int)r, t.nt, t.T, t.tpos, C.scale,
-      C.c.sink, C.c.recent, C.PK, t.Pref, t.logPref, C.rowv);
+  const int g = C.c.g, D = kCD;
+  const long long r = (long long)g * t.nt, nTT = (long long)t.nt * t.T, nD = (long long)t.nt * D;
+  q2_roundtrip(C, t.Kc, t.T, C.c.clip_k, nullptr);
+  gm(t.nt, t.T, D, t.qp, D, false, C.Kt, D, true, C.X, t.T, C.scale, g, nD, 0, nTT);
+  launch_pdl(&softmax_rows_kernel, dim3((unsigned)r), dim3(256), 0, C.st, C.X,
+             C.windows ? t.Lc : nullptr, t.nt, t.T, t.tpos, C.c.sink, C.c.recent, C.PK, t.Pref,
+             t.logPref, C.DP, C.rowv);
   // e_j = ((pk - p) V) W_j^T
-  sub_kernel<<<nblk(r * t.T), 256, 0, C.st>>>(C.PK, t.Pref, r * t.T, C.GV);
-  gm(t.nt, D, t.T, C.GV, t.T, false, t.V, D, false, C.DV, D, 1.0, 0.0, g, nTT, 0,
-     (long long)t.nt * D);
-  gm(t.nt, dm, D, C.DV, D, false, C.W, D, true, C.Eo, dm, 1.0, 0.0, g,
-     (long long)t.nt * D, (long long)dm * D, (long long)t.nt * dm);
-  row_sqsum_kernel<<<nwarp_blocks(r), 256, 0, C.st>>>(C.Eo, (int)r, dm, C.c.lam, 1, C.rowv);
-  loss_reduce_kernel<<<1, 1024, 0, C.st>>>(C.rowv, (int)r, (double)r, out);
+  gm(t.nt, D, t.T, C.DP, t.T, false, t.V, D, false, C.DV, D, 1.0, g, nTT, 0, nD);
+  output_error(C, t, C.c.lam, 1);
+  loss_mean(C, (int)r, out);
 }
 
-}  // namespace
-
-namespace {
+// dR = dKt^T Zh + X^T (inside * (dKt R))
+void rotation_grad(Calib& C, int T, const double* X) {
+  GemmCall gm = C.gemm();
+  const int D = kCD;
+  Gemm z = gm.args(T, D, D, C.dKt, D, false, C.R, D, false, C.dZh, D);
+  z.mul = C.inside;
+  gm.run(z, 1);
+  Gemm d = gm.args(D, D, T, C.dKt, D, true, C.Zh, D, false, C.dR, D);
+  d.A2 = X;
+  d.B2 = C.dZh;
+  gm.run(d, 1);
+}
 
 // dR of L_K (after key_forward on the same trace and rotation).
 void key_backward(Calib& C, Trace& t) {
   GemmCall gm = C.gemm();
-  const int g = C.c.g, D = kCD, dm = C.c.d_model;
+  const int g = C.c.g, D = kCD;
   const long long r = (long long)g * t.nt, nTT = (long long)t.nt * t.T;
-  // U_j = (2 lambda / d_model) e_j W_j;  GV_j = U_j V^T
-  gm(t.nt, D, dm, C.Eo, dm, false, C.W, D, false, C.U, D, 2.0 * C.c.lam / dm, 0.0, g,
-     (long long)t.nt * dm, (long long)dm * D, (long long)t.nt * D);
-  gm(t.nt, t.T, D, C.U, D, false, t.V, D, true, C.GV, t.T, 1.0, 0.0, g,
+  // GV_j = (2 lambda / d_model) U0_j V^T
+  output_grad(C, t);
+  gm(t.nt, t.T, D, C.U, D, false, t.V, D, true, C.GV, t.T, 2.0 * C.c.lam / C.c.d_model, g,
      (long long)t.nt * D, 0, nTT);
-  key_row_grad_kernel<<<nwarp_blocks(r), 256, 0, C.st>>>(
-      C.PK, t.Pref, C.GV, (int)r, t.nt, t.T, t.tpos, C.scale / (double)r, C.c.sink,
-      C.c.recent, C.windows);
+  launch_pdl(&key_row_grad_kernel, dim3((unsigned)r), dim3(256), 0, C.st, C.PK, C.DP, C.GV, t.nt,
+             t.T, t.tpos, C.scale / (double)r, C.c.sink, C.c.recent, C.windows);
   // dKt = sum_j dl_j^T q_j
-  for (int j = 0; j < g; ++j)
-    gm(t.T, D, t.nt, C.GV + j * nTT, t.T, true, t.q + j * D, (long long)g * D, false,
-       C.dKt, D, 1.0, j ? 1.0 : 0.0);
-  // dR = dKt^T Zh + Kc^T (inside * (dKt R))
-  gm(t.T, D, D, C.dKt, D, false, C.R, D, false, C.dZh, D);
-  gm(D, D, t.T, C.dKt, D, true, C.Zh, D, false, C.dR, D);
-  mask_mul_kernel<<<nblk((long long)t.T * D), 256, 0, C.st>>>(C.dZh, C.inside,
-                                                             (long long)t.T * D);
-  gm(D, D, t.T, t.Kc, D, true, C.dZh, D, false, C.dR, D, 1.0, 1.0);
+  gm(t.T, D, (int)r, C.GV, t.T, true, t.qp, D, false, C.dKt, D);
+  rotation_grad(C, t.T, t.Kc);
 }
 
 // Phat of trace t: the key-phase attention under C.R (the selected R_K),
@@ -1202,35 +1392,23 @@ void value_setup(Calib& C, Trace& t) {
 
 // L_V of trace t under C.R (the value rotation) into *out.
 void value_forward(Calib& C, Trace& t, double* out) {
-  GemmCall gm = C.gemm();
-  const int g = C.c.g, D = kCD, dm = C.c.d_model;
+  const int g = C.c.g, D = kCD;
   const long long r = (long long)g * t.nt, nTT = (long long)t.nt * t.T;
-  q2_roundtrip(C, t.V, t.T, C.c.clip_v);
-  sub_kernel<<<nblk((long long)t.T * D), 256, 0, C.st>>>(C.Kt, t.V, (long long)t.T * D,
-                                                        C.Kt);
-  gm(t.nt, D, t.T, t.Phat, t.T, false, C.Kt, D, false, C.DV, D, 1.0, 0.0, g, nTT, 0,
-     (long long)t.nt * D);
-  gm(t.nt, dm, D, C.DV, D, false, C.W, D, true, C.Eo, dm, 1.0, 0.0, g,
-     (long long)t.nt * D, (long long)dm * D, (long long)t.nt * dm);
-  row_sqsum_kernel<<<nwarp_blocks(r), 256, 0, C.st>>>(C.Eo, (int)r, dm, 1.0, 0, C.rowv);
-  loss_reduce_kernel<<<1, 1024, 0, C.st>>>(C.rowv, (int)r, (double)r, out);
+  q2_roundtrip(C, t.V, t.T, C.c.clip_v, t.V);
+  C.gemm()(t.nt, D, t.T, t.Phat, t.T, false, C.Kt, D, false, C.DV, D, 1.0, g, nTT, 0,
+           (long long)t.nt * D);
+  output_error(C, t, 1.0, 0);
+  loss_mean(C, (int)r, out);
 }
 
 // dR of L_V (after value_forward on the same trace and rotation).
 void value_backward(Calib& C, Trace& t) {
-  GemmCall gm = C.gemm();
-  const int g = C.c.g, D = kCD, dm = C.c.d_model;
-  const long long r = (long long)g * t.nt, nTT = (long long)t.nt * t.T;
-  gm(t.nt, D, dm, C.Eo, dm, false, C.W, D, false, C.U, D, 2.0 / ((double)dm * r), 0.0,
-     g, (long long)t.nt * dm, (long long)dm * D, (long long)t.nt * D);
-  for (int j = 0; j < g; ++j)
-    gm(t.T, D, t.nt, t.Phat + j * nTT, t.T, true, C.U + (long long)j * t.nt * D, D,
-       false, C.dKt, D, 1.0, j ? 1.0 : 0.0);
-  gm(t.T, D, D, C.dKt, D, false, C.R, D, false, C.dZh, D);
-  gm(D, D, t.T, C.dKt, D, true, C.Zh, D, false, C.dR, D);
-  mask_mul_kernel<<<nblk((long long)t.T * D), 256, 0, C.st>>>(C.dZh, C.inside,
-                                                             (long long)t.T * D);
-  gm(D, D, t.T, t.V, D, true, C.dZh, D, false, C.dR, D, 1.0, 1.0);
+  const int D = kCD;
+  const long long r = (long long)C.c.g * t.nt;
+  output_grad(C, t);
+  C.gemm()(t.T, D, (int)r, t.Phat, t.T, true, C.U, D, false, C.dKt, D,
+           2.0 / ((double)C.c.d_model * r));
+  rotation_grad(C, t.T, t.V);
 }
 
 // One Adam run of the appendix algorithm on generator A (from 0) for the
@@ -1297,7 +1475,10 @@ bool calib_init(Calib& C, const optr_calib_config* c, void* ws, const double* W_
   const struct {
     const void* kernel;
     size_t bytes;
-  } need[] = {{reinterpret_cast<const void*>(&gemm_digits_kernel), sizeof(GemmSmem)},
+  } need[] = {{reinterpret_cast<const void*>(&gemm_digits_kernel<64, 32>),
+               sizeof(GemmTile<64, 32>)},
+              {reinterpret_cast<const void*>(&gemm_digits_kernel<32, 16>),
+               sizeof(GemmTile<32, 16>)},
               {reinterpret_cast<const void*>(&mat_product_kernel<1>), sizeof(MatHalf)},
               {reinterpret_cast<const void*>(&mat_product_kernel<2>), 2 * sizeof(MatHalf)}};
   for (const auto& k : need)
@@ -1355,7 +1536,7 @@ extern "C" optr_status optr_calibrate_head(
   if (cudaMemsetAsync(C.err, 0, sizeof(unsigned), stream) != cudaSuccess ||
       cudaMemsetAsync(C.gcnt, 0, sizeof(int) * kGemmTiles, stream) != cudaSuccess)
     return OPTR_ERR_CUDA;
-  col_mean_kernel<<<1, kCD, 0, stream>>>(K, c->T, mu);
+  col_mean_kernel<<<kCD / 4, 256, 0, stream>>>(K, c->T, mu);
   const double* r0[2] = {R0_K, R0_V};
   for (int k = 0; k < 2; ++k) {
     if (r0[k]) copy_kernel<<<nblk(n), 256, 0, stream>>>(r0[k], n, C.R0[k]);
@@ -1371,6 +1552,7 @@ extern "C" optr_status optr_calibrate_head(
   } else {
     C.tr[1] = C.tr[0];
   }
+  output_setup(C);
   adam_run(C, 0, C.R0[0], hist_k);
   copy_kernel<<<nblk(n), 256, 0, stream>>>(C.best, n, R_K);
   copy_kernel<<<nblk(n), 256, 0, stream>>>(C.best, n, C.R);
@@ -1402,6 +1584,7 @@ extern "C" optr_status optr_calib_loss_grad(
   C.tr[0].q = q; C.tr[0].K = K; C.tr[0].V = V; C.tr[0].tpos = t_pos;
   C.tr[0].T = c->T; C.tr[0].nt = c->nt;
   trace_setup(C, C.tr[0], mu);
+  C.M = nullptr;
   if (which == 1) {
     copy_kernel<<<nblk(n), 256, 0, stream>>>(R_K, n, C.R);
     value_setup(C, C.tr[0]);

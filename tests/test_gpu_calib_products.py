@@ -78,3 +78,24 @@ def test_products_at_tile_edges(which, T, nt, g, d_model, ks, vs, ws):
 def test_non_finite_input_does_not_give_a_finite_loss(which, bad):
     loss, _, _, _ = _run(which, 100, 20, 2, 40, bad=bad)
     assert loss != loss or abs(loss) == float("inf")
+
+
+@pytest.mark.parametrize("T,nt,d_model,steps,group", [
+    (97, 16, 160, 5, 32),    # W^T W replaces W; odd token count
+    (97, 16, 128, 5, 128),
+    (130, 9, 127, 6, 32),    # too few output channels for it
+    (64, 4, 300, 4, 128),    # too few query rows for it
+])
+def test_calibration_with_and_without_output_products(T, nt, d_model, steps, group):
+    q, K, V, W_O, t_pos = synth.calib_trace(8, T=T, nt=nt, g=2, d_model=d_model)
+    ref = cal.calibrate_head(q, K, V, W_O, t_pos.long(), steps=steps, lr=0.01, group=group,
+                             select_every=2)
+    cfg = optr.calib_config(2, d_model, T, nt, steps=steps, select_every=2, group=group, lr=0.01)
+    got = optr.optr_calibrate_head(cfg, *[x.cuda() for x in (q, K, V, t_pos, W_O)])
+    R_K, R_V, mu, hk, hv = [torch.as_tensor(x, dtype=F64) for x in ref]
+    gR_K, gR_V, gmu, ghk, ghv = [x.cpu() for x in got]
+    assert float((gmu - mu).abs().max()) <= 1e-12 * float(mu.abs().max())
+    assert float(((ghk - hk) / hk).abs().max()) <= REL
+    assert float(((ghv - hv) / hv).abs().max()) <= REL
+    assert float((gR_K - R_K).abs().max()) <= REL
+    assert float((gR_V - R_V).abs().max()) <= REL
