@@ -38,9 +38,11 @@
 #include "f32x2.cuh"
 #include "quant.cuh"
 #include "tc05.cuh"
+#include "window.cuh"
 
 #include <cudaTypedefs.h>
 #include <mutex>
+#include <type_traits>
 
 namespace optr {
 
@@ -195,10 +197,12 @@ __device__ __forceinline__ void minmax32(const float (&x)[32], float& lo, float&
   hi = fmaxf(fmaxf(h[0], h[1]), fmaxf(h[2], h[3]));
 }
 
-template <bool kClamp, bool kG128>
+template <bool kClamp, bool kG128, bool kWin>
 __global__ void __launch_bounds__(kThreads, 1)
 append_tc05_kernel(const __grid_constant__ CUtensorMap tmap_k,
-                   const __grid_constant__ CUtensorMap tmap_v, int n_tok,
+                   const __grid_constant__ CUtensorMap tmap_v,
+                   const __nv_bfloat16* __restrict__ k_in,
+                   const __nv_bfloat16* __restrict__ v_in, int n_tok,
                    const int32_t* __restrict__ cu_new,
                    const int32_t* __restrict__ pos0,
                    const int32_t* __restrict__ bt, int B, int max_pages,
@@ -206,10 +210,19 @@ append_tc05_kernel(const __grid_constant__ CUtensorMap tmap_k,
                    const uint16_t* __restrict__ Rk_t5,
                    const uint16_t* __restrict__ Rv_t5,
                    const float* __restrict__ muR, float clip_k, float clip_v,
-                   unsigned* err) {
+                   int copies, WinArgs win, int sink, int recent, unsigned* err) {
   extern __shared__ __align__(1024) unsigned char dsm_[];
   Smem& S = *reinterpret_cast<Smem*>(dsm_);
   const int h = blockIdx.y, kind = blockIdx.z;
+  if (kWin && kind > 1) {  // window rows, `copies` CTAs
+    const int part = ((kind - 2) * h_kv + h) * gridDim.x + blockIdx.x;
+    if (part < copies)
+      window_rows_body(part, copies, kThreads / 32, k_in, v_in, n_tok, cu_new, pos0, B, win, h_kv,
+                       sink, recent, err);
+    else
+      pdl_wait();
+    return;
+  }
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int tiles = (n_tok + kRows - 1) / kRows;
   const int my_tiles = tiles > (int)blockIdx.x
@@ -568,11 +581,19 @@ cudaError_t launch_append_tc05(const optr_params* p, const __nv_bfloat16* k,
                                const __nv_bfloat16* v, int n_tok,
                                const int32_t* cu_new, const int32_t* pos0,
                                const int32_t* bt, int B, int max_pages,
-                               uint8_t* pool, int num_pages, cudaStream_t s) {
+                               uint8_t* pool, int num_pages, const WinArgs* win,
+                               cudaStream_t s) {
   const bool clamp = !(p->cfg.clip_k == 1.0f && p->cfg.clip_v == 1.0f);
   const bool g128 = p->cfg.group == 4 * kG;
-  auto fn = clamp ? (g128 ? append_tc05_kernel<true, true> : append_tc05_kernel<true, false>)
-                  : (g128 ? append_tc05_kernel<false, true> : append_tc05_kernel<false, false>);
+  // without windows the kernel is compiled without the copy: with it in, 4 x 32k
+  // tokens take 151.0 us, else 148.9
+  auto pick = [&](auto w) {
+    constexpr bool W = decltype(w)::value;
+    return clamp ? (g128 ? append_tc05_kernel<true, true, W> : append_tc05_kernel<true, false, W>)
+                 : (g128 ? append_tc05_kernel<false, true, W>
+                         : append_tc05_kernel<false, false, W>);
+  };
+  auto fn = win ? pick(std::true_type{}) : pick(std::false_type{});
   cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(fn), sizeof(Smem));
   if (e != cudaSuccess) return e;
   const int h_kv = p->cfg.h_kv;
@@ -584,11 +605,20 @@ cudaError_t launch_append_tc05(const optr_params* p, const __nv_bfloat16* k,
   // memory is never contended), spread over the (head, kind) pairs
   int per = max(1, p->num_sms / (2 * h_kv));
   per = min(per, tiles);
-  dim3 grid(per, h_kv, 2);
+  // Window rows: CTAs of this launch, 72 rows each, last in the grid: the SMs
+  // that the (head, kind) pairs leave over take them while the others convert
+  // (8 KV heads leave 8 of 152).  A copy of its own after this launch read every
+  // token to find the window's: 2000 tokens of one sequence (8 KV heads, 320 window
+  // rows) 18.0 us a call, now 8.5.
+  const long long rows = win ? (long long)B * (p->cfg.sink + p->cfg.recent) : 0;
+  constexpr int kRowsPerCta = kThreads / 32 * 4;
+  const int copies = (int)((rows + kRowsPerCta - 1) / kRowsPerCta);
+  dim3 grid(per, h_kv, 2 + (copies + per * h_kv - 1) / (per * h_kv));
   return launch_pdl(fn, grid, dim3(kThreads), sizeof(Smem), s,
-                    mk, mv, n_tok, cu_new, pos0, bt, B, max_pages, pool, num_pages,
+                    mk, mv, k, v, n_tok, cu_new, pos0, bt, B, max_pages, pool, num_pages,
                     h_kv, (const uint16_t*)p->Rk_t5, (const uint16_t*)p->Rv_t5,
-                    (const float*)p->muR, p->cfg.clip_k, p->cfg.clip_v, p->err);
+                    (const float*)p->muR, p->cfg.clip_k, p->cfg.clip_v,
+                    copies, win ? *win : WinArgs{}, p->cfg.sink, p->cfg.recent, p->err);
 }
 
 }  // namespace optr

@@ -404,11 +404,16 @@ optr_status optr_kv_append_win(const optr_params* p, const void* k,
                                 (const __nv_bfloat16*)v, n_tok, cu_new, pos0,
                                 block_table, B, max_pages, pool, num_pages,
                                 stream);
-  else
+  else {
+    // window rows found from the windows when those hold no more rows than
+    // the call writes tokens, else from the tokens after this launch
+    const bool fused = wa && (long long)B * (p->cfg.sink + p->cfg.recent) <= n_tok;
     e = launch_append_tc05(p, (const __nv_bfloat16*)k,
                              (const __nv_bfloat16*)v, n_tok, cu_new, pos0,
                              block_table, B, max_pages, pool, num_pages,
-                             stream);
+                             fused ? wa : nullptr, stream);
+    if (fused) wa = nullptr;
+  }
   prof_mark(p, 1, stream);
   if (e == cudaSuccess && wa)
     e = launch_window_copy(p, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v,

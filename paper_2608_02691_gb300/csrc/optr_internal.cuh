@@ -207,7 +207,8 @@ cudaError_t launch_append_tc05(const optr_params* p, const __nv_bfloat16* k,
                                const __nv_bfloat16* v, int n_tok,
                                const int32_t* cu_new, const int32_t* pos0,
                                const int32_t* bt, int B, int max_pages,
-                               uint8_t* pool, int num_pages, cudaStream_t s);
+                               uint8_t* pool, int num_pages, const WinArgs* win,
+                               cudaStream_t s);
 // The decode step's single-token cache write, fused into the decode's first
 // launch (optr_decode_step); null for a decode alone.
 struct StepAppend {
@@ -231,7 +232,8 @@ cudaError_t launch_decode(const optr_params* p, int variant,
 cudaError_t decode_one_limits(const optr_params* p, int (&clusters)[4]);
 
 // Window part of a cache write (positions of the BF16 windows copied into
-// the store); a separate launch after the INT2 write.
+// the store); a separate launch after the INT2 write, where that has not
+// written the windows itself (launch_append_tc05 with win).
 cudaError_t launch_window_copy(const optr_params* p, const __nv_bfloat16* k,
                                const __nv_bfloat16* v, int n_tok,
                                const int32_t* cu_new, const int32_t* pos0,

@@ -2,7 +2,8 @@
 // BF16 window; Sec. 4.1: sink and recent tokens stay in BF16, their keys
 // centered by the same mu; Sec. 5: 64 sink, 256 recent tokens).
 //
-//   window_copy_body   cache write: copy the window positions of the new
+//   window_copy_body, window_rows_body
+//                      cache write: copy the window positions of the new
 //                      tokens into the caller's window store.
 //   window_phase       decode: the softmax partials of the window positions,
 //                      one warp per run of 16-token units, before the warp's
@@ -76,6 +77,58 @@ __device__ __forceinline__ void window_copy_body(
     const __nv_bfloat16* src = (kind ? v : k) + ((size_t)tok * h_kv + hh) * kD + 8 * c;
     __nv_bfloat16* dst = win + base + (long long)(hh * 2 + kind) * rows * kD + 8 * c;
     *reinterpret_cast<uint4*>(dst) = __ldg(reinterpret_cast<const uint4*>(src));
+  }
+}
+
+// The same found from the windows' rows instead of the tokens: row j of
+// sequence b holds position j (j < sink) or the (j - sink + 1)-th last of the
+// written cache.  `warps` warps in each of `parts` CTAs, one row at a time: all
+// heads' K and V rows of its token.  For calls that write more tokens than
+// their windows hold.
+__device__ __forceinline__ void window_rows_body(
+    int part, int parts, int warps, const __nv_bfloat16* __restrict__ k,
+    const __nv_bfloat16* __restrict__ v, int n_tok, const int32_t* __restrict__ cu_new,
+    const int32_t* __restrict__ pos0, int B, const WinArgs& w, int h_kv, int sink, int recent,
+    unsigned* err) {
+  const int lane = threadIdx.x & 31, rows = sink + recent;
+  const long long n = (long long)B * rows, step = (long long)parts * warps;
+  pdl_wait();  // inputs may come from earlier kernels
+  pdl_trigger();
+  for (long long i = (long long)part * warps + (threadIdx.x >> 5); i < n; i += step) {
+    const int b = (int)(i / rows), j = (int)(i % rows);
+    const long long c0 = __ldg(cu_new + b), c1 = __ldg(cu_new + b + 1), p0 = __ldg(pos0 + b);
+    const int slot = __ldg(w.slot + b);
+    const long long end = p0 + (c1 - c0);
+    const long long s = j < sink ? j : end - 1 - (j - sink);
+    const long long tok = c0 + (s - p0);
+    // (cu_new and pos0 out of range: the INT2 write flags them)
+    if (s < 0 || (j >= sink && s < sink) || s < p0 || s >= end || tok < 0 || tok >= n_tok) continue;
+    if (slot < 0 || slot >= w.n_slots) {
+      if (lane == 0) atomicOr(err, OPTR_DEVERR_WIN_SLOT);
+      continue;
+    }
+    __nv_bfloat16* dst = w.win + (long long)slot * h_kv * 2 * rows * kD +
+                         (long long)win_row(s, sink, recent) * kD;
+    const long long t0 = tok * h_kv * kD;
+    // 16-byte pieces, head hh, kind, piece c of the 256-byte row
+    const int per_tok = 2 * h_kv * (kD / 8);
+    for (int r0 = lane; r0 < per_tok; r0 += 4 * 32) {
+      uint4 x[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int r = r0 + 32 * u, kind = r >= per_tok / 2;
+        if (r < per_tok)
+          x[u] = __ldg(reinterpret_cast<const uint4*>((kind ? v : k) + t0) +
+                       (r - kind * (per_tok / 2)));
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int r = r0 + 32 * u, kind = r >= per_tok / 2, q = r - kind * (per_tok / 2);
+        if (r < per_tok)
+          *reinterpret_cast<uint4*>(dst + (long long)(q / (kD / 8) * 2 + kind) * rows * kD +
+                                    8 * (q % (kD / 8))) = x[u];
+      }
+    }
   }
 }
 
