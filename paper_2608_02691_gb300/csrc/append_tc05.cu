@@ -15,23 +15,32 @@
 //                   tensor copies (channels 0-63 and 64-127, 128-byte
 //                   swizzle) into a shared-memory stage (4 stages in
 //                   flight);
-//   16 epilogue warps, two groups of 8 taking alternate tiles: two threads
-//                   own token row t, one per half of the channels; each
-//                   converts its half row to f16 and stores it to tensor
-//                   memory as the MMA's A operand, then reads its half of
-//                   the accumulator row back and quantizes and packs its two
-//                   channel groups; the pair's code bytes meet in shared
-//                   memory and the first thread writes the 32 code bytes,
-//                   each thread its 8 scale/min bytes.  A group converts its
-//                   next tile while the tensor core works on the current one
-//                   (two A buffers per group);
+//   8 converter warps  two threads own token row t, one per half of the
+//                   channels: f16 into tensor memory, as the MMA's A operand
+//                   (four buffers); the first half's also find the place of
+//                   the row's record, its table entry requested a tile ahead;
 //   MMA warp        one thread issues the 16 tcgen05.mma of a tile (8
 //                   K-steps x {R hi, R lo}) from tensor-memory A and
 //                   shared-memory B (R, 64 KB, loaded once) into the
-//                   group's tensor-memory accumulator.
-// Tensor memory (512 columns): per epilogue group g an accumulator D[g]
-// (128 columns, at 128 g) and two A operands (64 columns each, at
-// 256 + 128 g + 64 b).
+//                   accumulator of the tile's epilogue group;
+//   16 epilogue warps, two groups of 8 taking alternate tiles: again two
+//                   threads per row; each reads its half of the accumulator
+//                   row back, 32 columns at a time, and quantizes and packs
+//                   its two channel groups; the pair's code bytes meet in
+//                   shared memory and the first thread writes the 32 code
+//                   bytes, each thread its 8 scale/min bytes.
+// Tensor memory (512 columns): an accumulator D[g] per epilogue group g (128
+// columns, at 128 g) and the A operands (64 columns each, at 256 + 64 b).
+//
+// What bounds it: issue slots (66% used, the rest fixed-latency and memory
+// stalls), with DRAM 60% and the tensor pipe 50% busy.  The epilogue warps used
+// to convert their own next tile: 18 warps of 96 registers, each stalled most of
+// the time, and a tile's conversion and quantization one after the other.  As
+// warps of their own, with the record places found once per row instead of twice,
+// 26 warps of 72 registers overlap them: 4 x 32768 tokens, 8 KV heads (637 MB)
+// 147.7 -> 139.8 us, 4.6 TB/s.  Four converter warps (whole rows, 80 registers)
+// were themselves busy all the time: 140.7 us, and 9.4 instead of 8.3 us for
+// 2000 tokens.
 // The quantizer is quant.cuh's float32 formula.
 #include "append_common.cuh"
 #include "decode_common.cuh"
@@ -79,10 +88,17 @@ constexpr int kStages = 4;        // tiles in flight from global memory
 constexpr uint32_t kStageBytes = kRows * kD * 2;  // two 16 KB TMA boxes
 constexpr int kEpiWarps = 16;     // two groups of 8
 constexpr int kGroupThreads = 256;
-constexpr int kThreads = (kEpiWarps + 2) * 32;
-constexpr int kProducerWarp = kEpiWarps, kMmaWarp = kEpiWarps + 1;
+constexpr int kConvWarps = 8;     // lane quarter x channel half
+constexpr int kThreads = (kEpiWarps + kConvWarps + 2) * 32;
+constexpr int kConvWarp = kEpiWarps;  // first converter warp (a multiple of 4)
+constexpr int kProducerWarp = kConvWarp + kConvWarps, kMmaWarp = kProducerWarp + 1;
 constexpr uint32_t kTmemCols = 512;
-constexpr uint32_t kColD0 = 0, kColA0 = 256;  // D[g] at 128 g, A[g][b] at 256 + 128 g + 64 b
+constexpr int kABufs = 4;         // A operands in tensor memory
+// Tiles whose record places are in flight.  Entry i % 8 is written again for
+// tile i + 8 once MMA i + 4 is done, which was issued after every epilogue
+// thread had read the accumulator of tile i + 2, i.e. had finished tile i.
+constexpr int kRing = 8;
+constexpr uint32_t kColD0 = 0, kColA0 = 256;  // D[g] at 128 g, A[b] at 256 + 64 b
 constexpr uint32_t kIdesc = tc05::idesc_f16(128, 128);
 
 struct Smem {
@@ -96,7 +112,8 @@ struct Smem {
   uint4 xchg[2][kRows][2];               // second-half code words per row
   // G = 128: each half row's (min, max), per tile group, tile parity, half
   float2 mmx[2][2][2 * kRows];
-  uint64_t full[kStages], empty[kStages], aready[2][2], dready[2], dfree[2];
+  int2 place[kRing][kRows];  // each row's (page * h_kv + h or -1, slot)
+  uint64_t full[kStages], empty[kStages], aready[kRing], aempty[kABufs], dready[2], dfree[2];
   uint64_t xready[2], xdone[2];  // the exchange slot of group g written / read
   uint64_t rready[2];            // G = 128: both halves' ranges of the tile written
   uint32_t tmem;
@@ -242,11 +259,11 @@ append_tc05_kernel(const __grid_constant__ CUtensorMap tmap_k,
   if (tid == 0) {
     for (int s = 0; s < kStages; ++s) {
       tc05::bar_init(&S.full[s], 1);
-      tc05::bar_init(&S.empty[s], kGroupThreads);
+      tc05::bar_init(&S.empty[s], kConvWarps * 32);
     }
+    for (int i = 0; i < kRing; ++i) tc05::bar_init(&S.aready[i], kConvWarps * 32);
+    for (int b = 0; b < kABufs; ++b) tc05::bar_init(&S.aempty[b], 1);
     for (int g = 0; g < 2; ++g) {
-      tc05::bar_init(&S.aready[g][0], kGroupThreads);
-      tc05::bar_init(&S.aready[g][1], kGroupThreads);
       tc05::bar_init(&S.dready[g], 1);
       tc05::bar_init(&S.dfree[g], kGroupThreads);
       tc05::bar_init(&S.xready[g], kGroupThreads / 2);
@@ -301,14 +318,13 @@ append_tc05_kernel(const __grid_constant__ CUtensorMap tmap_k,
     if (lane == 0) {
       const uint32_t b0 = tc05::smem_addr(&S.b[0][0]);
       for (int i = 0; i < my_tiles; ++i) {
-        // tile i is the k-th of group g, its A operand in buffer k % 2; the
-        // group's previous tile must have been read out of D[g]
-        const int g = i & 1, k = i >> 1;
-        if (!tc05::bar_wait(&S.aready[g][k & 1], (k >> 1) & 1, abort)) break;
+        // tile i is the k-th of group g; the group's previous tile must
+        // have been read out of D[g]
+        const int g = i & 1, k = i >> 1, b = i % kABufs;
+        if (!tc05::bar_wait(&S.aready[i % kRing], (i / kRing) & 1, abort)) break;
         if (k > 0 && !tc05::bar_wait(&S.dfree[g], (k - 1) & 1, abort)) break;
         tc05::fence_after();
-        const uint32_t d = tmem + kColD0 + 128u * g,
-                       a = tmem + kColA0 + 128u * g + 64u * (k & 1);
+        const uint32_t d = tmem + kColD0 + 128u * g, a = tmem + kColA0 + 64u * b;
 #pragma unroll
         for (int ks = 0; ks < 8; ++ks)
 #pragma unroll
@@ -317,12 +333,94 @@ append_tc05_kernel(const __grid_constant__ CUtensorMap tmap_k,
                          tc05::smem_desc(b0 + term * kD * kD * 2 + ks * 256, 128, 2048),
                          kIdesc, (ks | term) != 0);
         tc05::mma_commit(&S.dready[g]);
+        tc05::mma_commit(&S.aempty[b]);
         last = i;
       }
       // the tensor core must be done with tensor memory before it is freed
-      if (last >= 0) tc05::bar_wait_drain(&S.dready[last & 1], (last >> 1) & 1);
+      if (last >= 0) {
+        tc05::bar_wait_drain(&S.dready[last & 1], (last >> 1) & 1);
+        tc05::bar_wait_drain(&S.aempty[last % kABufs], (last / kABufs) & 1);
+      }
     }
     __syncwarp();
+  } else if (warp >= kConvWarp) {
+    // -------------------------------------------------------- converters
+    // thread = half a token row: its 64 channels as f16 into A buffer i % 4
+    // (columns j <-> channels 2j, 2j+1); the first half's thread finds the
+    // place of the row's record
+    const int q = warp & 3, hp = (warp - kConvWarp) >> 2, row = 32 * q + lane;
+    const uint32_t tA0 = tmem + ((uint32_t)(32 * q) << 16) + kColA0 + 32u * hp;
+    const int* cu = cached ? S.cu : cu_new;
+    const int* p0 = cached ? S.p0 : pos0;
+    // resolve_slot() in two halves: the block-table entry is requested a tile
+    // ahead and checked when it is needed
+    int page = -1, slot = 0;
+    unsigned bad = 0;
+    auto request = [&](int tok) {
+      page = -1;
+      slot = 0;
+      bad = 0;
+      if (hp == 0 && tok < n_tok) {
+        int lo = 0, hi = B;
+        while (hi - lo > 1) {
+          const int mid = (lo + hi) >> 1;
+          if (cu[mid] <= tok) lo = mid; else hi = mid;
+        }
+        const int c0 = cu[lo], c1 = cu[lo + 1];
+        const long long pos = (long long)p0[lo] + (tok - c0);
+        if (!(c0 <= tok && tok < c1)) {
+          bad = OPTR_DEVERR_CU_NEW;
+        } else if (pos < 0 || pos >= (long long)max_pages * kPage) {
+          bad = OPTR_DEVERR_POSITION;
+        } else {
+          slot = (int)(pos % kPage);
+          page = __ldg(bt + (size_t)lo * max_pages + pos / kPage);
+        }
+      }
+      __syncwarp();
+    };
+    request((int)blockIdx.x * kRows + row);
+    for (int i = 0; i < my_tiles; ++i) {
+      const int s = i % kStages, b = i % kABufs;
+      const int tok = ((int)blockIdx.x + i * (int)gridDim.x) * kRows + row;
+      if (!__all_sync(0xffffffffu, tc05::bar_wait(&S.full[s], (i / kStages) & 1, abort))) break;
+      if (i >= kABufs) {
+        if (!__all_sync(0xffffffffu, tc05::bar_wait(&S.aempty[b], ((i / kABufs) - 1) & 1, abort)))
+          break;
+        tc05::fence_after();
+      }
+      {
+        const uint8_t* rb = S.stage[s] + hp * (kStageBytes / 2) + row * 128;
+        uint32_t a[32];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const uint4 x = *reinterpret_cast<const uint4*>(rb + ((c ^ (row & 7)) << 4));
+          a[4 * c + 0] = bf16x2_to_f16x2(x.x);
+          a[4 * c + 1] = bf16x2_to_f16x2(x.y);
+          a[4 * c + 2] = bf16x2_to_f16x2(x.z);
+          a[4 * c + 3] = bf16x2_to_f16x2(x.w);
+        }
+        tc05::tmem_st32(tA0 + 64u * b, a);
+      }
+      tc05::bar_arrive(&S.empty[s]);  // stage s read (values in registers)
+      if (hp == 0) {
+        int unit = -1;
+        if (tok < n_tok) {
+          if (bad)
+            atomicOr(err, bad);
+          else if (page < 0 || page >= num_pages)
+            atomicOr(err, OPTR_DEVERR_PAGE_ID);
+          else
+            unit = page * h_kv + h;
+        }
+        S.place[i % kRing][row] = make_int2(unit, slot);
+      }
+      __syncwarp();
+      tc05::tmem_wait_st();
+      tc05::fence_before();
+      tc05::bar_arrive(&S.aready[i % kRing]);
+      if (i + 1 < my_tiles) request(tok + (int)gridDim.x * kRows);
+    }
   } else {
     // ---------------------------------------------------------- epilogue
     // warp w: group g = w / 8; lane quarter q = w % 4 (its tensor-memory
@@ -335,60 +433,13 @@ append_tc05_kernel(const __grid_constant__ CUtensorMap tmap_k,
     const uint32_t lane_base = (uint32_t)(32 * q) << 16;
     const uint32_t tD = tmem + lane_base + kColD0 + 128u * g;
     const int n_mine = my_tiles > g ? (my_tiles - 1 - g) / 2 + 1 : 0;
-    auto token = [&](int k) {
-      return ((int)blockIdx.x + (g + 2 * k) * (int)gridDim.x) * kRows + row;
-    };
-    // destination of this row's record in the group's k-th tile (the
-    // block-table load completes during the conversion and the MMA)
-    auto resolve = [&](int k, int& slot) -> long long {
-      const int tok = token(k);
-      long long d = -1;
-      if (tok < n_tok)
-        d = cached ? resolve_slot_cached(tok, h, S.cu, S.p0, bt, B, max_pages,
-                                         num_pages, h_kv, &slot, err, chunk_bytes(kG128))
-                   : resolve_slot(tok, h, cu_new, pos0, bt, B, max_pages,
-                                  num_pages, h_kv, &slot, err, chunk_bytes(kG128));
-      __syncwarp();  // converged for the warp-wide tensor-memory accesses
-      return d;
-    };
-    // the row of the group's k-th tile as f16 into A buffer k % 2:
-    // columns j <-> channels 2j, 2j+1
-    auto convert = [&](int k) -> bool {
-      const int i = g + 2 * k, s = i % kStages;
-      if (!__all_sync(0xffffffffu, tc05::bar_wait(&S.full[s], (i / kStages) & 1, abort)))
-        return false;
-      const uint32_t tA = tmem + lane_base + kColA0 + 128u * g + 64u * (k & 1) + 32u * hp;
-      {
-        const uint8_t* rb = S.stage[s] + hp * (kStageBytes / 2) + row * 128;
-        uint32_t a[32];
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          const uint4 x = *reinterpret_cast<const uint4*>(rb + ((c ^ (row & 7)) << 4));
-          a[4 * c + 0] = bf16x2_to_f16x2(x.x);
-          a[4 * c + 1] = bf16x2_to_f16x2(x.y);
-          a[4 * c + 2] = bf16x2_to_f16x2(x.z);
-          a[4 * c + 3] = bf16x2_to_f16x2(x.w);
-        }
-        tc05::tmem_st32(tA, a);
-      }
-      tc05::bar_arrive(&S.empty[s]);  // stage s read (values in registers)
-      tc05::tmem_wait_st();
-      tc05::fence_before();
-      tc05::bar_arrive(&S.aready[g][k & 1]);
-      return true;
-    };
-
-    int slot_next = 0;
-    long long dst_next = n_mine > 0 ? resolve(0, slot_next) : -1;
-    bool ok = n_mine == 0 || convert(0);
-    for (int k = 0; ok && k < n_mine; ++k) {
-      const long long dst = dst_next;
-      const int slot = slot_next;
-      const int tok = token(k);
-      if (k + 1 < n_mine) {
-        dst_next = resolve(k + 1, slot_next);
-        if (!convert(k + 1)) break;
-      }
+    for (int k = 0; k < n_mine; ++k) {
+      const int i = g + 2 * k;
+      // the converters' places of the tile's records
+      if (!__all_sync(0xffffffffu,
+                      tc05::bar_wait(&S.aready[i % kRing], (i / kRing) & 1, abort)))
+        break;
+      const int2 place = S.place[i % kRing][row];
       if (!__all_sync(0xffffffffu, tc05::bar_wait(&S.dready[g], k & 1, abort))) break;
       tc05::fence_after();
 
@@ -397,14 +448,6 @@ append_tc05_kernel(const __grid_constant__ CUtensorMap tmap_k,
       bool range_err = false;
       {
         const int G2 = 2 * hp;  // this thread's two channel groups
-        uint32_t acc[2][32];
-        tc05::tmem_ld32(tD + 32u * G2, acc[0]);
-        tc05::tmem_ld32(tD + 32u * (G2 + 1), acc[1]);
-        tc05::tmem_wait_ld();
-        if constexpr (!kG128) {
-          tc05::fence_before();
-          tc05::bar_arrive(&S.dfree[g]);  // D[g] read: the next MMA may start
-        }
         uint32_t bytes[2][8];
         const float xs = kind ? 64.0f : 1.0f;  // x = xs * z
         // x = z = acc / 64 - mu R (keys; acc / 64 is exact, so one
@@ -453,14 +496,16 @@ append_tc05_kernel(const __grid_constant__ CUtensorMap tmap_k,
           // exchange, so no registers hold it meanwhile; D[g] is released
           // after that second read)
           float lo, hi;
-          {
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            uint32_t acc[32];
+            tc05::tmem_ld32(tD + 32u * (G2 + e), acc);
+            tc05::tmem_wait_ld();
             float x[32], l1, h1;
-            row_values(0, acc[0], x);
-            minmax32(x, lo, hi);
-            row_values(1, acc[1], x);
+            row_values(e, acc, x);
             minmax32(x, l1, h1);
-            lo = fminf(lo, l1);
-            hi = fmaxf(hi, h1);
+            lo = e ? fminf(lo, l1) : l1;
+            hi = e ? fmaxf(hi, h1) : h1;
           }
           float2* mm = S.mmx[g][k & 1];
           mm[hp * kRows + row] = make_float2(lo, hi);
@@ -483,8 +528,15 @@ append_tc05_kernel(const __grid_constant__ CUtensorMap tmap_k,
         } else {
 #pragma unroll
           for (int e = 0; e < 2; ++e) {
+            uint32_t acc[32];
+            tc05::tmem_ld32(tD + 32u * (G2 + e), acc);
+            tc05::tmem_wait_ld();
+            if (e == 1) {
+              tc05::fence_before();
+              tc05::bar_arrive(&S.dfree[g]);  // D[g] read: the next MMA may start
+            }
             float x[32];
-            row_values(e, acc[e], x);
+            row_values(e, acc, x);
             float lo, hi;
             minmax32(x, lo, hi);
             const FastQuant q = scaled_params(lo, hi);
@@ -498,7 +550,8 @@ append_tc05_kernel(const __grid_constant__ CUtensorMap tmap_k,
 #pragma unroll
         for (int w = 0; w < 8; ++w) word[w] = __byte_perm(bytes[0][w], bytes[1][w], sel);
       }
-      if (range_err && tok < n_tok) atomicOr(err, OPTR_DEVERR_FP16_RANGE);
+      if (range_err && ((int)blockIdx.x + i * (int)gridDim.x) * kRows + row < n_tok)
+        atomicOr(err, OPTR_DEVERR_FP16_RANGE);
       // the second half's code bytes to its partner, through shared memory
       uint4* xw = S.xchg[g][row];
       if (hp) {
@@ -515,8 +568,9 @@ append_tc05_kernel(const __grid_constant__ CUtensorMap tmap_k,
         word[0] |= y0.x; word[1] |= y0.y; word[2] |= y0.z; word[3] |= y0.w;
         word[4] |= y1.x; word[5] |= y1.y; word[6] |= y1.z; word[7] |= y1.w;
       }
-      if (dst >= 0) {
-        uint8_t* rec = pool + dst;
+      if (place.x >= 0) {
+        uint8_t* rec = pool + (size_t)place.x * chunk_bytes(kG128);
+        const int slot = place.y;
         if (!hp) {
           *reinterpret_cast<uint4*>(rec + codes_off + slot * 32) =
               make_uint4(word[0], word[1], word[2], word[3]);
@@ -586,7 +640,7 @@ cudaError_t launch_append_tc05(const optr_params* p, const __nv_bfloat16* k,
   const bool clamp = !(p->cfg.clip_k == 1.0f && p->cfg.clip_v == 1.0f);
   const bool g128 = p->cfg.group == 4 * kG;
   // without windows the kernel is compiled without the copy: with it in, 4 x 32k
-  // tokens take 151.0 us, else 148.9
+  // tokens took 2 us longer
   auto pick = [&](auto w) {
     constexpr bool W = decltype(w)::value;
     return clamp ? (g128 ? append_tc05_kernel<true, true, W> : append_tc05_kernel<true, false, W>)
@@ -605,13 +659,13 @@ cudaError_t launch_append_tc05(const optr_params* p, const __nv_bfloat16* k,
   // memory is never contended), spread over the (head, kind) pairs
   int per = max(1, p->num_sms / (2 * h_kv));
   per = min(per, tiles);
-  // Window rows: CTAs of this launch, 72 rows each, last in the grid: the SMs
+  // Window rows: CTAs of this launch, 52 rows each, last in the grid: the SMs
   // that the (head, kind) pairs leave over take them while the others convert
   // (8 KV heads leave 8 of 152).  A copy of its own after this launch read every
   // token to find the window's: 2000 tokens of one sequence (8 KV heads, 320 window
-  // rows) 18.0 us a call, now 8.5.
+  // rows) 18.0 us a call, now 8.2.
   const long long rows = win ? (long long)B * (p->cfg.sink + p->cfg.recent) : 0;
-  constexpr int kRowsPerCta = kThreads / 32 * 4;
+  constexpr int kRowsPerCta = kThreads / 32 * 2;
   const int copies = (int)((rows + kRowsPerCta - 1) / kRowsPerCta);
   dim3 grid(per, h_kv, 2 + (copies + per * h_kv - 1) / (per * h_kv));
   return launch_pdl(fn, grid, dim3(kThreads), sizeof(Smem), s,
