@@ -14,7 +14,7 @@ namespace optr {
 // tokens; the slices are added in shared memory, then warp t quantizes and
 // packs token t group by group.  T = 4 for at most 64 new tokens (4x the
 // CTAs, a quarter of the FMAs per thread: the decode step's latency), else
-// 16.
+// 16; a decode step's prologue always takes 4 (its CTAs share SMs in pairs).
 constexpr int kSmallTok = 16;
 constexpr int kSmallTokFew = 4;
 constexpr int kSmallCuCache = 512;   // sequences whose cu_new / pos0 a CTA caches
@@ -32,7 +32,6 @@ struct AppendSmallSmemT {
   int s_cu[kSmallCuCache + 1];
   int s_p0[kSmallCuCache];
 };
-using AppendSmallSmem = AppendSmallSmemT<kSmallTok>;  // the larger one
 
 // CTA (tblk, h, kind) of the cache write: tokens [T*tblk, T*tblk + T),
 // KV head h, kind 0 = keys, 1 = values.  512 threads.

@@ -25,9 +25,9 @@ constexpr float kLog2e = 1.4426950408889634f;
 
 // ---------------------------------------------------------------- qrot
 
-// CTA (b, h) of the query rotation; 512 threads.
+// CTA (sequences [b0, b0 + nb), h) of the query rotation; 512 threads.
 __device__ __forceinline__ void qrot_body(
-    int b, int h, QrotSmem& sm, const __nv_bfloat16* __restrict__ q,
+    int b0, int nb, int h, QrotSmem& sm, const __nv_bfloat16* __restrict__ q,
     const float* __restrict__ R_k, int B, int h_q, int h_kv, float qscale,
     const int32_t* __restrict__ seq_lens, int max_pages,
     float* __restrict__ qf, float* __restrict__ qs, uint32_t* __restrict__ frag,
@@ -41,12 +41,14 @@ __device__ __forceinline__ void qrot_body(
   load_rotation_slice(R_k, h, rv);
   pdl_wait();  // the query, lengths and workspace may belong to earlier kernels
   pdl_trigger();
-  const size_t row = (size_t)b * h_q + 4 * h, seg = (size_t)b * h_kv + h;
-  rotate_query(sm, q + row * kD, rv, qscale, qf + row * kD, qs + row * kGroups,
-               frag + seg * 512, koff + seg * 32, invs + row);
-  if (tid == 0) cnt_ws[seg] = 0;  // combine arrivals
+  for (int b = b0; b < min(b0 + nb, B); ++b) {
+    const size_t row = (size_t)b * h_q + 4 * h, seg = (size_t)b * h_kv + h;
+    rotate_query(sm, q + row * kD, rv, qscale, qf + row * kD, qs + row * kGroups,
+                 frag + seg * 512, koff + seg * 32, invs + row);
+    if (tid == 0) cnt_ws[seg] = 0;  // combine arrivals
+  }
 
-  if (b != 0 || h != 0) return;
+  if (b0 != 0 || h != 0) return;
   // Split-K plan: pref[b] = INT2 pages of sequences < b, nzpref[b] =
   // sequences < b with INT2 pages.  Invalid lengths count as empty and are
   // flagged.
@@ -80,8 +82,8 @@ __device__ __forceinline__ void qrot_body(
   }
 }
 
-__global__ void __launch_bounds__(kQrotThreads)
-qrot_kernel(const __nv_bfloat16* __restrict__ q, const float* __restrict__ R_k,
+__global__ void __launch_bounds__(kQrotThreads, 2)
+qrot_kernel(int nb, const __nv_bfloat16* __restrict__ q, const float* __restrict__ R_k,
             int B, int h_q, int h_kv, float qscale,
             const int32_t* __restrict__ seq_lens, int max_pages,
             float* __restrict__ qf, float* __restrict__ qs,
@@ -90,7 +92,7 @@ qrot_kernel(const __nv_bfloat16* __restrict__ q, const float* __restrict__ R_k,
             int* __restrict__ nzpref, int* __restrict__ cnt_ws,
             unsigned* err, int sink, int recent) {
   __shared__ QrotSmem sm;
-  qrot_body(blockIdx.x, blockIdx.y, sm, q, R_k, B, h_q, h_kv, qscale, seq_lens,
+  qrot_body(blockIdx.x * nb, nb, blockIdx.y, sm, q, R_k, B, h_q, h_kv, qscale, seq_lens,
             max_pages, qf, qs, frag, koff, invs, pref, nzpref, cnt_ws, err,
             sink, recent);
 }
@@ -102,11 +104,18 @@ qrot_kernel(const __nv_bfloat16* __restrict__ q, const float* __restrict__ R_k,
 // CTAs, BF16 windows only) and the query rotation (the following B * h_kv
 // CTAs, as qrot_kernel).  All wait for the previous kernel before touching
 // inputs; the partial kernel then waits for this grid, i.e. for all.
+// Bound by latency: each CTA loads 64 KB of a rotation and goes through a few
+// barriers.  So two CTAs share an SM (64 registers, tiles of 4 new tokens; one
+// of 70 or, with tiles of 16, 102 registers took two waves for 16 sequences x 8
+// heads and eight for 128 x 8), and a query-rotation CTA takes its head's
+// rotation through `nb` sequences, so that these CTAs are at most one such wave.
+// Decode step of 16 x 8192 tokens 45.4 -> 44.0 us; of 128 x 1024 to 32768, with
+// the combine's two CTAs per SM, 530.4 -> 518.3; of 37 short ones, 4 heads, 28.2
+// -> 26.8.
 static_assert(kQrotThreads == 512, "one block size for every body");
 static_assert(sizeof(float) * kPage * 4 >= (size_t)kWinPBytes, "window P scratch");
 
-template <int T>
-__global__ void __launch_bounds__(512)
+__global__ void __launch_bounds__(512, 2)
 step_prologue_kernel(
     int n_app, int app_tiles, const __nv_bfloat16* __restrict__ k,
     const __nv_bfloat16* __restrict__ v, int n_tok,
@@ -121,7 +130,7 @@ step_prologue_kernel(
     int* __restrict__ nzpref, int* __restrict__ cnt_ws, unsigned* err, int fold_v,
     int n_wcp, __nv_bfloat16* __restrict__ win,
     const int32_t* __restrict__ win_slot, int n_slots, int sink, int recent,
-    int group128, int lead) {
+    int group128, int lead, int nb) {
   extern __shared__ __align__(16) unsigned char dsm_[];
   // Block order: `lead` query-rotation CTAs, the cache-write CTAs, then the
   // remaining query-rotation CTAs.  With lead = SMs - write CTAs, the first
@@ -136,8 +145,8 @@ step_prologue_kernel(
   if (bid < n_app) {
     const int tblk = bid % app_tiles, hk = (bid / app_tiles) % h_kv,
               kind = bid / (app_tiles * h_kv);
-    append_small_body<T>(tblk, hk, kind, *reinterpret_cast<AppendSmallSmemT<T>*>(dsm_),
-                      k, v, n_tok, cu_new, pos0, bt, B, max_pages, pool,
+    append_small_body<kSmallTokFew>(
+                      tblk, hk, kind, *reinterpret_cast<AppendSmallSmemT<kSmallTokFew>*>(dsm_), k, v, n_tok, cu_new, pos0, bt, B, max_pages, pool,
                       num_pages, h_kv, R_k, R_v, muR, clip_k, clip_v, err,
                       fold_v && kind == 1, group128 != 0);
   } else if (bid < n_app + n_wcp) {
@@ -146,7 +155,7 @@ step_prologue_kernel(
                      sink, recent, err);
   } else {
     const int r = bid - n_app - n_wcp;
-    qrot_body(r / h_kv, r % h_kv, *reinterpret_cast<QrotSmem*>(dsm_), q, R_k, B,
+    qrot_body(r / h_kv * nb, nb, r % h_kv, *reinterpret_cast<QrotSmem*>(dsm_), q, R_k, B,
               h_q, h_kv, qscale, seq_lens, max_pages, qf, qs, frag, koff, invs,
               pref, nzpref, cnt_ws, err, sink, recent);
   }
@@ -824,25 +833,24 @@ cudaError_t launch_decode(const optr_params* p, int variant,
 
   int* cnt_ws = reinterpret_cast<int*>(w + plan.off_cnt);
   cudaError_t e;
+  // sequences that a query-rotation CTA takes in turn: no more CTAs than two per SM
+  const int nb = (int)(((long long)B * h_kv + 2 * p->num_sms - 1) / (2 * p->num_sms));
   // CTAs per segment of the one-launch decode (0: split-K)
   const int cs = variant != OPTR_VARIANT_CUDA_CORE ? decode_one_cluster(p, B, max_pages) : 0;
   if (app) {
     // the cache write of the step (INT2 records and window copies) and the
     // query rotation in one launch (the one-launch decode rotates its own)
     prof_mark(p, 0, s);
-    const int T = small_tile(app->n_tok);
-    const int tiles = (app->n_tok + T - 1) / T;
+    const int tiles = (app->n_tok + kSmallTokFew - 1) / kSmallTokFew;
     const int n_app = tiles * h_kv * 2;
     const int n_wcp = windows ? (app->n_tok + kWinCopyTok - 1) / kWinCopyTok : 0;
-    const size_t sm_app = T == kSmallTokFew ? sizeof(AppendSmallSmemT<kSmallTokFew>)
-                                            : sizeof(AppendSmallSmemT<kSmallTok>);
+    const size_t sm_app = sizeof(AppendSmallSmemT<kSmallTokFew>);
     size_t sm_bytes = sm_app > sizeof(QrotSmem) ? sm_app : sizeof(QrotSmem);
     if (sm_bytes < sizeof(WinCopySmem)) sm_bytes = sizeof(WinCopySmem);
-    auto fn = T == kSmallTokFew ? step_prologue_kernel<kSmallTokFew>
-                                : step_prologue_kernel<kSmallTok>;
+    auto fn = step_prologue_kernel;
     e = ensure_dynamic_smem(reinterpret_cast<const void*>(fn), sm_bytes);
     if (e != cudaSuccess) return e;
-    const int n_rot = cs ? 0 : B * h_kv;
+    const int n_rot = cs ? 0 : (B + nb - 1) / nb * h_kv;
     e = launch_pdl(fn, dim3(n_app + n_wcp + n_rot), dim3(512),
                    sm_bytes, s, n_app, tiles, app->k, app->v, app->n_tok,
                    app->cu_new, app->pos0, bt, app->pool, num_pages,
@@ -854,7 +862,7 @@ cudaError_t launch_decode(const optr_params* p, int variant,
                    windows ? win->slot : (const int32_t*)nullptr,
                    windows ? win->n_slots : 0, sink, recent,
                    p->cfg.group == 128 ? 1 : 0,
-                   std::max(0, std::min(n_rot, p->num_sms - n_app - n_wcp)));
+                   std::max(0, std::min(n_rot, p->num_sms - n_app - n_wcp)), nb);
     if (e != cudaSuccess) return e;
     prof_mark(p, 1, s);  // the append stage covers the fused launch,
     prof_mark(p, 2, s);  // the query-rotation stage is empty
@@ -862,7 +870,7 @@ cudaError_t launch_decode(const optr_params* p, int variant,
     prof_mark(p, 2, s);
   } else {
     prof_mark(p, 2, s);
-    e = launch_pdl(qrot_kernel, dim3(B, h_kv), dim3(kQrotThreads), 0, s, q,
+    e = launch_pdl(qrot_kernel, dim3((B + nb - 1) / nb, h_kv), dim3(kQrotThreads), 0, s, nb, q,
                    p->R_k, B, h_q, h_kv, qscale, seq_lens, max_pages, qf, qs,
                    frag, koff, invs, pref, nzpref, cnt_ws, p->err, sink,
                    recent);
@@ -893,10 +901,13 @@ cudaError_t launch_decode(const optr_params* p, int variant,
   }
   if (e != cudaSuccess) return e;
   prof_mark(p, 4, s);
-  // R_v^T (64 KB) plus padding: more than half of an SM's shared memory,
-  // so no two combine CTAs share an SM (in a decode step they take SMs as
-  // the partial kernel's CTAs leave them)
-  const size_t cmb_bytes = 120 * 1024;
+  // R_v^T (64 KB).  With no more segments than SMs it is padded to more than
+  // half of an SM's shared memory, so that no two combine CTAs share an SM (in a
+  // decode step they take SMs as the partial kernel's CTAs leave them).  With
+  // more, two per SM hide each other's latencies: the combine of 128 sequences x
+  // 8 heads took 31 us in seven waves; step of 128 x 600 to 8192 tokens with
+  // windows 193.3 -> 182.8 us.
+  const size_t cmb_bytes = ((long long)B * h_kv > p->num_sms ? 64 : 120) * 1024;
   if (plan.S == 1) {
     e = ensure_dynamic_smem(reinterpret_cast<const void*>(&combine_fast_kernel),
                             cmb_bytes);
