@@ -222,14 +222,15 @@ __device__ __forceinline__ void digits_step(float (&acc)[kWeights][4], const __h
   }
 }
 
-// sum_d acc_d 256^-d of output i as an integer with unit 2^-43 (|sum| < 2^62
-// over a depth of 128)
+// sum_d acc_d 256^-d of output i as an integer with unit 2^-43 (|sum| < 2^63
+// over a depth of 128).  A weight alone is below 2^24, a pair of them past 32
+// bits: |w_6| reaches 128 x 6 x 2^14 where digits repeat (constant rows).
 __device__ __forceinline__ long long digits_sum(const float (&acc)[kWeights][4], int i) {
   int w[kWeights];
 #pragma unroll
   for (int d = 0; d < kWeights; ++d) w[d] = __float2int_rn(acc[d][i]);
-  return ((long long)(w[0] * 256 + w[1]) << 35) + ((long long)(w[2] * 256 + w[3]) << 19) +
-         ((long long)(w[4] * 256 + w[5]) << 3) + ((w[6] * 256 + w[7] + 4096) >> 13);
+  auto pair = [&](int d) { return (long long)w[d] * 256 + w[d + 1]; };
+  return (pair(0) << 35) + (pair(2) << 19) + (pair(4) << 3) + ((pair(6) + 4096) >> 13);
 }
 
 // v + t 2^(E0 + E1 - 55 - f), |x| < 2^E in a row, E = e - 1022

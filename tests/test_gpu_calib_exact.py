@@ -1,0 +1,81 @@
+"""The calibration's float64 products on inputs whose exact result is known.
+
+One token (its softmax weight is 1), identity rotations and values below 2^-26
+(every level of Q2 is then fp16 zero) leave Vt - V = -V, so the value loss is
+the mean over query rows and heads of |W_O[j] V|^2 / d_model: one product of
+depth 128 whose operands a test chooses freely, compared with exact rational
+arithmetic.  The tolerance is what a float64 FMA chain guarantees for terms of
+one sign: 128 roundings per product (twice in the square), plus the roundings of
+the sums of squares and of the mean (at most one per 32 channels, 256 rows and
+a few more).
+"""
+from fractions import Fraction
+
+import pytest
+import torch
+
+from paper_2608_02691_gb300 import optr
+
+pytestmark = pytest.mark.gpu
+
+F64 = torch.float64
+D = 128
+U = 2.0 ** -53
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _setup():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2608_02691_gb300 import build
+    build.build()
+    torch.cuda.set_device(0)
+
+
+def _value_loss(v, W, nt):
+    """(loss, tolerance) of one token with value v [128] under W [g][d_model][128]."""
+    g, dm, _ = W.shape
+    cfg = optr.calib_config(g, dm, 1, nt)
+    I = torch.eye(D, dtype=F64)
+    zeros = torch.zeros(1, D, dtype=F64)
+    loss, _ = optr.optr_calib_loss_grad(
+        cfg, 1, *[x.cuda() for x in (torch.zeros(nt, g, D, dtype=F64), zeros, v.view(1, D),
+                                     torch.zeros(nt, dtype=torch.int32), W, zeros[0], I,
+                                     torch.zeros(D, D, dtype=F64))], R_K=I.cuda(), grad=False)
+    return float(loss.item()), (2 * D + dm / 32 + g * nt / 256 + 32) * U
+
+
+def _exact(v, W):
+    vs = [Fraction(x) for x in v.tolist()]
+    sq = {}
+    for w in W.flatten(0, 1).tolist():
+        key = tuple(w)
+        if key not in sq:
+            sq[key] = [sum(a * Fraction(b) for a, b in zip(vs, w)) ** 2, 0]
+        sq[key][1] += 1
+    return sum(x * n for x, n in sq.values()) / (W.shape[0] * W.shape[1])
+
+
+# (query rows, output channels): both tile shapes of the product, whole and
+# ragged
+SHAPES = [(1, 1), (65, 1249)]
+
+
+def _const(c, last=1.0):
+    x = torch.full((D,), c, dtype=F64)
+    x[-1] *= last
+    return x
+
+
+@pytest.mark.parametrize("nt,dm", SHAPES)
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+@pytest.mark.parametrize("x", [
+    _const(15 / 17), _const(41 / 51), _const(259 / 510), _const(float.fromhex("0x1.fc04040404040p0")),
+    _const(1 / 17, 8.0), _const(9 / 17, 64.0),
+], ids=["15/17", "41/51", "259/510", "1.984", "8/17", "64*9/17"])
+def test_constant_rows(x, sign, nt, dm):
+    """Digits that repeat over the whole depth: the largest sums per weight."""
+    v, W = x * 2.0 ** -36, (sign * x).expand(1, dm, D).contiguous()
+    loss, rel = _value_loss(v, W, nt)
+    ref = _exact(v, W)
+    assert abs(Fraction(loss) - ref) <= rel * ref
