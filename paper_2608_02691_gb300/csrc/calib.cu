@@ -9,7 +9,7 @@
 //
 // Everything is float64: the calibration is a one-time offline pass, and float64
 // keeps its trajectory reproducible.  The matrix products, its bulk, run on the
-// fp16 tensor cores as exact integer products (gemm_digits_kernel), the rest on
+// fp16 tensor cores as exact products of digits (gemm_digits_kernel), the rest on
 // the CUDA cores.
 // The gradient is written out (no autograd):
 //   keys    Z = (K - mu) R, Zh = Q2(Z), Kt = Zh R^T, l = scale q Kt^T
@@ -58,29 +58,41 @@ struct Gemm {
   const double* sub;  // C = .. - sub when given, likewise
 };
 
-// The product runs on the fp16 tensor cores, exactly, after a split of both
-// factors into small integers (the scheme of Ozaki, Ogita, Oishi and Rump,
-// "Error-free transformations of matrix multiplication", 2012): this GPU does
+// The product runs on the fp16 tensor cores after a split of both factors into
+// small integers, whose products are exact (the scheme of Ozaki, Ogita, Oishi and
+// Rump, "Error-free transformations of matrix multiplication", 2012): this GPU does
 // 2 float64 FMAs per clock and SM, three orders of magnitude below its tensor
-// cores.  Per k chunk of 128, a row of A (a column of B) is written as
-// fixed-point numbers under its own largest exponent, 54 bits and sign, in
-// seven balanced base-256 digits d_0 .. d_6 (|d_0| <= 64, else |d| <= 128),
+// cores.  Per k chunk of 128, a row of A (a column of B) is rounded to
+// fixed-point numbers under its own largest exponent, 62 bits and sign, in
+// eight balanced base-256 digits d_0 .. d_7 (|d_0| <= 64, else |d| <= 128),
 // which are exact fp16 values.  All digit products of one weight d = i + j are
-// summed in one float32 accumulator: at most 7 x 128 x 2^14 < 2^24, so every
-// sum is exact.  The weights 0 .. 7 (34 of the 49 products; what is left out of
-// one product is below 2^-59 of the largest one) are put together in 64-bit
-// integers and added to the float64 result, one rounding per 128 products.  Against sums in
-// extended precision that is 2 to 5 times closer than a float64 FMA chain
-// (relative error 1.5e-16 to 2.8e-16 on keys x rotation, probabilities x
-// values, powers of the generator; FMA chain 2.8e-16 to 1.5e-15).
-// A row or column with a NaN or an infinity gives NaN throughout.
-// What bounds it: per CTA and chunk 272 mma a warp (4.4 us at one m16n8k16 per 8
-// cycles and SM quarter), the split of both tiles (24 values a thread, ~45
+// summed in one float32 accumulator: at most 128 x 7 x 2^14 < 2^24, so every
+// sum is exact.  The weights 0 .. 8 (43 of the 64 products; what is left out of
+// one product is below 2^-67 of the largest one) are put together in 64-bit
+// integers and added to the float64 result, one rounding per 128 products.
+//
+// What the split loses is bounded by the largest elements of the row and of the
+// column, about 2^-62 of max|a| max|b| per chunk, not by the sum: far better than
+// a float64 FMA chain while large elements meet large ones, unbounded where they
+// do not (an outlier channel against a zero of the rotation).  So one more mma
+// per step multiplies the magnitudes, two digits each, and outputs with
+// sum |a b| below 1/1024 of the largest product possible take their chunk's sum
+// from float64 FMAs (float64_sums; as good as none in a calibration on synthetic
+// traces), rows and columns with a NaN or an infinity too.  Largest error against
+// sum |a b| at depth 128, float64 FMA chain / digits alone / both as here: normal
+// 6e-16 / 5e-17 / 5e-17; softmax of logits of deviation 3 and 10 x t(4) 2e-15 /
+// 1e-14 / 3e-16; exponents spread over 80 bits 1.4e-15 / 9e-9 / 3e-16; an outlier
+// channel of 1e8 2.7e-15 / 6e-15 / 6e-16, times an identity 0 / 4e-6 / 0.  (Seven
+// digits, 54 bits, need that line at 1/8 for the errors of an FMA chain: 6% of the
+// probabilities x values of a calibration, 20 steps 33.7 ms.)
+// What bounds it: per CTA and chunk 352 mma a warp (5.7 us at one m16n8k16 per 8
+// cycles and SM quarter), the split of both tiles (24 values a thread, ~50
 // integer instructions each, 2.5 us) and the load's latency, one after the
-// other, as 172 KB of digits leave room for one CTA per SM.  64 x 32 tiles make
+// other, as 197 KB of digits leave room for one CTA per SM.  64 x 32 tiles make
 // the calibration's products (2048 or 4 x 64 rows, 128 columns or the reverse)
-// one wave of 128 CTAs: 2048 x 128 x 128 takes 19 us from cold caches, 25 with
-// 32 x 32 tiles in two waves, 21 with 64-deep chunks and two CTAs per SM.
+// one wave of 128 CTAs: 2048 x 128 x 128 takes 20.6 us from cold caches (with
+// seven digits 17.8, 25 with 32 x 32 tiles in two waves, 21 with 64-deep chunks
+// and two CTAs per SM).
 // Products with fewer than half as many tiles and chunks as SMs take 32 x 16
 // tiles (8 steps on 256 tokens: 4.4 ms, 5.0 with 64 x 32 throughout).
 //
@@ -89,8 +101,8 @@ struct Gemm {
 // counter, left at 0 again) adds the parts in a fixed order, z = 0 .. kc-1,
 // so the result does not depend on which CTA that is.
 constexpr int kGK = 128;     // k chunk
-constexpr int kDigits = 7;
-constexpr int kWeights = 8;
+constexpr int kDigits = 8;
+constexpr int kWeights = 9;
 constexpr int kBadExp = 1 << 20;  // exponent of a row with a non-finite value
 
 // MT x NT outputs, one warp per 16 x 8 of them
@@ -125,18 +137,19 @@ __device__ __forceinline__ int row_exponent(int f) {
   return f == 0x7ff00000 ? kBadExp : max(f >> 20, 1);
 }
 
-// x as a fixed-point integer with unit 2^(e_row - 1076), rounded, |result| <=
-// 2^54, plus the bias that makes its bytes digit + 128.
+// x as a fixed-point integer with unit 2^(e_row - 1084), rounded, |result| <=
+// 2^62, plus the bias that makes its bytes digit + 128.
+constexpr unsigned long long kBias = 0x8080808080808080ull;
 __device__ __noinline__ unsigned long long fixed_point_small(double x, int e_row) {
   const unsigned long long bits = __double_as_longlong(x);
-  if (bits << 1 == 0) return 0x80808080808080ull;
+  if (bits << 1 == 0) return kBias;
   const int e = (int)(bits >> 52) & 2047;
   unsigned long long m = (bits & 0xfffffffffffffull) | (e ? 1ull << 52 : 0ull);
   const int sh = e_row - max(e, 1);
-  m <<= 1;
-  if (sh > 0) m = sh < 56 ? (m + (1ull << (sh - 1))) >> sh : 0ull;
+  m <<= 9;
+  if (sh > 0) m = sh < 64 ? (m + (1ull << (sh - 1))) >> sh : 0ull;
   const long long f = (long long)bits < 0 ? -(long long)m : (long long)m;
-  return (unsigned long long)f + 0x80808080808080ull;
+  return (unsigned long long)f + kBias;
 }
 // The same for e_row >= kFastExp, in 15 integer instructions: zeros and
 // subnormals (no implicit bit) are shifted out with the rest of what is below
@@ -146,12 +159,12 @@ __device__ __forceinline__ unsigned long long fixed_point(double x, int e_row) {
   const int hi = __double2hiint(x);
   const unsigned lo = (unsigned)__double2loint(x);
   const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
-  // two fractional bits, then one addition rounds (half away from zero)
-  const unsigned long long m = ((unsigned long long)__funnelshift_l(lo, mh, 2) << 32) | (lo << 2);
+  // one fractional bit more, then one addition rounds (half away from zero)
+  const unsigned long long m = ((unsigned long long)__funnelshift_l(lo, mh, 10) << 32) | (lo << 10);
   const int sh = min(e_row - ((hi >> 20) & 2047), 63);
   const unsigned long long t = ((m >> sh) + 1) >> 1;
   const unsigned long long sg = (long long)(hi >> 31);
-  return (t ^ sg) - sg + 0x80808080808080ull;
+  return (t ^ sg) - sg + kBias;
 }
 
 // The digits of eight k of row r (piece kg) into the planes.
@@ -172,12 +185,12 @@ __device__ __forceinline__ void store_digits(__half (*planes)[ROWS][KS], int r, 
     }
     const uint32_t l0 = (uint32_t)f0, l1 = (uint32_t)f1, u0 = (uint32_t)(f0 >> 32), u1 = (uint32_t)(f1 >> 32);
     const uint32_t b01 = __byte_perm(l0, l1, 0x5140), b23 = __byte_perm(l0, l1, 0x7362),
-                   b45 = __byte_perm(u0, u1, 0x5140), b6 = __byte_perm(u0, u1, 0x7362);
+                   b45 = __byte_perm(u0, u1, 0x5140), b67 = __byte_perm(u0, u1, 0x7362);
     const uint32_t w[kDigits] = {
-        __byte_perm(b6, 0x64646464u, 0x4140),  __byte_perm(b45, 0x64646464u, 0x4342),
-        __byte_perm(b45, 0x64646464u, 0x4140), __byte_perm(b23, 0x64646464u, 0x4342),
-        __byte_perm(b23, 0x64646464u, 0x4140), __byte_perm(b01, 0x64646464u, 0x4342),
-        __byte_perm(b01, 0x64646464u, 0x4140)};
+        __byte_perm(b67, 0x64646464u, 0x4342), __byte_perm(b67, 0x64646464u, 0x4140),
+        __byte_perm(b45, 0x64646464u, 0x4342), __byte_perm(b45, 0x64646464u, 0x4140),
+        __byte_perm(b23, 0x64646464u, 0x4342), __byte_perm(b23, 0x64646464u, 0x4140),
+        __byte_perm(b01, 0x64646464u, 0x4342), __byte_perm(b01, 0x64646464u, 0x4140)};
 #pragma unroll
     for (int d = 0; d < kDigits; ++d) {
       const __half2 v = __hsub2(*reinterpret_cast<const __half2*>(&w[d]), off);
@@ -190,21 +203,27 @@ __device__ __forceinline__ void store_digits(__half (*planes)[ROWS][KS], int r, 
         make_uint4(h[d][0], h[d][1], h[d][2], h[d][3]);
 }
 
-// One 16-deep step of the 34 digit products on the 16 x 8 outputs at (r0, c0);
-// p0: first of the step's two 16-byte pieces.
+// |256 d_0 + d_1| of two values as fp16 (at most 16512)
+__device__ __forceinline__ uint32_t digits_abs(uint32_t d0, uint32_t d1) {
+  const __half2 m = __hfma2(*reinterpret_cast<const __half2*>(&d0), __float2half2_rn(256.f),
+                            *reinterpret_cast<const __half2*>(&d1));
+  return *reinterpret_cast<const uint32_t*>(&m) & 0x7fff7fffu;
+}
+
+// One 16-deep step of the 43 digit products on the 16 x 8 outputs at (r0, c0),
+// and of the magnitudes in mag; p0: first of the step's two 16-byte pieces.
 template <int MT, int NT, int KS>
-__device__ __forceinline__ void digits_step(float (&acc)[kWeights][4], const __half (*a)[MT][KS],
-                                            const __half (*b)[NT][KS], int r0, int c0, int p0,
-                                            int lane) {
-  uint32_t fb[kDigits + 1][2];
+__device__ __forceinline__ void digits_step(float (&acc)[kWeights][4], float (&mag)[4],
+                                            const __half (*a)[MT][KS], const __half (*b)[NT][KS],
+                                            int r0, int c0, int p0, int lane) {
+  uint32_t fb[kDigits][2];
   {
     // lanes 0-15 address digit j, 16-31 digit j + 1
     const int r = c0 + (lane & 7), p = p0 + ((lane >> 3) & 1);
 #pragma unroll
     for (int j = 0; j < kDigits; j += 2) {
       uint32_t x[4];
-      const int jj = min(j + (lane >> 4), kDigits - 1);
-      digits_ldsm(x, &b[jj][r][(p ^ (r & 7)) * 8]);
+      digits_ldsm(x, &b[j + (lane >> 4)][r][(p ^ (r & 7)) * 8]);
       fb[j][0] = x[0];
       fb[j][1] = x[1];
       fb[j + 1][0] = x[2];
@@ -212,6 +231,7 @@ __device__ __forceinline__ void digits_step(float (&acc)[kWeights][4], const __h
     }
   }
   const int r = r0 + (lane & 15), p = p0 + (lane >> 4);
+  uint32_t ma[4];
 #pragma unroll
   for (int i = 0; i < kDigits; ++i) {
     uint32_t fa[4];
@@ -219,27 +239,81 @@ __device__ __forceinline__ void digits_step(float (&acc)[kWeights][4], const __h
 #pragma unroll
     for (int j = 0; j < kDigits; ++j)
       if (i + j < kWeights) digits_mma(acc[i + j], fa, fb[j][0], fb[j][1]);
+    if (i < 2) {
+#pragma unroll
+      for (int x = 0; x < 4; ++x) ma[x] = i == 0 ? fa[x] : digits_abs(ma[x], fa[x]);
+      if (i == 1)
+        digits_mma(mag, ma, digits_abs(fb[0][0], fb[1][0]), digits_abs(fb[0][1], fb[1][1]));
+    }
   }
 }
 
-// sum_d acc_d 256^-d of output i as an integer with unit 2^-43 (|sum| < 2^63
-// over a depth of 128).  A weight alone is below 2^24, a pair of them past 32
-// bits: |w_6| reaches 128 x 6 x 2^14 where digits repeat (constant rows).
-__device__ __forceinline__ long long digits_sum(const float (&acc)[kWeights][4], int i) {
+// Whether a chunk's sum of digit products is too small against its row's and
+// column's largest elements (exponents e0, e1; all zero or below 2^-1021: e = 1)
+// to be as accurate as float64 operations, or has a factor that is not finite:
+// see gemm_digits_kernel.
+constexpr float kMagMin = 262144.f;  // 2^28 / 1024
+__device__ __forceinline__ bool digits_lost(float mag, int e0, int e1) {
+  return max(e0, e1) >= kBadExp || (mag < kMagMin && min(e0, e1) > 1);
+}
+
+// For the lanes with `lost`: v = sum_{k < n} a[k sa] b[k sb] in float64.  Four of
+// them at a time, eight lanes each; the whole warp calls it.
+__device__ __forceinline__ void float64_sums(bool lost, const double* a, long long sa,
+                                             const double* b, long long sb, int n, double& v) {
+  const int lane = threadIdx.x & 31;
+  unsigned todo = __ballot_sync(0xffffffffu, lost);
+  while (todo != 0) {
+    int who[4];  // -1: none left
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      who[i] = __ffs(todo) - 1;
+      todo &= todo - 1;
+    }
+    const int lo = lane & 8 ? who[1] : who[0], hi = lane & 8 ? who[3] : who[2];
+    const int src = lane & 16 ? hi : lo;
+    const double* x = reinterpret_cast<const double*>(
+        __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(a), src & 31));
+    const double* y = reinterpret_cast<const double*>(
+        __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(b), src & 31));
+    double s = 0.0;
+    if (src >= 0) {
+#pragma unroll 4
+      for (int k = lane & 7; k < n; k += 8) s = fma(__ldcg(x + k * sa), __ldcg(y + k * sb), s);
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const double r = __shfl_sync(0xffffffffu, s, 8 * i);
+      if (lane == who[i]) v = r;
+    }
+  }
+}
+
+// sum_d acc_d 256^-d of output i as hi 2^-24 + lo 2^-64 (|sum| < 2^20 over a depth
+// of 128).  A weight alone is below 2^24, a pair of them past 32 bits: |w_7|
+// reaches 128 x 7 x 2^14 where digits repeat (constant rows).
+struct DigitSum {
+  long long hi, lo;
+};
+__device__ __forceinline__ DigitSum digits_sum(const float (&acc)[kWeights][4], int i) {
   int w[kWeights];
 #pragma unroll
   for (int d = 0; d < kWeights; ++d) w[d] = __float2int_rn(acc[d][i]);
   auto pair = [&](int d) { return (long long)w[d] * 256 + w[d + 1]; };
-  return (pair(0) << 35) + (pair(2) << 19) + (pair(4) << 3) + ((pair(6) + 4096) >> 13);
+  return {(pair(0) << 16) + pair(2), (pair(4) << 24) + (pair(6) << 8) + w[8]};
 }
 
-// v + t 2^(E0 + E1 - 55 - f), |x| < 2^E in a row, E = e - 1022
-__device__ __forceinline__ double digits_add(double v, long long t, int e0, int e1, int f) {
-  const int sc = e0 + e1 - 2 * 1022 - 55 - f;
+// v + t 2^(E0 + E1 - 12 - f), |x| < 2^E in a row, E = e - 1022; of t at least the
+// first 61 bits are kept
+__device__ __forceinline__ double digits_add(double v, DigitSum t, int e0, int e1, int f) {
+  const int drop = max(43 - __clzll(t.hi ^ (t.hi >> 63)), 0);  // of the 40 bits below hi
+  const long long n = (t.hi << (40 - drop)) + ((t.lo + ((1ll << drop) >> 1)) >> drop);
+  const int sc = e0 + e1 - 2 * 1022 - 76 + drop - f;
   if (sc >= -1022 && sc <= 1023)
-    return fma((double)t, __hiloint2double((sc + 1023) << 20, 0), v);
-  if (max(e0, e1) >= kBadExp) return __hiloint2double(0x7ff80000, 0);
-  return v + scalbn((double)t, sc);
+    return fma((double)n, __hiloint2double((sc + 1023) << 20, 0), v);
+  return v + scalbn((double)n, sc);
 }
 
 // The pieces of a tile of R rows that a thread loads and splits: piece p of a
@@ -336,17 +410,34 @@ __global__ void __launch_bounds__(GemmTile<MT, NT>::kThreads)
       pb.split(S.b, S.emax + MT, S.e + MT, b_rows);
       __syncthreads();
     }
-    float acc[kWeights][4];
+    float acc[kWeights][4], mag[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int d = 0; d < kWeights; ++d)
 #pragma unroll
       for (int i = 0; i < 4; ++i) acc[d][i] = 0.f;
 #pragma unroll 1
-    for (int ks = 0; ks < kGK / 16; ++ks) digits_step(acc, S.a, S.b, wm, wn, 2 * ks, lane);
+    for (int ks = 0; ks < kGK / 16; ++ks) digits_step(acc, mag, S.a, S.b, wm, wn, 2 * ks, lane);
+    unsigned lost = 0;
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-      out[i] = digits_add(out[i], digits_sum(acc, i), S.e[wm + (lane >> 2) + 8 * (i >> 1)],
-                          S.e[MT + wn + 2 * (lane & 3) + (i & 1)], 0);
+    for (int i = 0; i < 4; ++i) {
+      const int r = wm + (lane >> 2) + 8 * (i >> 1), c = wn + 2 * (lane & 3) + (i & 1);
+      const int e0 = S.e[r], e1 = S.e[MT + c];
+      if (!digits_lost(mag[i], e0, e1)) out[i] = digits_add(out[i], digits_sum(acc, i), e0, e1, 0);
+      else if (m0 + r < g.M && n0 + c < g.N) lost |= 1u << i;
+    }
+    if (__any_sync(0xffffffffu, lost != 0)) {
+#pragma unroll 1
+      for (int i = 0; i < 4; ++i) {
+        const int r = m0 + wm + (lane >> 2) + 8 * (i >> 1), c = n0 + wn + 2 * (lane & 3) + (i & 1);
+        double x = 0.0;
+        float64_sums(lost >> i & 1, a_rows ? A + r * g.lda + k0 : A + k0 * g.lda + r,
+                     a_rows ? 1 : g.lda, b_rows ? B + c * g.ldb + k0 : B + k0 * g.ldb + c,
+                     b_rows ? 1 : g.ldb, min(kGK, g.K - k0), x);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (j == i) out[j] += x;
+      }
+    }
     if (ch + 1 < ce) __syncthreads();
   }
   auto store = [&](int r, int c, double x) {
@@ -396,14 +487,14 @@ __global__ void __launch_bounds__(GemmTile<MT, NT>::kThreads)
 //   out0 = v_0, out1 = v_1, P = diag I + cy[0] Y[0] + cy[1] Y[1]
 //          + cy[2] v_0 + cy[3] v_1                            (out[1] given)
 // with f = 2^-(fs *s), s the device-decided number of squarings.  In digit
-// products as above, over the whole depth of 128 under one exponent (sums below
-// 7 x 128 x 2^14 < 2^24, still exact).
+// products as above, over the whole depth of 128 under one exponent.
 //
 // What bounds it: the chain, 26 to 32 links per Adam step, so a link's latency
-// (launch, one load, the split, 68 mma per warp, the sum over the four warps
+// (launch, one load, the split, 88 mma per warp, the sum over the four warps
 // that share the depth).  16 x 16 tiles on 64 CTAs of one or two halves (256
-// threads each) take 6.6 us (10 with two products) where the 32 x 32 tiles above,
-// 16 of them in two chunks, take 9.4 us a product.
+// threads each) take 7.2 us (10.4 with two products); with seven digits 6.6, where
+// 32 x 32 tiles of the kernel above, 16 of them in two chunks, took 9.4 us a
+// product.
 constexpr int kMT = 16;
 constexpr int kMaxSquare = 16;  // norms up to 2^15
 
@@ -428,7 +519,8 @@ struct MatOp {
 
 struct MatHalf {
   __half d[2][kDigits][kMT][kCD];  // as in GemmTile
-  long long part[4][kMT][kMT];     // sums of the four depth slices
+  DigitSum part[4][kMT][kMT];      // sums of the four depth slices
+  float mag[4][kMT][kMT];
   int emax[kMT][17];
   int e[2][kMT];
   double v[kMT][kMT];
@@ -506,21 +598,37 @@ __global__ void __launch_bounds__(256 * H) mat_product_kernel(MatOp o) {
     if (ka == 0) S.e[0][ra] = ea;
     if (kb == 0) S.e[1][rb] = eb;
     __syncthreads();
-    float acc[kWeights][4];
+    float acc[kWeights][4], mag[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int d = 0; d < kWeights; ++d)
 #pragma unroll
       for (int i = 0; i < 4; ++i) acc[d][i] = 0.f;
 #pragma unroll
     for (int ks = 0; ks < 2; ++ks)
-      digits_step(acc, S.d[0], S.d[1], 0, 8 * wn, 4 * ws + 2 * ks, lane);
+      digits_step(acc, mag, S.d[0], S.d[1], 0, 8 * wn, 4 * ws + 2 * ks, lane);
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-      S.part[ws][(lane >> 2) + 8 * (i >> 1)][8 * wn + 2 * (lane & 3) + (i & 1)] =
-          digits_sum(acc, i);
+    for (int i = 0; i < 4; ++i) {
+      const int ri = (lane >> 2) + 8 * (i >> 1), ci = 8 * wn + 2 * (lane & 3) + (i & 1);
+      S.part[ws][ri][ci] = digits_sum(acc, i);
+      S.mag[ws][ri][ci] = mag[i];
+    }
     __syncthreads();
-    const long long t = S.part[0][r][c] + S.part[1][r][c] + S.part[2][r][c] + S.part[3][r][c];
-    v = digits_add(v, t, S.e[0][r], S.e[1][c], o.fs * s);
+    DigitSum t = S.part[0][r][c];
+    float m = S.mag[0][r][c];
+#pragma unroll
+    for (int i = 1; i < 4; ++i) {
+      t.hi += S.part[i][r][c].hi;
+      t.lo += S.part[i][r][c].lo;
+      m += S.mag[i][r][c];
+    }
+    const bool lost = digits_lost(m, S.e[0][r], S.e[1][c]);
+    if (!lost) v = digits_add(v, t, S.e[0][r], S.e[1][c], o.fs * s);
+    if (__any_sync(0xffffffffu, lost)) {
+      double x = 0.0;
+      float64_sums(lost, o.tA ? A + m0 + r : A + (m0 + r) * kCD, o.tA ? kCD : 1, B + n0 + c, kCD,
+                   kCD, x);
+      v += ldexp(x, -o.fs * s);
+    }
   }
   const int idx = (m0 + r) * kCD + n0 + c;
   const double dg = m0 + r == n0 + c ? o.diag : 0.0;

@@ -79,3 +79,74 @@ def test_constant_rows(x, sign, nt, dm):
     loss, rel = _value_loss(v, W, nt)
     ref = _exact(v, W)
     assert abs(Fraction(loss) - ref) <= rel * ref
+
+
+def _spread(seed, lo, hi):
+    """Positive values with exponents uniform in [lo, hi)."""
+    gen = torch.Generator().manual_seed(seed)
+    m = 1.0 + torch.rand(D, generator=gen, dtype=F64)
+    return m * 2.0 ** torch.randint(lo, hi, (D,), generator=gen).to(F64)
+
+
+def _outlier(seed, k, e):
+    x = _spread(seed, 0, 2)
+    x[k] = 2.0 ** e
+    return x
+
+
+WIDE = {
+    # the row's largest element meets a zero, or the column's smallest
+    "outlier x zero": (_outlier(1, 5, 60), _outlier(2, 5, -2000)),
+    "outlier x small": (_outlier(1, 5, 40), _outlier(2, 5, -50)),
+    "both outliers": (_outlier(1, 5, 50), _outlier(2, 6, 50)),
+    "one element x zeros": (_outlier(1, 0, 200), torch.cat([torch.zeros(1), torch.ones(127)]).double()),
+    "spread 10": (_spread(3, 0, 10), _spread(4, 0, 10)),
+    "spread 80": (_spread(3, 0, 80), _spread(4, 0, 80)),
+    "spread 600": (_spread(3, -600, 0), _spread(4, -400, 0)),
+    "softmax": (torch.exp(10 * torch.randn(D, generator=torch.Generator().manual_seed(5), dtype=F64) - 40),
+                _spread(6, 0, 12)),
+}
+
+
+@pytest.mark.parametrize("nt,dm", SHAPES)
+@pytest.mark.parametrize("name", WIDE)
+def test_wide_range_inside_a_row(name, nt, dm):
+    """Elements far below their row's or column's largest keep their own precision."""
+    v, w = WIDE[name]
+    v = v / v.max() * 2.0 ** -36
+    W = w.expand(1, dm, D).contiguous()
+    loss, rel = _value_loss(v, W, nt)
+    ref = _exact(v, W)
+    assert ref > 0
+    assert abs(Fraction(loss) - ref) <= rel * ref
+
+
+@pytest.mark.parametrize("nt,dm", SHAPES)
+def test_infinite_weight_gives_an_infinite_loss(nt, dm):
+    W = _spread(7, 0, 4).expand(1, dm, D).contiguous()
+    W[0, dm // 2, 17] = float("inf")
+    assert _value_loss(_spread(8, -40, -36), W, nt)[0] == float("inf")
+    W[0, dm // 2, 17] = float("nan")
+    loss = _value_loss(_spread(8, -40, -36), W, nt)[0]
+    assert loss != loss
+
+
+@pytest.mark.parametrize("lo", [0, -8, -80])
+def test_gradient_elements_keep_their_own_precision(lo):
+    """With one token, one output channel and identity rotations the generator's
+    gradient is V_i u_j - V_j u_i with u = -2 (w V) w, through every product of
+    the backward pass; each element against the size of its own two terms.  Four
+    products of depth 128 are on the way (and a few single roundings)."""
+    v, w = _spread(11, lo, 1) * 2.0 ** -36, _spread(12, lo, 1)
+    cfg = optr.calib_config(1, 1, 1, 1)
+    I, zero = torch.eye(D, dtype=F64), torch.zeros(1, D, dtype=F64)
+    _, dA = optr.optr_calib_loss_grad(
+        cfg, 1, *[x.cuda() for x in (zero.view(1, 1, D), zero, v.view(1, D),
+                                     torch.zeros(1, dtype=torch.int32), w.view(1, 1, D), zero[0], I,
+                                     torch.zeros(D, D, dtype=F64))], R_K=I.cuda())
+    vs, ws = [[Fraction(x) for x in t.tolist()] for t in (v, w)]
+    e = -sum(a * b for a, b in zip(vs, ws))
+    for i, row in enumerate(dA.cpu().tolist()):
+        for j, got in enumerate(row):
+            a, b = vs[i] * 2 * e * ws[j], vs[j] * 2 * e * ws[i]
+            assert abs(Fraction(got) - (a - b)) <= (4 * D + 16) * U * (abs(a) + abs(b))
