@@ -969,18 +969,19 @@ __global__ void zero_window_kernel(double* __restrict__ P, int rows, int nt, int
     if (is_window(s, t, sink, recent)) P[row * (long long)T + s] = 0.0;
 }
 
-// rowv[row] = (add ? rowv[row] : 0) + lam * (sum_c A[row][c] B[row][c]) / dm,
-// rows of n
-__global__ void row_dot_kernel(const double* A, const double* B, int rows, int n, int dm,
-                               double lam, int add, double* rowv) {
+// rowv[row] = (add ? rowv[row] : 0) + lam * (sum_c E[row][c]^2) / dm
+__global__ void row_sqsum_kernel(const double* E, int rows, int dm, double lam, int add,
+                                 double* rowv) {
   const int lane = threadIdx.x & 31;
   const long long row = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   pdl_wait();
   pdl_trigger();
   if (row >= rows) return;
   double s = 0.0;
-  for (int c = lane; c < n; c += 32)
-    s += __ldcg(A + row * (long long)n + c) * __ldcg(B + row * (long long)n + c);
+  for (int c = lane; c < dm; c += 32) {
+    const double e = __ldcg(E + row * (long long)dm + c);
+    s += e * e;
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if (lane == 0) {
@@ -1149,7 +1150,6 @@ struct Calib {
   int* s_dev;
   unsigned* err;
   const double* W;  // [g][d_model][d]
-  double* M;        // [g][d][d] W^T W, or null
   double* gsc;      // split-K scratch of the GEMMs
   int* gcnt;        // split-K arrival counters (kGemmTiles, zero between calls)
   cudaStream_t st;
@@ -1198,7 +1198,6 @@ size_t carve(Calib& C, char* base) {
   C.PK = L.take<double>(g * nm * Tm);
   C.GV = L.take<double>(g * nm * Tm);
   C.DP = L.take<double>(g * nm * Tm);
-  C.M = L.take<double>(g * D2);
   C.rowv = L.take<double>(g * nm);
   C.DV = L.take<double>(g * nm * D);
   C.U = L.take<double>(g * nm * D);
@@ -1398,44 +1397,23 @@ void q2_roundtrip(Calib& C, const double* X, int T, double clip, const double* s
   gm.run(k, 1);
 }
 
-// rowv[j, t] (+)= lam ||e_j||^2 / d_model with e_j = DV_j W_j^T.  With the
-// products M_j = W_j^T W_j at hand ||e||^2 = DV (DV M)^T, and U0 = DV M, the
-// gradient e_j W_j, is done as well; else e_j goes to Eo.
+// e_j = DV_j W_j^T into Eo, rowv[j, t] (+)= lam ||e_j||^2 / d_model.  (||e||^2 as
+// DV (W^T W) DV^T, with W^T W once per call, took 0.1 ms less per Adam step at
+// d_model = 4096, but its error grows with the square of W's condition number:
+// 4e-6 of the term at 1e6, and below zero for a rank-deficient W.)
 void output_error(Calib& C, Trace& t, double lam, int add) {
-  GemmCall gm = C.gemm();
   const int g = C.c.g, D = kCD, dm = C.c.d_model, r = g * t.nt;
-  const long long nD = (long long)t.nt * D;
-  if (C.M != nullptr) {
-    gm(t.nt, D, D, C.DV, D, false, C.M, D, false, C.U, D, 1.0, g, nD, (long long)kD2, nD);
-    launch_pdl(&row_dot_kernel, dim3(nwarp_blocks(r)), dim3(256), 0, C.st, C.DV, C.U, r, D, dm, lam,
-               add, C.rowv);
-    return;
-  }
-  gm(t.nt, dm, D, C.DV, D, false, C.W, D, true, C.Eo, dm, 1.0, g, nD, (long long)dm * D,
-     (long long)t.nt * dm);
-  launch_pdl(&row_dot_kernel, dim3(nwarp_blocks(r)), dim3(256), 0, C.st, C.Eo, C.Eo, r, dm, dm, lam,
-             add, C.rowv);
+  C.gemm()(t.nt, dm, D, C.DV, D, false, C.W, D, true, C.Eo, dm, 1.0, g, (long long)t.nt * D,
+           (long long)dm * D, (long long)t.nt * dm);
+  launch_pdl(&row_sqsum_kernel, dim3(nwarp_blocks(r)), dim3(256), 0, C.st, C.Eo, r, dm, lam, add,
+             C.rowv);
 }
 
 // U0 = e_j W_j (after output_error on the same trace)
 void output_grad(Calib& C, Trace& t) {
   const int g = C.c.g, D = kCD, dm = C.c.d_model;
-  if (C.M == nullptr)
-    C.gemm()(t.nt, D, dm, C.Eo, dm, false, C.W, D, false, C.U, D, 1.0, g,
-             (long long)t.nt * dm, (long long)dm * D, (long long)t.nt * D);
-}
-
-// The products M_j pay when they replace more than they cost: per step and
-// phase 2 nt rows through W (once for e, once for U) become nt rows through a
-// d x d matrix; M_j itself costs d rows through W.
-void output_setup(Calib& C) {
-  const optr_calib_config& c = C.c;
-  if (c.d_model < kCD || (double)c.steps * c.nt < kCD / 2) {
-    C.M = nullptr;
-    return;
-  }
-  C.gemm()(kCD, kCD, c.d_model, C.W, kCD, true, C.W, kCD, false, C.M, kCD, 1.0, c.g,
-           (long long)c.d_model * kCD, (long long)c.d_model * kCD, (long long)kD2);
+  C.gemm()(t.nt, D, dm, C.Eo, dm, false, C.W, D, false, C.U, D, 1.0, g, (long long)t.nt * dm,
+           (long long)dm * D, (long long)t.nt * D);
 }
 
 void loss_mean(Calib& C, int rows, double* out) {
@@ -1453,7 +1431,7 @@ void key_forward(Calib& C, Trace& t, double* out) {
   launch_pdl(&softmax_rows_kernel, dim3((unsigned)r), dim3(256), 0, C.st, C.X,
              C.windows ? t.Lc : nullptr, t.nt, t.T, t.tpos, C.c.sink, C.c.recent, C.PK, t.Pref,
              t.logPref, C.DP, C.rowv);
-  // e_j = ((pk - p) V) W_j^T
+  // DV_j = (pk - p) V
   gm(t.nt, D, t.T, C.DP, t.T, false, t.V, D, false, C.DV, D, 1.0, g, nTT, 0, nD);
   output_error(C, t, C.c.lam, 1);
   loss_mean(C, (int)r, out);
@@ -1661,7 +1639,6 @@ extern "C" optr_status optr_calibrate_head(
   } else {
     C.tr[1] = C.tr[0];
   }
-  output_setup(C);
   adam_run(C, 0, C.R0[0], hist_k);
   copy_kernel<<<nblk(n), 256, 0, stream>>>(C.best, n, R_K);
   copy_kernel<<<nblk(n), 256, 0, stream>>>(C.best, n, C.R);
@@ -1693,7 +1670,6 @@ extern "C" optr_status optr_calib_loss_grad(
   C.tr[0].q = q; C.tr[0].K = K; C.tr[0].V = V; C.tr[0].tpos = t_pos;
   C.tr[0].T = c->T; C.tr[0].nt = c->nt;
   trace_setup(C, C.tr[0], mu);
-  C.M = nullptr;
   if (which == 1) {
     copy_kernel<<<nblk(n), 256, 0, stream>>>(R_K, n, C.R);
     value_setup(C, C.tr[0]);

@@ -150,3 +150,25 @@ def test_gradient_elements_keep_their_own_precision(lo):
         for j, got in enumerate(row):
             a, b = vs[i] * 2 * e * ws[j], vs[j] * 2 * e * ws[i]
             assert abs(Fraction(got) - (a - b)) <= (4 * D + 16) * U * (abs(a) + abs(b))
+
+
+@pytest.mark.parametrize("size", [1e3, 1e6])
+def test_output_error_in_the_weak_directions_of_W(size):
+    """hist_v[0] of a calibration whose value lies where a badly conditioned W_O is
+    weak: the rows are size s_m (1, 1, 0, ..) + b_m and V = (x, -x, 0, ..), so that
+    W V = x (W_m0 - W_m1), a difference that float64 forms exactly while the squares
+    of W round at size^2."""
+    nt, dm = 64, 1024
+    gen = torch.Generator().manual_seed(21)
+    W = torch.rand(1, dm, D, generator=gen, dtype=F64)
+    W[..., :2] += size * torch.randn(1, dm, 1, generator=gen, dtype=F64)
+    v = torch.zeros(D, dtype=F64)
+    v[0], v[1] = 2.0 ** -36, -2.0 ** -36
+    zeros, I = torch.zeros(1, D, dtype=F64), torch.eye(D, dtype=F64)
+    cfg = optr.calib_config(1, dm, 1, nt, steps=1, select_every=1)
+    *_, hist_v = optr.optr_calibrate_head(
+        cfg, *[x.cuda() for x in (torch.zeros(nt, 1, D, dtype=F64), zeros, v.view(1, D),
+                                  torch.zeros(nt, dtype=torch.int32), W)], R0_K=I.cuda(), R0_V=I.cuda())
+    ref = _exact(v, W)
+    # a term has the roundings of its two products, the square and the sums theirs
+    assert abs(Fraction(hist_v[0].item()) - ref) <= (dm / 32 + nt / 256 + 32) * U * ref
