@@ -537,9 +537,12 @@ __global__ void __launch_bounds__(256 * H) mat_product_kernel(MatOp o) {
   pdl_trigger();
   int s = 0;
   if (o.norm != nullptr) {
-    // non-negative doubles compare as their bits; a NaN is the largest
+    // Non-negative doubles compare as their bits, here plus 1.  A NaN is 0, the
+    // smallest: a generator with NaN in some rows gives NaN results, one with NaN
+    // in all of them is out of range.
     if (threadIdx.x < kCD) {
       unsigned long long b = __double_as_longlong(__ldcg(o.norm + threadIdx.x));
+      b = b > 0x7ff0000000000000ull ? 0 : b + 1;
 #pragma unroll
       for (int i = 16; i > 0; i >>= 1) {
         const unsigned long long u = __shfl_xor_sync(0xffffffffu, b, i);
@@ -551,7 +554,7 @@ __global__ void __launch_bounds__(256 * H) mat_product_kernel(MatOp o) {
     unsigned long long b = s_norm[0];
 #pragma unroll
     for (int i = 1; i < 4; ++i) b = s_norm[i] > b ? s_norm[i] : b;
-    double nrm = __longlong_as_double(b);
+    double nrm = __longlong_as_double(b - 1);  // (0: all bits set, a NaN)
     while (nrm > 0.5 && s < o.s_max) {
       nrm *= 0.5;
       ++s;

@@ -172,3 +172,24 @@ def test_output_error_in_the_weak_directions_of_W(size):
     ref = _exact(v, W)
     # a term has the roundings of its two products, the square and the sums theirs
     assert abs(Fraction(hist_v[0].item()) - ref) <= (dm / 32 + nt / 256 + 32) * U * ref
+
+
+@pytest.mark.parametrize("rows", [1, D])
+def test_generator_with_nan(rows):
+    """NaN in some rows of A - A^T gives a NaN loss; a generator without a finite
+    row is out of the exponential's range."""
+    A = torch.zeros(D, D, dtype=F64)
+    A[:rows, 7] = float("nan")
+    if rows == D:
+        A[:] = float("nan")
+    I, zeros = torch.eye(D, dtype=F64), torch.zeros(2, D, dtype=F64)
+    args = [x.cuda() for x in (torch.ones(1, 1, D, dtype=F64), zeros, zeros + 0.5,
+                               torch.ones(1, dtype=torch.int32), torch.ones(1, 3, D, dtype=F64),
+                               zeros[0], I, A)]
+    call = lambda: optr.optr_calib_loss_grad(optr.calib_config(1, 3, 2, 1), 1, *args, R_K=I.cuda())
+    if rows == D:
+        with pytest.raises(optr.OptrError):
+            call()
+    else:
+        loss, _ = call()
+        assert loss.isnan().all()
