@@ -14,7 +14,7 @@ namespace optr {
 // tokens; the slices are added in shared memory, then warp t quantizes and
 // packs token t group by group.  T = 4 for at most 64 new tokens (4x the
 // CTAs, a quarter of the FMAs per thread: the decode step's latency), else
-// 16; a decode step's prologue always takes 4 (its CTAs share SMs in pairs).
+// 16 (a decode step's prologue: see prologue_tile in decode.cu).
 constexpr int kSmallTok = 16;
 constexpr int kSmallTokFew = 4;
 constexpr int kSmallCuCache = 512;   // sequences whose cu_new / pos0 a CTA caches

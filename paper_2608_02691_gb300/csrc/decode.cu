@@ -105,17 +105,19 @@ qrot_kernel(int nb, const __nv_bfloat16* __restrict__ q, const float* __restrict
 // CTAs, as qrot_kernel).  All wait for the previous kernel before touching
 // inputs; the partial kernel then waits for this grid, i.e. for all.
 // Bound by latency: each CTA loads 64 KB of a rotation and goes through a few
-// barriers.  So two CTAs share an SM (64 registers, tiles of 4 new tokens; one
-// of 70 or, with tiles of 16, 102 registers took two waves for 16 sequences x 8
-// heads and eight for 128 x 8), and a query-rotation CTA takes its head's
+// barriers.  With tiles of T = 4 new tokens two CTAs share an SM (64 registers;
+// one of 70 or, with tiles of 16, 128 registers takes two waves for 16 sequences
+// x 8 heads and eight for 128 x 8), and a query-rotation CTA takes its head's
 // rotation through `nb` sequences, so that these CTAs are at most one such wave.
 // Decode step of 16 x 8192 tokens 45.4 -> 44.0 us; of 128 x 1024 to 32768, with
 // the combine's two CTAs per SM, 530.4 -> 518.3; of 37 short ones, 4 heads, 28.2
-// -> 26.8.
+// -> 26.8.  Where the cache write is the longer part (prologue_tile) tiles of 16
+// load a rotation a quarter as often.
 static_assert(kQrotThreads == 512, "one block size for every body");
 static_assert(sizeof(float) * kPage * 4 >= (size_t)kWinPBytes, "window P scratch");
 
-__global__ void __launch_bounds__(512, 2)
+template <int T>
+__global__ void __launch_bounds__(512, T == kSmallTokFew ? 2 : 1)
 step_prologue_kernel(
     int n_app, int app_tiles, const __nv_bfloat16* __restrict__ k,
     const __nv_bfloat16* __restrict__ v, int n_tok,
@@ -145,10 +147,9 @@ step_prologue_kernel(
   if (bid < n_app) {
     const int tblk = bid % app_tiles, hk = (bid / app_tiles) % h_kv,
               kind = bid / (app_tiles * h_kv);
-    append_small_body<kSmallTokFew>(
-                      tblk, hk, kind, *reinterpret_cast<AppendSmallSmemT<kSmallTokFew>*>(dsm_), k, v, n_tok, cu_new, pos0, bt, B, max_pages, pool,
-                      num_pages, h_kv, R_k, R_v, muR, clip_k, clip_v, err,
-                      fold_v && kind == 1, group128 != 0);
+    append_small_body<T>(tblk, hk, kind, *reinterpret_cast<AppendSmallSmemT<T>*>(dsm_), k, v,
+                         n_tok, cu_new, pos0, bt, B, max_pages, pool, num_pages, h_kv, R_k, R_v,
+                         muR, clip_k, clip_v, err, fold_v && kind == 1, group128 != 0);
   } else if (bid < n_app + n_wcp) {
     window_copy_body(bid - n_app, *reinterpret_cast<WinCopySmem*>(dsm_), k, v,
                      n_tok, cu_new, pos0, B, win, win_slot, n_slots, h_kv,
@@ -159,6 +160,18 @@ step_prologue_kernel(
               h_q, h_kv, qscale, seq_lens, max_pages, qf, qs, frag, koff, invs,
               pref, nzpref, cnt_ws, err, sink, recent);
   }
+}
+
+// Tokens per cache-write CTA of the prologue.  Many new tokens for few segments
+// (several tokens each: drafts, a chunk of a prompt) make the cache write the
+// longer part: 16 x 8192 with 5, 8, 16 tokens each 47.7, 50.9, 57.2 us with tiles
+// of 4, 46.3, 49.5, 55.5 with 16; 8 x 2048 with windows, 32 tokens 35.7 / 32.0.
+// With more segments than SMs the query rotations and the number of CTAs count:
+// 66 and 128 sequences x 8 heads, one token each, 60.0 / 64.1 and 76.4 / 77.9; 38
+// with 2 and 4 tokens 60.1 / 59.8 and 64.3 / 64.8.
+static int prologue_tile(const optr_params* p, int n_tok, int B) {
+  return small_tile(n_tok) == kSmallTok && (long long)B * p->cfg.h_kv <= p->num_sms ? kSmallTok
+                                                                                 : kSmallTokFew;
 }
 
 // Window part of a separate cache write (512 threads per 16 new tokens).
@@ -841,13 +854,16 @@ cudaError_t launch_decode(const optr_params* p, int variant,
     // the cache write of the step (INT2 records and window copies) and the
     // query rotation in one launch (the one-launch decode rotates its own)
     prof_mark(p, 0, s);
-    const int tiles = (app->n_tok + kSmallTokFew - 1) / kSmallTokFew;
+    const int T = prologue_tile(p, app->n_tok, B);
+    const int tiles = (app->n_tok + T - 1) / T;
     const int n_app = tiles * h_kv * 2;
     const int n_wcp = windows ? (app->n_tok + kWinCopyTok - 1) / kWinCopyTok : 0;
-    const size_t sm_app = sizeof(AppendSmallSmemT<kSmallTokFew>);
+    const size_t sm_app = T == kSmallTokFew ? sizeof(AppendSmallSmemT<kSmallTokFew>)
+                                            : sizeof(AppendSmallSmemT<kSmallTok>);
     size_t sm_bytes = sm_app > sizeof(QrotSmem) ? sm_app : sizeof(QrotSmem);
     if (sm_bytes < sizeof(WinCopySmem)) sm_bytes = sizeof(WinCopySmem);
-    auto fn = step_prologue_kernel;
+    auto fn = T == kSmallTokFew ? step_prologue_kernel<kSmallTokFew>
+                                : step_prologue_kernel<kSmallTok>;
     e = ensure_dynamic_smem(reinterpret_cast<const void*>(fn), sm_bytes);
     if (e != cudaSuccess) return e;
     const int n_rot = cs ? 0 : (B + nb - 1) / nb * h_kv;
