@@ -347,6 +347,7 @@ partial_body(const uint8_t* __restrict__ pool,
   OneSmem& O = *reinterpret_cast<OneSmem*>(smem + kWarps);
   const int cs = ONE ? (int)cluster_size() : 1, rank = ONE ? (int)cluster_rank() : 0;
   const int oseg = ONE ? (int)blockIdx.x / cs : 0, ob = oseg / h_kv, oh = oseg - ob * h_kv;
+  int units = 0;  // window units that the sequence has
   float rv[ONE ? 32 : 1];
   if constexpr (ONE) {
     load_rotation_slice(one.R_k, oh, rv);
@@ -362,7 +363,7 @@ partial_body(const uint8_t* __restrict__ pool,
     F = bad ? 0 : int2_pages(len, sink, recent);
     if constexpr (WIN) {
       // lane i: how long a CTA with i window warps takes; the fewest pages
-      const int units = ((bad ? 0 : win_count(len, sink, recent)) + kWinUnit - 1) / kWinUnit;
+      units = ((bad ? 0 : win_count(len, sink, recent)) + kWinUnit - 1) / kWinUnit;
       const int np = (F + cs - 1) / cs, nu = (units + cs - 1) / cs;
       int cost = 1 << 24;
       if (lane <= kWarps && (nu == 0 || lane > 0) && (np == 0 || lane < kWarps))
@@ -487,9 +488,9 @@ partial_body(const uint8_t* __restrict__ pool,
         if (lane < 8) mine[kPartM + lane] = lane < 4 ? -INFINITY : 0.f;
         __syncwarp();
         const int ww = rank * (kWarps - kInt) + warp - kInt, n = cs * (kWarps - kInt);
-        window_phase((long long)oseg * wp.Uw + (long long)ww * wp.Uw / n,
-                     (long long)oseg * wp.Uw + (long long)(ww + 1) * wp.Uw / n, wp, mine, -oseg,
-                     &S.stage[0][0], reinterpret_cast<uint8_t*>(&S.qfr[0][0]));
+        const long long u = (long long)oseg * wp.Uw;
+        window_phase(u + (long long)ww * units / n, u + (long long)(ww + 1) * units / n, wp, mine,
+                     -oseg, &S.stage[0][0], reinterpret_cast<uint8_t*>(&S.qfr[0][0]));
       }
     }
   }
