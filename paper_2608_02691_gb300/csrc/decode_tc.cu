@@ -63,6 +63,12 @@ static_assert(offsetof(WarpSmemTC, pt) + sizeof(WarpSmemTC::pt) -
                       offsetof(WarpSmemTC, stage) >= (size_t)kWinStageBytes,
               "window row scratch");
 static_assert(sizeof(WarpSmemTC::qfr) >= (size_t)kWinPBytes, "window P scratch");
+// the one-launch decode's end keeps a warp's partial in its page stages and eight
+// rows of R_v^T in qfr and kq, one array then
+static_assert(sizeof(WarpSmemTC::stage) >= sizeof(float) * kPartFloats, "partial scratch");
+static_assert(offsetof(WarpSmemTC, kq) == offsetof(WarpSmemTC, qfr) + sizeof(WarpSmemTC::qfr) &&
+                  sizeof(WarpSmemTC::qfr) + sizeof(WarpSmemTC::kq) >= 8 * kD * sizeof(float),
+              "R_v^T scratch");
 
 // one-launch decode: pages that take as long as a unit of 16 window tokens
 constexpr int kUnitPages = 4;
@@ -896,7 +902,7 @@ partial_body(const uint8_t* __restrict__ pool,
       mine[kPartM + lane] = lane < 4 ? -INFINITY : 0.f;  // (nothing: m, l)
     }
     // R_v^T columns [rank sw, (rank + 1) sw), eight rows per warp, into the
-    // warp's query fragments (free now)
+    // warp's query fragments and start values (free now)
     const int sw = kD / cs;
     float* rows = reinterpret_cast<float*>(&S.qfr[0][0]);
     __syncwarp();
