@@ -896,6 +896,7 @@ partial_body(const uint8_t* __restrict__ pool,
     flush();
   } else {
     float* mine = reinterpret_cast<float*>(&S.stage[0][0]);  // partial of this warp
+    __syncwarp();  // every lane has read the last pages: the partial goes over them
     if (f0 < f1) {
       flush();
     } else if (int_warp && lane < 8) {
