@@ -517,6 +517,10 @@ optr_status optr_decode_step_win(const optr_params* p, const void* q,
   // anything else runs as the two calls
   if (n_tok == 0 || n_tok > 256 || p->cfg.decode_variant == OPTR_VARIANT_CUDA_CORE ||
       p->cfg.append_variant == OPTR_VARIANT_CUDA_CORE) {
+    // (what the decode refuses is refused before the cache is written)
+    const void* dev = nullptr;
+    if (!io_pointer(q, &dev, nullptr) || !io_pointer(out, &dev, nullptr))
+      return OPTR_ERR_INVALID_ARG;
     optr_status st = optr_kv_append_win(p, k, v, n_tok, cu_new, pos0,
                                         block_table, B, max_pages, pool,
                                         num_pages, win, win_slot, n_slots,
