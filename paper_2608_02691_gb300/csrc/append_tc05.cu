@@ -663,10 +663,12 @@ cudaError_t launch_append_tc05(const optr_params* p, const __nv_bfloat16* k,
   // that the (head, kind) pairs leave over take them while the others convert
   // (8 KV heads leave 8 of 152).  A copy of its own after this launch read every
   // token to find the window's: 2000 tokens of one sequence (8 KV heads, 320 window
-  // rows) 18.0 us a call, now 8.2.
+  // rows) 18.0 us a call, now 8.2.  At most 16 of them per SM, which then take more
+  // rows: the grid's z extent is limited.
   const long long rows = win ? (long long)B * (p->cfg.sink + p->cfg.recent) : 0;
   constexpr int kRowsPerCta = kThreads / 32 * 2;
-  const int copies = (int)((rows + kRowsPerCta - 1) / kRowsPerCta);
+  const int copies =
+      (int)min((rows + kRowsPerCta - 1) / kRowsPerCta, (long long)16 * p->num_sms);
   dim3 grid(per, h_kv, 2 + (copies + per * h_kv - 1) / (per * h_kv));
   return launch_pdl(fn, grid, dim3(kThreads), sizeof(Smem), s,
                     mk, mv, k, v, n_tok, cu_new, pos0, bt, B, max_pages, pool, num_pages,
