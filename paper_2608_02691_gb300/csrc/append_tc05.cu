@@ -33,7 +33,7 @@
 // columns, at 128 g) and the A operands (64 columns each, at 256 + 64 b).
 //
 // What bounds it: issue slots (66% used, the rest fixed-latency and memory
-// stalls), with DRAM 60% and the tensor pipe 50% busy.  The epilogue warps used
+// stalls), with DRAM 58% and the tensor pipe 49% busy.  The epilogue warps used
 // to convert their own next tile: 18 warps of 96 registers, each stalled most of
 // the time, and a tile's conversion and quantization one after the other.  As
 // warps of their own, with the record places found once per row instead of twice,

@@ -84,7 +84,7 @@ struct Gemm {
 // 1e-14 / 3e-16; exponents spread over 80 bits 1.4e-15 / 9e-9 / 3e-16; an outlier
 // channel of 1e8 2.7e-15 / 6e-15 / 6e-16, times an identity 0 / 4e-6 / 0.  (Seven
 // digits, 54 bits, need that line at 1/8 for the errors of an FMA chain: 6% of the
-// probabilities x values of a calibration, 20 steps 33.7 ms.)
+// probabilities x values of a calibration, 20 + 20 steps 33.7 ms instead of 26.2.)
 // What bounds it: per CTA and chunk 352 mma a warp (5.7 us at one m16n8k16 per 8
 // cycles and SM quarter), the split of both tiles (24 values a thread, ~50
 // integer instructions each, 2.5 us) and the load's latency, one after the

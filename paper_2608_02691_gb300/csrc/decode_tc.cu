@@ -1084,7 +1084,10 @@ cudaError_t decode_one_limits(const optr_params* p, int (&clusters)[4]) {
 // long sequence has fewer pages than the table's width suggests), stay below
 // that.  Measured, us per call with uniform lengths, split-K / one launch:
 // decode 1 x 1024 15.1 / 11.4, 8 x 2048 20.8 / 14.9, 16 x 2048 23.5 / 19.1,
-// 1 x 16384 20.5 / 19.4 (x = 8, u = 0.4), 1 x 32768 24.2 / 27.2.
+// 1 x 16384 20.5 / 19.4 (x = 8, u = 0.4), 1 x 32768 24.2 / 27.2.  The largest
+// tables taken, 8 heads: 1 x 12319 19.2 / 16.8, 2 x 18623 23.4 / 23.2, 9 x 5327 27.0 /
+// 19.9, with windows 1 x 11039 21.5 / 21.7, 16 x 1039 27.5 / 21.4; 4 heads, windows,
+// 19 x 4479 25.6 / 26.5, where lengths differ 31 to 39 / 25.7 to 25.9.
 int decode_one_cluster(const optr_params* p, int B, int max_pages) {
   const long long segs = (long long)B * p->cfg.h_kv;
   int i = 3;

@@ -194,7 +194,7 @@ constexpr int kWinPBytes = kWinUnit * 8 * 2;             // P [16 tok][8] bf16
 
 // Window partials of units [u0, u1).  The units (b, h, j) = 16 window tokens
 // [16j, 16j + 16) of sequence b, KV head h, indexed u = (b * h_kv + h) * Uw + j,
-// are cut into contiguous ranges, one per window warp (window_units(ww) of Ww);
+// are cut into contiguous ranges, one per window warp (window_warp below);
 // a warp merges the units of one (b, h) in its range by an online softmax and
 // writes one partial (o[4][128], m[4], l[4]; log2 domain, values in the
 // unrotated basis) to slot base + b * h_kv + h of out.  Units past a sequence's

@@ -1,8 +1,9 @@
-"""The calibration's float64 products (split into fp16 digits, 32 x 32 tiles,
-64-deep chunks) where they can go wrong: rows, columns and depths that are no
-multiple of a tile or a chunk, one row or one token, more output channels than
-one chunk, split depths, operands of very different magnitude, and non-finite
-input.  Loss and generator gradient against the float64 oracle; both sides
+"""The calibration's float64 products (split into fp16 digits, 128-deep chunks;
+at these sizes nearly all in 32 x 16 tiles, test_gpu_calib_tiles.py has the 64 x 32
+ones) where they can go wrong: rows, columns and depths that are no multiple of a
+tile or a chunk, one row or one token, more output channels than one chunk, split
+depths, operands whose magnitudes differ as wholes (test_gpu_calib_exact.py has the
+ones that differ inside a row), and non-finite input.  Loss and generator gradient against the float64 oracle; both sides
 round differently at a few 1e-16 per product, and 1e-9 of the largest
 magnitude is allowed (tests/test_gpu_calibration.py states why).
 """
